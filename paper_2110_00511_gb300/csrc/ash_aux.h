@@ -28,8 +28,11 @@ void launch_prefetch_l2(const void* base, int64_t bytes, const Launch& L);
 // Publishes the control block to a host-visible snapshot (publish_snapshot).
 void launch_snapshot(Ctrl* ctrl, Snap* snap, uint32_t seq, const Launch& L);
 void launch_iota(int32_t* h, int64_t from, int64_t to, const Launch& L);
-void launch_scatter_rows(const ValueCopy& vc, const int32_t* idx, const uint8_t* mask, int64_t n, const Launch& L);
-void launch_gather_rows(const ValueCopy& vc, const int32_t* list, int64_t n, const Launch& L);
+// Value rows of an insert's winners (idx[p] >= 0): dst_j row idx[p] <- src_j row p.
+void launch_scatter_rows(const ValueCopy& vc, const int32_t* idx, int64_t n, const Launch& L);
+// dst_j row r <- src_j row list[r] for every value buffer (compacting rehash;
+// the list's indices lie below the source buffers' capacity).
+void launch_gather_rows(const ValueCopy& vc, int64_t capacity, const int32_t* list, int64_t n, const Launch& L);
 void launch_gather_keys(const int32_t* kb, int ks, int d, int64_t capacity, const int32_t* indices, int64_t n,
                         const long long* n_dev, int32_t* out, const Launch& L);
 void launch_gather_values(const void* src, int64_t row_bytes, int vec, int64_t capacity, const int32_t* indices,

@@ -374,24 +374,4 @@ __device__ __forceinline__ int block_count(bool flag, int* s_cnt) {
   return *s_cnt;
 }
 
-// ---------------------------------------------------------------- value rows
-template <typename T>
-__device__ __forceinline__ void copy_elems(void* dst, const void* src, int64_t n_elems, int64_t start, int64_t step) {
-  T* d = static_cast<T*>(dst);
-  const T* s = static_cast<const T*>(src);
-  for (int64_t e = start; e < n_elems; e += step) d[e] = s[e];
-}
-
-// Copies one row of `bytes` bytes with vector width `vec`, elements
-// start, start+step, ... (step = 1 for one thread, 32 for a warp).
-__device__ __forceinline__ void copy_row(void* dst, const void* src, int64_t bytes, int vec, int64_t start, int64_t step) {
-  switch (vec) {
-    case 16: copy_elems<uint4>(dst, src, bytes / 16, start, step); break;
-    case 8: copy_elems<uint2>(dst, src, bytes / 8, start, step); break;
-    case 4: copy_elems<uint32_t>(dst, src, bytes / 4, start, step); break;
-    case 2: copy_elems<uint16_t>(dst, src, bytes / 2, start, step); break;
-    default: copy_elems<uint8_t>(dst, src, bytes, start, step); break;
-  }
-}
-
 }  // namespace ash

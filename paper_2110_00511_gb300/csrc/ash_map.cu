@@ -631,7 +631,7 @@ ash_status rebuild_to(ash_map* m, int64_t new_capacity, int64_t size, cudaStream
         vc.row_bytes[j] = m->row_bytes[j];
         vc.vec[j] = vec_width(m->row_bytes[j], vb[j], m->vb[j]);
       }
-      ash::launch_gather_rows(vc, list, size, L);
+      ash::launch_gather_rows(vc, m->capacity, list, size, L);
     }
   }
   // 2) re-insert the live keys into the new table (preferred slots first)
@@ -875,7 +875,7 @@ ash_status insert_impl(ash_map* m, const int32_t* keys, const void* const* value
     m->K.commit(ckpt, tv, ckeys, n, cidx, cmask, inline_value ? &vr : nullptr, L);
   }
   if (log_p > 0) partition_finish(m, pb, n, idx, mask, st);
-  if (vc.n > 0) ash::launch_scatter_rows(vc, idx, mask, n, L);
+  if (vc.n > 0) ash::launch_scatter_rows(vc, idx, n, L);
   if (!pref) m->pref_placed = false;  // the bucket-first claim places keys in slot order
   m->win_bits_clean = true;  // the commits clear every winner-flag word they read
   m->size_ub += n;
