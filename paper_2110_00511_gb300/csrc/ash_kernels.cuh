@@ -70,133 +70,233 @@ __device__ __forceinline__ int32_t find_key(const TableView& t, const int32_t (&
   return -1;
 }
 
-// Scalar lookup of input row pos (the slow path of find).
-template <int D, int S, class In>
-__device__ __noinline__ int32_t find_one(const TableView t, const In keys, int64_t pos) {
-  int32_t k[D];
-  load_input_key<D>(keys, pos, k);
-  return find_key<D, S>(t, k);
+// The same out of line, for find_keys when a fingerprint match is not the key.
+template <int D>
+struct KeyOf {
+  int32_t v[D];
+};
+
+template <int D, int S>
+__device__ __noinline__ int32_t find_slow(const TableView t, const KeyOf<D> k) {
+  return find_key<D, S>(t, k.v);
 }
 
-// Radius neighbour query (the radius search of Sec. 6.2): thread per (query,
-// offset) pair.  Offsets enumerate [-radius, radius]^D row-major (the last
-// coordinate fastest) and are added with int32 wrap-around; the (2r+1)^D
-// query keys are never materialised.  Outputs are [n, (2r+1)^D].
-template <int D, int S>
-__global__ void __launch_bounds__(256) neighbors_kernel(TableView t, const int32_t* __restrict__ keys, int64_t n,
-                                                        int radius, int64_t n_off, int32_t* __restrict__ idx,
-                                                        uint8_t* __restrict__ mask) {
-  const int64_t total = n * n_off;
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  const int width = 2 * radius + 1;
-  for (int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < total; e += stride) {
-    const int64_t r = e / n_off;
-    int64_t o = e - r * n_off;
-    int32_t k[D];
-    load_input_key<D>(keys, r, k);
+// One probe round of KPT keys: the buckets b[q] of the keys still searched
+// (go[q]) are loaded together, then the verify loads of their first
+// fingerprint matches, then everything is compared.  Settled keys leave go;
+// a match that is another key, or one of several, raises rare.
+template <int D, int S, int KPT, bool ALL>
+__device__ __forceinline__ void probe_round(const TableView& t, const int32_t (&k)[KPT][D], const uint32_t (&fp)[KPT],
+                                            const uint32_t (&b)[KPT], bool (&go)[KPT], int32_t (&out)[KPT],
+                                            bool& rare) {
+  constexpr int KS = KeyStride<D>::value;
+  uint64_t w[KPT][S];
 #pragma unroll
-    for (int j = D - 1; j >= 0; --j) {
-      const int digit = static_cast<int>(o % width);
-      o /= width;
-      k[j] = static_cast<int32_t>(static_cast<uint32_t>(k[j]) + static_cast<uint32_t>(digit - radius));
+  for (int q = 0; q < KPT; ++q)
+    if (ALL || go[q]) load_bucket<S, true>(t.slots + static_cast<size_t>(b[q]) * S, w[q]);
+  uint32_t cand[KPT];
+  int ncand[KPT];
+  bool stop[KPT];
+#pragma unroll
+  for (int q = 0; q < KPT; ++q) {
+    cand[q] = kNoIndex;
+    ncand[q] = 0;
+    stop[q] = false;
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      stop[q] |= (w[q][s] == kEmpty);
+      const bool m = hi32(w[q][s]) == fp[q] && lo32(w[q][s]) < kClaimBit;
+      if (m && ncand[q] == 0) cand[q] = lo32(w[q][s]);
+      ncand[q] += m ? 1 : 0;
     }
-    const int32_t out = find_key<D, S>(t, k);
-    idx[e] = out;
-    mask[e] = out >= 0 ? 1 : 0;
+    if (!ALL && !go[q]) ncand[q] = 0;
+  }
+  int32_t row[KPT][KS];
+#pragma unroll
+  for (int q = 0; q < KPT; ++q) {
+    if (ncand[q] > 0) {
+      load_kb<D>(t.kb, cand[q], row[q]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < KS; ++j) row[q][j] = 0;
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < KPT; ++q) {
+    bool eq = ncand[q] > 0;
+#pragma unroll
+    for (int j = 0; j < D; ++j) eq &= (row[q][j] == k[q][j]);
+    if (eq) out[q] = static_cast<int32_t>(cand[q]);
+    rare |= go[q] && ncand[q] > 0 && !eq;
+    go[q] &= !eq && !stop[q];
   }
 }
 
-// Neighbour query over an explicit offset table (the neighbour tables of
-// Sec. 6.2-6.4: 1-radius 3^D, 1-cube 2^D, 1-ring): thread per (query, offset)
-// pair; offsets is [n_off, D] int32 in device memory, added with int32
-// wrap-around.  Outputs are [n, n_off].
-template <int D, int S>
-__global__ void __launch_bounds__(256) offsets_kernel(TableView t, const int32_t* __restrict__ keys, int64_t n,
-                                                      const int32_t* __restrict__ offsets, int64_t n_off,
-                                                      int32_t* __restrict__ idx, uint8_t* __restrict__ mask) {
-  const int64_t total = n * n_off;
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < total; e += stride) {
-    const int64_t r = e / n_off;
-    const int64_t o = e - r * n_off;
-    int32_t k[D];
-    load_input_key<D>(keys, r, k);
+// Looks KPT keys up together (ok[q] false: a key that nobody asked for; its
+// bucket is loaded, in bounds, and its result unused).  At the usual load of
+// one half, about one home bucket in six is full without the key, so nearly
+// every warp has lanes that probe on: they go on from the next bucket, with
+// hash and key in registers.  Searching such a key again from its home
+// bucket in an out-of-line loop instead made the 27-neighbourhood kernel
+// issue 495 instructions per warp and query at 12 active lanes of 32 (now
+// 270 at 19).  GB300: 6M finds, half absent, on 5M entries 161 -> 127 us; 4M
+// finds, all present, 72 -> 61 us.
+template <int D, int S, int KPT>
+__device__ __forceinline__ void find_keys(const TableView& t, const int32_t (&k)[KPT][D], const bool (&ok)[KPT],
+                                          int32_t (&out)[KPT]) {
+  uint32_t fp[KPT], b[KPT];
+  bool go[KPT];
+  bool rare = false;
+#pragma unroll
+  for (int q = 0; q < KPT; ++q) {
+    const uint64_t h = hash_key<D>(k[q]);
+    fp[q] = fingerprint(h);
+    b[q] = home_bucket(h, t.n_buckets);
+    go[q] = ok[q];
+    out[q] = -1;
+  }
+  probe_round<D, S, KPT, true>(t, k, fp, b, go, out, rare);
+  for (uint32_t probe = 1; probe < t.max_probes; ++probe) {
+    bool any = false;
+#pragma unroll
+    for (int q = 0; q < KPT; ++q) any |= go[q];
+    if (!any) break;
+#pragma unroll
+    for (int q = 0; q < KPT; ++q) b[q] = next_bucket(b[q], t.n_buckets);
+    probe_round<D, S, KPT, false>(t, k, fp, b, go, out, rare);
+  }
+  if (rare) {
+#pragma unroll
+    for (int q = 0; q < KPT; ++q) {
+      if (ok[q] && out[q] < 0) {
+        KeyOf<D> key;
+#pragma unroll
+        for (int j = 0; j < D; ++j) key.v[j] = k[q][j];
+        out[q] = find_slow<D, S>(t, key);
+      }
+    }
+  }
+}
+
+// Offsets of a neighbour query.  RadiusOffsets: [-radius, radius]^D row-major
+// (the last coordinate fastest), digit by digit of the offset's number in
+// base width = 2 radius + 1; the division by width is a multiplication by
+// magic = ceil(2^32 / width), exact for the offset numbers allowed (below
+// 2^20, with width <= 17), and 0 for width 1, whose only number is 0.
+struct RadiusOffsets {
+  uint32_t radius, width, magic;
+  template <int D>
+  __device__ __forceinline__ void add(uint32_t o, int32_t (&k)[D]) const {
+#pragma unroll
+    for (int j = D - 1; j >= 0; --j) {
+      const uint32_t q = __umulhi(o, magic);
+      k[j] = static_cast<int32_t>(static_cast<uint32_t>(k[j]) + (o - q * width) - radius);
+      o = q;
+    }
+  }
+};
+
+// TableOffsets: an explicit [n_off, D] int32 table in device memory.
+struct TableOffsets {
+  const int32_t* __restrict__ table;
+  template <int D>
+  __device__ __forceinline__ void add(uint32_t o, int32_t (&k)[D]) const {
 #pragma unroll
     for (int j = 0; j < D; ++j)
-      k[j] = static_cast<int32_t>(static_cast<uint32_t>(k[j]) + static_cast<uint32_t>(__ldg(offsets + o * D + j)));
-    const int32_t out = find_key<D, S>(t, k);
-    idx[e] = out;
-    mask[e] = out >= 0 ? 1 : 0;
+      k[j] = static_cast<int32_t>(static_cast<uint32_t>(k[j]) + static_cast<uint32_t>(__ldg(table + o * D + j)));
+  }
+};
+
+constexpr int kNeighborUnroll = 1;
+
+// Neighbour query (the radius search and the neighbour tables of Sec.
+// 6.2-6.4): the n x n_off (query, offset) pairs flattened, outputs [n, n_off].
+// Offsets are added with int32 wrap-around; the query keys are never
+// materialised.  Blocks take tiles of U * blockDim consecutive pairs, U per
+// thread, so the key rows of a tile come from L1 and the outputs are
+// coalesced; a thread's (query, offset) moves by two constant strides, so
+// the only divisions are at its start.
+template <int D, int S, int U, class Off>
+__global__ void __launch_bounds__(256) neighbors_kernel(TableView t, const int32_t* __restrict__ keys, int64_t n,
+                                                        const Off off, uint32_t n_off, int32_t* __restrict__ idx,
+                                                        uint8_t* __restrict__ mask) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int64_t total = n * n_off;
+  const int64_t tile = static_cast<int64_t>(blockDim.x) * U;
+  const int64_t jump = (gridDim.x - 1) * tile;
+  const int64_t first = static_cast<int64_t>(blockIdx.x) * tile + threadIdx.x;
+  const uint32_t step_r = blockDim.x / n_off, step_o = blockDim.x - step_r * n_off;
+  const int64_t jump_r = jump / n_off;
+  const uint32_t jump_o = static_cast<uint32_t>(jump - jump_r * n_off);
+  int64_t r = first / n_off;
+  uint32_t o = static_cast<uint32_t>(first - r * n_off);
+  for (int64_t e = first; e < total; e += gridDim.x * tile) {
+    int32_t k[U][D];
+    bool ok[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      ok[u] = e + u * blockDim.x < total;
+      if (ok[u]) {
+        load_input_key<D>(keys, r, k[u]);
+        off.add(o, k[u]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < D; ++j) k[u][j] = 0;
+      }
+      r += step_r;
+      o += step_o;
+      if (o >= n_off) {
+        o -= n_off;
+        ++r;
+      }
+    }
+    int32_t out[U];
+    find_keys<D, S, U>(t, k, ok, out);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (ok[u]) {
+        idx[e + u * blockDim.x] = out[u];
+        mask[e + u * blockDim.x] = out[u] >= 0 ? 1 : 0;
+      }
+    }
+    r += jump_r;
+    o += jump_o;
+    if (o >= n_off) {
+      o -= n_off;
+      ++r;
+    }
   }
 }
 
 // KPT keys per thread: positions base, base + blockDim.x, ... so every load
-// instruction stays coalesced across the warp.  All home buckets are loaded
-// before any is examined, and all verify loads are issued before any compare.
+// instruction stays coalesced across the warp.
 template <int D, int S, int KPT, class In = const int32_t*>
 __global__ void __launch_bounds__(256) find_kernel(TableView t, const In keys, int64_t n,
                                                    int32_t* __restrict__ idx, uint8_t* __restrict__ mask) {
   // a programmatic dependent of the previous kernel: wait for its grid (a no-op otherwise)
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  constexpr int KS = KeyStride<D>::value;
   const int64_t step = static_cast<int64_t>(gridDim.x) * blockDim.x * KPT;
   for (int64_t base = static_cast<int64_t>(blockIdx.x) * blockDim.x * KPT + threadIdx.x; base < n; base += step) {
-    int32_t k[KPT][D];
-    uint32_t fp[KPT], b[KPT];
+    int32_t k[KPT][D], out[KPT];
+    bool ok[KPT];
 #pragma unroll
     for (int q = 0; q < KPT; ++q) {
       const int64_t pos = base + static_cast<int64_t>(q) * blockDim.x;
-      if (pos < n) {
+      ok[q] = pos < n;
+      if (ok[q]) {
         load_input_key<D>(keys, pos, k[q]);
       } else {
 #pragma unroll
         for (int j = 0; j < D; ++j) k[q][j] = 0;
       }
-      const uint64_t h = hash_key<D>(k[q]);
-      fp[q] = fingerprint(h);
-      b[q] = home_bucket(h, t.n_buckets);
     }
-    uint64_t w[KPT][S];
-#pragma unroll
-    for (int q = 0; q < KPT; ++q) load_bucket<S, true>(t.slots + static_cast<size_t>(b[q]) * S, w[q]);
-    uint32_t cand[KPT];
-    int ncand[KPT];
-    bool stop[KPT];
-#pragma unroll
-    for (int q = 0; q < KPT; ++q) {
-      cand[q] = kNoIndex;
-      ncand[q] = 0;
-      stop[q] = false;
-#pragma unroll
-      for (int s = 0; s < S; ++s) {
-        stop[q] |= (w[q][s] == kEmpty);
-        const bool m = hi32(w[q][s]) == fp[q] && lo32(w[q][s]) < kClaimBit;
-        if (m && ncand[q] == 0) cand[q] = lo32(w[q][s]);
-        ncand[q] += m ? 1 : 0;
-      }
-    }
-    int32_t row[KPT][KS];
-#pragma unroll
-    for (int q = 0; q < KPT; ++q) {
-      if (ncand[q] > 0) {
-        load_kb<D>(t.kb, cand[q], row[q]);
-      } else {
-#pragma unroll
-        for (int j = 0; j < KS; ++j) row[q][j] = 0;
-      }
-    }
+    find_keys<D, S, KPT>(t, k, ok, out);
 #pragma unroll
     for (int q = 0; q < KPT; ++q) {
       const int64_t pos = base + static_cast<int64_t>(q) * blockDim.x;
-      if (pos < n) {
-        bool eq = ncand[q] > 0;
-#pragma unroll
-        for (int j = 0; j < D; ++j) eq &= (row[q][j] == k[q][j]);
-        int32_t out = -1;
-        if (eq) out = static_cast<int32_t>(cand[q]);
-        else if (ncand[q] > 0 || !stop[q]) out = find_one<D, S, In>(t, keys, pos);  // rare
-        idx[pos] = out;
-        mask[pos] = out >= 0 ? 1 : 0;
+      if (ok[q]) {
+        idx[pos] = out[q];
+        mask[pos] = out[q] >= 0 ? 1 : 0;
       }
     }
   }
@@ -1410,29 +1510,30 @@ struct DimLaunchers {
     else if (S == 8) rebuild_s<8>(t, kb_src, list, n, n_dev, preserve, copy_keys, L);
     else rebuild_s<16>(t, kb_src, list, n, n_dev, preserve, copy_keys, L);
   }
-  template <int S>
-  static void neighbors_s(const TableView& t, const int32_t* keys, int64_t n, int radius, int64_t n_off, int32_t* idx,
-                          uint8_t* mask, const Launch& L) {
+  template <int S, class Off>
+  static void neighbors_s(const TableView& t, const int32_t* keys, int64_t n, const Off& off, int64_t n_off,
+                          int32_t* idx, uint8_t* mask, const Launch& L) {
     TraceScope ts(kKNeighbors, L.stream);
-    neighbors_kernel<D, S><<<grid_for(n * n_off, L), L.block, 0, L.stream>>>(t, keys, n, radius, n_off, idx, mask);
+    constexpr int U = kNeighborUnroll;
+    launch_dependent(neighbors_kernel<D, S, U, Off>, grid_for((n * n_off + U - 1) / U, L), L.block, L.stream, t, keys,
+                     n, off, static_cast<uint32_t>(n_off), idx, mask);
+  }
+  template <class Off>
+  static void neighbors_off(int S, const TableView& t, const int32_t* keys, int64_t n, const Off& off, int64_t n_off,
+                            int32_t* idx, uint8_t* mask, const Launch& L) {
+    if (S == 4) neighbors_s<4>(t, keys, n, off, n_off, idx, mask, L);
+    else if (S == 8) neighbors_s<8>(t, keys, n, off, n_off, idx, mask, L);
+    else neighbors_s<16>(t, keys, n, off, n_off, idx, mask, L);
   }
   static void neighbors(int S, const TableView& t, const int32_t* keys, int64_t n, int radius, int64_t n_off,
                         int32_t* idx, uint8_t* mask, const Launch& L) {
-    if (S == 4) neighbors_s<4>(t, keys, n, radius, n_off, idx, mask, L);
-    else if (S == 8) neighbors_s<8>(t, keys, n, radius, n_off, idx, mask, L);
-    else neighbors_s<16>(t, keys, n, radius, n_off, idx, mask, L);
-  }
-  template <int S>
-  static void offsets_s(const TableView& t, const int32_t* keys, int64_t n, const int32_t* off, int64_t n_off,
-                        int32_t* idx, uint8_t* mask, const Launch& L) {
-    TraceScope ts(kKNeighbors, L.stream);
-    offsets_kernel<D, S><<<grid_for(n * n_off, L), L.block, 0, L.stream>>>(t, keys, n, off, n_off, idx, mask);
+    const uint32_t width = 2 * static_cast<uint32_t>(radius) + 1;
+    const uint32_t magic = width > 1 ? static_cast<uint32_t>(((uint64_t{1} << 32) + width - 1) / width) : 0u;
+    neighbors_off(S, t, keys, n, RadiusOffsets{static_cast<uint32_t>(radius), width, magic}, n_off, idx, mask, L);
   }
   static void offsets(int S, const TableView& t, const int32_t* keys, int64_t n, const int32_t* off, int64_t n_off,
                       int32_t* idx, uint8_t* mask, const Launch& L) {
-    if (S == 4) offsets_s<4>(t, keys, n, off, n_off, idx, mask, L);
-    else if (S == 8) offsets_s<8>(t, keys, n, off, n_off, idx, mask, L);
-    else offsets_s<16>(t, keys, n, off, n_off, idx, mask, L);
+    neighbors_off(S, t, keys, n, TableOffsets{off}, n_off, idx, mask, L);
   }
   template <int S>
   static void find_group_s(const TableView& t, const int32_t* keys, int64_t n, int32_t* idx, uint8_t* mask,
