@@ -744,7 +744,7 @@ def main(argv=None):
         "find": bytes_find(N, 0),
         "list_active": bytes_list(N, n_unique),
         "gather_keys": bytes_gather_keys(n_unique),
-        "heap_iota": 4 * N,
+        "storage_init": (16 + 4 + 4) * N + N // 8 + 32,  # table, heap, values, winner flags, counters
     }
     kernels = {}
     total_kernel_ms = sum(ms for ms, n in trace.values())

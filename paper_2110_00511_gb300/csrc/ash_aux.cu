@@ -221,39 +221,84 @@ void launch_list_active(bool heap_identity, const int32_t* heap, int64_t capacit
   compact_live_kernel<<<n_blocks, kListThreads, 0, L.stream>>>(bitmap, capacity, ctrl, out, out_cap, count_out);
 }
 
-// ------------------------------------------------------------------- heap
-// h[i] = i for i in [from, to): scalar head and tail, int4 stores between.
-__global__ void iota_kernel(int32_t* __restrict__ h, int64_t from, int64_t to) {
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  const int64_t tid = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int64_t a = min(to, (from + 3) & ~int64_t{3});  // first multiple of 4
-  const int64_t b = max(a, to & ~int64_t{3});
-  for (int64_t i = from + tid; i < a; i += stride) h[i] = static_cast<int32_t>(i);
-  for (int64_t q = a / 4 + tid; q < b / 4; q += stride) {
-    const int32_t v = static_cast<int32_t>(4 * q);
-    reinterpret_cast<int4*>(h)[q] = make_int4(v, v + 1, v + 2, v + 3);
+// ------------------------------------------------------- storage in one launch
+// A block takes 16 KiB chunks of the plan's ranges: 16-byte stores, four per
+// thread (copies: four loads, then four stores); the bytes before the first
+// 16-byte boundary and after the last belong to a range's first chunk.  One
+// launch instead of a memset or copy per buffer, a kernel for the heap and
+// one for the counters: on small maps the launches are the cost, on large
+// ones HBM writes bound both alike (2 GB cleared in 304 us, 0.97 of the copy
+// peak).  GB300: a map created for 4M points, filled and read 292 -> 277 us;
+// 1.2M keys inserted from a capacity of 16k, growing five times, 544 -> 408
+// us (with the listing that a growth under the identity heap no longer
+// needs).
+__device__ __forceinline__ char init_byte(const InitSeg& g, int64_t off) {
+  switch (g.kind) {
+    case InitPlan::kOnes: return static_cast<char>(0xFF);
+    case InitPlan::kCopy: return g.src[off];
+    case InitPlan::kIota: return static_cast<char>((g.word + static_cast<uint64_t>(off >> 2)) >> (8 * (off & 3)));
+    case InitPlan::kWord: return static_cast<char>(g.word >> (8 * off));
+    default: return 0;
   }
-  for (int64_t i = b + tid; i < to; i += stride) h[i] = static_cast<int32_t>(i);
 }
 
-void launch_iota(int32_t* h, int64_t from, int64_t to, const Launch& L) {
-  if (to <= from) return;
-  TraceScope ts(kKIota, L.stream);
-  iota_kernel<<<grid_for((to - from + 3) / 4, L), L.block, 0, L.stream>>>(h, from, to);
+__global__ void __launch_bounds__(256) init_kernel(const __grid_constant__ InitPlan plan, int64_t chunks) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  constexpr int kUnits = static_cast<int>(InitPlan::kChunk / 16);
+  for (int64_t c = blockIdx.x; c < chunks; c += gridDim.x) {
+    int j = 0;
+    int64_t at = c;
+    while (at >= plan.seg[j].chunks) at -= plan.seg[j++].chunks;
+    const InitSeg& g = plan.seg[j];
+    const int64_t to_align = static_cast<int64_t>(-reinterpret_cast<uintptr_t>(g.dst) & 15);
+    const int64_t head = to_align < g.bytes ? to_align : g.bytes;
+    const int64_t units = (g.bytes - head) / 16;
+    if (at == 0) {
+      const int64_t tail0 = head + units * 16;
+      if (threadIdx.x < head) g.dst[threadIdx.x] = init_byte(g, threadIdx.x);
+      if (threadIdx.x < g.bytes - tail0) g.dst[tail0 + threadIdx.x] = init_byte(g, tail0 + threadIdx.x);
+    }
+    const int64_t u0 = at * kUnits + threadIdx.x;
+    uint4* dst = reinterpret_cast<uint4*>(g.dst + head);
+    if (g.kind == InitPlan::kCopy) {
+      const char* src = g.src + head;
+      if ((reinterpret_cast<uintptr_t>(src) & 15) == 0) {
+        uint4 v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (u0 + q * 256 < units) v[q] = __ldg(reinterpret_cast<const uint4*>(src) + u0 + q * 256);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (u0 + q * 256 < units) dst[u0 + q * 256] = v[q];
+      } else {
+        const int64_t b1 = (at + 1) * kUnits < units ? (at + 1) * InitPlan::kChunk : units * 16;
+        for (int64_t k = at * InitPlan::kChunk + threadIdx.x; k < b1; k += blockDim.x) g.dst[head + k] = src[k];
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int64_t u = u0 + q * 256;
+        if (u >= units) break;
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (g.kind == InitPlan::kOnes) {
+          v = make_uint4(~0u, ~0u, ~0u, ~0u);
+        } else if (g.kind == InitPlan::kIota) {
+          const uint32_t first = static_cast<uint32_t>(g.word) + static_cast<uint32_t>((head + u * 16) >> 2);
+          v = make_uint4(first, first + 1, first + 2, first + 3);
+        }
+        dst[u] = v;
+      }
+    }
+  }
 }
 
-__global__ void set_top_used_kernel(Ctrl* ctrl, unsigned long long top_used) { ctrl->top_used = top_used; }
-
-// used slots := the listed live count (heap top unchanged), after a rebuild
-// whose count only the device knows.
-__global__ void set_used_from_count_kernel(Ctrl* ctrl) {
-  const unsigned long long top = ctrl->top_used & 0xFFFFFFFFull;
-  ctrl->top_used = (ctrl->count << 32) | top;
-}
-
-void launch_set_used_from_count(Ctrl* ctrl, const Launch& L) {
-  TraceScope ts(kKSetCtrl, L.stream);
-  set_used_from_count_kernel<<<1, 1, 0, L.stream>>>(ctrl);
+void launch_init(const InitPlan& plan, const Launch& L) {
+  int64_t chunks = 0;
+  for (int j = 0; j < plan.n; ++j) chunks += plan.seg[j].chunks;
+  if (chunks == 0) return;
+  TraceScope ts(kKInit, L.stream);
+  const int64_t cap = static_cast<int64_t>(L.sms > 0 ? L.sms : 128) * 8;
+  launch_dependent(init_kernel, static_cast<int>(chunks < cap ? chunks : cap), 256, L.stream, plan, chunks);
 }
 
 __global__ void snapshot_kernel(Ctrl* ctrl, Snap* snap, uint32_t seq) {
@@ -263,12 +308,6 @@ __global__ void snapshot_kernel(Ctrl* ctrl, Snap* snap, uint32_t seq) {
 void launch_snapshot(Ctrl* ctrl, Snap* snap, uint32_t seq, const Launch& L) {
   TraceScope ts(kKSetCtrl, L.stream);
   snapshot_kernel<<<1, 32, 0, L.stream>>>(ctrl, snap, seq);
-}
-
-void launch_set_top_used(Ctrl* ctrl, int64_t top, int64_t used, const Launch& L) {
-  const unsigned long long v = (static_cast<unsigned long long>(used) << 32) | static_cast<unsigned long long>(top);
-  TraceScope ts(kKSetCtrl, L.stream);
-  set_top_used_kernel<<<1, 1, 0, L.stream>>>(ctrl, v);
 }
 
 // -------------------------------------------------------------- value rows

@@ -1226,21 +1226,34 @@ __global__ void __launch_bounds__(256) erase_resolve_kernel(TableView t, int64_t
 }
 
 // ------------------------------------------------------------------ rebuild
-// Inserts n unique keys taken from kb_src rows list[j] into an empty table.
-// preserve: the entry keeps buffer index list[j]; otherwise it becomes j.
-// The key row is copied to kb_dst when kb_dst != kb_src or !preserve.
+// Inserts n unique keys taken from kb_src rows list[j] into an empty table
+// (list == nullptr: rows 0..n-1, the live entries while the heap is the
+// identity).  preserve: the entry keeps buffer index list[j]; otherwise it
+// becomes j.  The key row is copied to kb_dst when kb_dst != kb_src or
+// !preserve.  How many entries there are: kCountExact, n; otherwise at most
+// n, the listing's count or the heap top as the device knows them (so that a
+// rebuild can be enqueued without the host knowing), and the used-slot count
+// becomes that number.
+constexpr int kCountExact = 0;
+constexpr int kCountListed = 1;
+constexpr int kCountTop = 2;
+
 template <int D, int S>
-// n_dev (optional): the live count on the device (written by the listing);
-// the kernel then processes min(n, *n_dev) entries, so a rebuild can be
-// enqueued without the host knowing the count.
 __global__ void __launch_bounds__(256) rebuild_kernel(TableView t, const int32_t* __restrict__ kb_src,
-                                                      const int32_t* __restrict__ list, int64_t n,
-                                                      const unsigned long long* __restrict__ n_dev, int preserve,
-                                                      int copy_keys) {
-  if (n_dev) n = min(n, static_cast<int64_t>(*n_dev));
+                                                      const int32_t* __restrict__ list, int64_t n, int count,
+                                                      int preserve, int copy_keys) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (count != kCountExact) {
+    // the low word (the heap top) does not change, so blocks may read it
+    // before or after the first one's store
+    const unsigned long long top = t.ctrl->top_used & 0xFFFFFFFFull;
+    const unsigned long long live = count == kCountListed ? t.ctrl->count : top;
+    n = min(n, static_cast<int64_t>(live));
+    if (blockIdx.x == 0 && threadIdx.x == 0) t.ctrl->top_used = (live << 32) | top;
+  }
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; j < n; j += stride) {
-    const uint32_t a = static_cast<uint32_t>(list[j]);
+    const uint32_t a = static_cast<uint32_t>(list ? list[j] : j);
     int32_t row[KeyStride<D>::value];
     load_kb<D>(kb_src, a, row);
     int32_t k[D];
@@ -1373,8 +1386,7 @@ struct DimKernels {
   void (*commit)(int kpt, const TableView&, const int32_t*, int64_t, int32_t*, uint8_t*, const ValueRow*,
                  const Launch&);
   void (*erase_mark)(int S, const TableView&, const int32_t*, int64_t, int32_t*, const Launch&);
-  void (*rebuild)(int S, const TableView&, const int32_t*, const int32_t*, int64_t, const unsigned long long*, int, int,
-                  const Launch&);
+  void (*rebuild)(int S, const TableView&, const int32_t*, const int32_t*, int64_t, int, int, int, const Launch&);
   void (*neighbors)(int S, const TableView&, const int32_t*, int64_t, int, int64_t, int32_t*, uint8_t*, const Launch&);
   void (*offsets)(int S, const TableView&, const int32_t*, int64_t, const int32_t*, int64_t, int32_t*, uint8_t*,
                   const Launch&);
@@ -1500,15 +1512,16 @@ struct DimLaunchers {
   }
   template <int S>
   static void rebuild_s(const TableView& t, const int32_t* kb_src, const int32_t* list, int64_t n,
-                        const unsigned long long* n_dev, int preserve, int copy_keys, const Launch& L) {
+                        int count, int preserve, int copy_keys, const Launch& L) {
     TraceScope ts(kKRebuild, L.stream);
-    rebuild_kernel<D, S><<<grid_for(n, L), L.block, 0, L.stream>>>(t, kb_src, list, n, n_dev, preserve, copy_keys);
+    launch_dependent(rebuild_kernel<D, S>, grid_for(n, L), L.block, L.stream, t, kb_src, list, n, count, preserve,
+                     copy_keys);
   }
   static void rebuild(int S, const TableView& t, const int32_t* kb_src, const int32_t* list, int64_t n,
-                      const unsigned long long* n_dev, int preserve, int copy_keys, const Launch& L) {
-    if (S == 4) rebuild_s<4>(t, kb_src, list, n, n_dev, preserve, copy_keys, L);
-    else if (S == 8) rebuild_s<8>(t, kb_src, list, n, n_dev, preserve, copy_keys, L);
-    else rebuild_s<16>(t, kb_src, list, n, n_dev, preserve, copy_keys, L);
+                      int count, int preserve, int copy_keys, const Launch& L) {
+    if (S == 4) rebuild_s<4>(t, kb_src, list, n, count, preserve, copy_keys, L);
+    else if (S == 8) rebuild_s<8>(t, kb_src, list, n, count, preserve, copy_keys, L);
+    else rebuild_s<16>(t, kb_src, list, n, count, preserve, copy_keys, L);
   }
   template <int S, class Off>
   static void neighbors_s(const TableView& t, const int32_t* keys, int64_t n, const Off& off, int64_t n_off,

@@ -477,8 +477,9 @@ ash_status check_launch(const char* where) {
   return ASH_OK;
 }
 
-// Allocates and initialises table, buffers and heap for `capacity`.
-ash_status alloc_storage(ash_map* m, int64_t capacity, cudaStream_t st) {
+// Allocates and initialises table, buffers and heap for `capacity`, together
+// with what `plan` already holds.
+ash_status alloc_storage(ash_map* m, int64_t capacity, ash::InitPlan& plan, cudaStream_t st) {
   const int64_t n_slots = slots_for(capacity, m->tuning);
   if (n_slots >= (int64_t{1} << 31)) return fail(ASH_ERR_INVALID, "capacity too large for 31-bit slot indices");
   const ash::Launch L = launch_of(m, st);
@@ -498,9 +499,10 @@ ash_status alloc_storage(ash_map* m, int64_t capacity, cudaStream_t st) {
   m->n_buckets = static_cast<uint32_t>(n_slots / m->S);
   m->pref_placed = true;
   m->heap_identity = true;
-  ASH_CUDA(cudaMemsetAsync(m->slots, 0xFF, n_slots * 8, st));
-  for (int j = 0; j < m->n_values; ++j) ASH_CUDA(cudaMemsetAsync(m->vb[j], 0, capacity * m->row_bytes[j], st));
-  ash::launch_iota(m->heap, 0, capacity, L);
+  plan.ones(m->slots, n_slots * 8);
+  plan.iota(m->heap, 0, capacity);
+  for (int j = 0; j < m->n_values; ++j) plan.zero(m->vb[j], capacity * m->row_bytes[j]);
+  ash::launch_init(plan, L);
   return check_launch("alloc_storage");
 }
 
@@ -528,18 +530,20 @@ ash_status ensure_scratch(ash_map* m, int64_t bytes, cudaStream_t st) {
   return ASH_OK;
 }
 
+ash_status alloc_win_bits(ash_map* m, int64_t bytes, cudaStream_t st) {
+  m->win_bits = static_cast<uint32_t*>(dev_alloc(m, bytes, st));
+  m->win_bits_bytes = m->win_bits ? bytes : 0;
+  return m->win_bits ? ASH_OK : fail(ASH_ERR_OOM, "winner-flag allocation failed");
+}
+
 // Winner flags of an insert of n keys: one bit per input position.
 ash_status ensure_win_bits(ash_map* m, int64_t n, cudaStream_t st) {
   const int64_t bytes = (n + 31) / 32 * 4;
   if (m->win_bits_bytes >= bytes) return ASH_OK;
   dev_free(m, m->win_bits, st);
   const int64_t want = std::max<int64_t>(bytes, m->win_bits_bytes * 2);
-  m->win_bits = static_cast<uint32_t*>(dev_alloc(m, want, st));
-  if (!m->win_bits) {
-    m->win_bits_bytes = 0;
-    return fail(ASH_ERR_OOM, "winner-flag allocation failed");
-  }
-  m->win_bits_bytes = want;
+  const ash_status s = alloc_win_bits(m, want, st);
+  if (s != ASH_OK) return s;
   // all bits start clear; every insert's commit clears the words it read
   ASH_CUDA(cudaMemsetAsync(m->win_bits, 0, want, st));
   m->win_bits_clean = true;
@@ -560,22 +564,46 @@ ash_status ensure_list_scratch(ash_map* m, cudaStream_t st) {
   return ASH_OK;
 }
 
+// The buffers of a growth that keeps indices: contents copied, value rows
+// beyond them zero, the heap continued with the new indices.
+void plan_growth(const ash_map* m, int64_t new_capacity, int32_t* kb, int32_t* heap, const std::vector<void*>& vb,
+                 ash::InitPlan& plan) {
+  const int64_t c = m->capacity;
+  plan.copy(kb, m->kb, c * m->ks * 4);
+  if (m->heap_identity) {
+    plan.iota(heap, 0, new_capacity);
+  } else {
+    plan.copy(heap, m->heap, c * 4);
+    plan.iota(heap, c, new_capacity);
+  }
+  for (int j = 0; j < m->n_values; ++j) {
+    const int64_t rb = m->row_bytes[j];
+    plan.copy(vb[j], m->vb[j], c * rb);
+    plan.zero(static_cast<char*>(vb[j]) + c * rb, (new_capacity - c) * rb);
+  }
+}
+
 // Rebuilds the table for new_capacity from the live entries (Sec. 4.5).
 // size: the exact live count (caller synchronised).
 ash_status rebuild_to(ash_map* m, int64_t new_capacity, int64_t size, cudaStream_t st) {
   __atomic_fetch_add(&m->rebuilds, 1, __ATOMIC_RELAXED);
   const ash::Launch L = launch_of(m, st);
-  // 1) collect the active indices
-  int32_t* list = static_cast<int32_t*>(dev_alloc(m, std::max<int64_t>(size, 1) * 4, st));
-  if (!list) return fail(ASH_ERR_OOM, "rehash list allocation failed");
-  ash_status s = ensure_list_scratch(m, st);
-  if (s != ASH_OK) {
-    dev_free(m, list, st);
-    return s;
+  // 1) the active indices: 0..size-1 while the heap is the identity
+  const bool identity = m->heap_identity;
+  int32_t* list = nullptr;
+  ash_status s = ASH_OK;
+  if (!identity) {
+    list = static_cast<int32_t*>(dev_alloc(m, std::max<int64_t>(size, 1) * 4, st));
+    if (!list) return fail(ASH_ERR_OOM, "rehash list allocation failed");
+    s = ensure_list_scratch(m, st);
+    if (s != ASH_OK) {
+      dev_free(m, list, st);
+      return s;
+    }
+    ash::launch_list_active(false, m->heap, m->capacity, m->ctrl, m->list_scratch, list, size, nullptr, L);
+    s = check_launch("rehash listing");
+    if (s != ASH_OK) return s;
   }
-  ash::launch_list_active(m->heap_identity, m->heap, m->capacity, m->ctrl, m->list_scratch, list, size, nullptr, L);
-  s = check_launch("rehash listing");
-  if (s != ASH_OK) return s;
 
   ash_map old = *m;  // shallow copy of the old storage pointers
   const bool preserve = new_capacity >= m->capacity;
@@ -589,7 +617,6 @@ ash_status rebuild_to(ash_map* m, int64_t new_capacity, int64_t size, cudaStream
     dev_free(m, list, st);
     return fail(ASH_ERR_OOM, "rehash table allocation failed");
   }
-  ASH_CUDA(cudaMemsetAsync(slots, 0xFF, n_slots * 8, st));
 
   int32_t* kb = m->kb;
   int32_t* heap = m->heap;
@@ -608,24 +635,29 @@ ash_status rebuild_to(ash_map* m, int64_t new_capacity, int64_t size, cudaStream
       dev_free(m, slots, st);
       return fail(ASH_ERR_OOM, "rehash buffer allocation failed");
     }
-    if (preserve) {
-      // indices are kept: copy buffers, extend the heap with the new indices
-      ASH_CUDA(cudaMemcpyAsync(kb, m->kb, m->capacity * m->ks * 4, cudaMemcpyDeviceToDevice, st));
-      ASH_CUDA(cudaMemcpyAsync(heap, m->heap, m->capacity * 4, cudaMemcpyDeviceToDevice, st));
-      ash::launch_iota(heap, m->capacity, new_capacity, L);
-      for (int j = 0; j < m->n_values; ++j) {
-        const int64_t rb = m->row_bytes[j];
-        ASH_CUDA(cudaMemcpyAsync(vb[j], m->vb[j], m->capacity * rb, cudaMemcpyDeviceToDevice, st));
-        ASH_CUDA(cudaMemsetAsync(static_cast<char*>(vb[j]) + m->capacity * rb, 0, (new_capacity - m->capacity) * rb, st));
-      }
-    } else {
-      // compaction: entry j of the list becomes index j
-      ash::launch_iota(heap, 0, new_capacity, L);
-      m->heap_identity = true;
+  }
+  ash::InitPlan plan;
+  plan.ones(slots, n_slots * 8);
+  plan.word(&m->ctrl->top_used, (static_cast<uint64_t>(size) << 32) | static_cast<uint64_t>(size));
+  if (grow && preserve) {
+    // indices are kept: copy buffers, extend the heap with the new indices
+    plan_growth(m, new_capacity, kb, heap, vb, plan);
+  } else if (grow) {
+    // compaction: entry j of the list becomes index j
+    plan.iota(heap, 0, new_capacity);
+    for (int j = 0; j < m->n_values; ++j) {
+      const int64_t rb = m->row_bytes[j];
+      if (identity) plan.copy(vb[j], m->vb[j], size * rb);
+      plan.zero(static_cast<char*>(vb[j]) + size * rb, (new_capacity - size) * rb);
+    }
+  }
+  ash::launch_init(plan, L);
+  if (grow && !preserve) {
+    m->heap_identity = true;
+    if (!identity) {
       ash::ValueCopy vc{};
       vc.n = m->n_values;
       for (int j = 0; j < m->n_values; ++j) {
-        ASH_CUDA(cudaMemsetAsync(vb[j], 0, new_capacity * m->row_bytes[j], st));
         vc.dst[j] = vb[j];
         vc.src[j] = m->vb[j];
         vc.row_bytes[j] = m->row_bytes[j];
@@ -645,10 +677,9 @@ ash_status rebuild_to(ash_map* m, int64_t new_capacity, int64_t size, cudaStream
   m->heap = heap;
   m->vb = vb;
   ash::TableView tv = view_of(m);
-  m->K.rebuild(m->S, tv, old.kb, list, size, nullptr, preserve ? 1 : 0, (!preserve) ? 1 : 0, L);
+  m->K.rebuild(m->S, tv, old.kb, list, size, ash::kCountExact, preserve ? 1 : 0, (!preserve) ? 1 : 0, L);
   s = check_launch("rehash rebuild");
   if (s != ASH_OK) return s;
-  ash::launch_set_top_used(m->ctrl, size, size, L);
   // 3) release the old storage
   dev_free(m, old.slots, st);
   if (grow) {
@@ -673,14 +704,19 @@ ash_status grow_async(ash_map* m, int64_t new_capacity, cudaStream_t st) {
   __atomic_fetch_add(&m->rebuilds, 1, __ATOMIC_RELAXED);
   const ash::Launch L = launch_of(m, st);
   const int64_t c = m->capacity;
-  int32_t* list = static_cast<int32_t*>(dev_alloc(m, c * 4, st));
-  if (!list) return fail(ASH_ERR_OOM, "growth list allocation failed");
-  ash_status s = ensure_list_scratch(m, st);
-  if (s != ASH_OK) {
-    dev_free(m, list, st);
-    return s;
+  // the live entries: 0..t-1 while the heap is the identity, else listed
+  const bool identity = m->heap_identity;
+  int32_t* list = nullptr;
+  if (!identity) {
+    list = static_cast<int32_t*>(dev_alloc(m, c * 4, st));
+    if (!list) return fail(ASH_ERR_OOM, "growth list allocation failed");
+    ash_status s = ensure_list_scratch(m, st);
+    if (s != ASH_OK) {
+      dev_free(m, list, st);
+      return s;
+    }
+    ash::launch_list_active(false, m->heap, c, m->ctrl, m->list_scratch, list, c, nullptr, L);
   }
-  ash::launch_list_active(m->heap_identity, m->heap, c, m->ctrl, m->list_scratch, list, c, nullptr, L);
   const int64_t n_slots = slots_for(new_capacity, m->tuning);
   if (n_slots >= (int64_t{1} << 31)) {
     dev_free(m, list, st);
@@ -712,17 +748,10 @@ ash_status grow_async(ash_map* m, int64_t new_capacity, cudaStream_t st) {
     }
     return fail(ASH_ERR_OOM, "growth allocation failed");
   }
-  ASH_CUDA(cudaMemsetAsync(slots, 0xFF, n_slots * 8, st));
-  if (grow) {
-    ASH_CUDA(cudaMemcpyAsync(kb, m->kb, c * m->ks * 4, cudaMemcpyDeviceToDevice, st));
-    ASH_CUDA(cudaMemcpyAsync(heap, m->heap, c * 4, cudaMemcpyDeviceToDevice, st));
-    ash::launch_iota(heap, c, new_capacity, L);
-    for (int j = 0; j < m->n_values; ++j) {
-      const int64_t rb = m->row_bytes[j];
-      ASH_CUDA(cudaMemcpyAsync(vb[j], m->vb[j], c * rb, cudaMemcpyDeviceToDevice, st));
-      ASH_CUDA(cudaMemsetAsync(static_cast<char*>(vb[j]) + c * rb, 0, (new_capacity - c) * rb, st));
-    }
-  }
+  ash::InitPlan plan;
+  plan.ones(slots, n_slots * 8);
+  if (grow) plan_growth(m, new_capacity, kb, heap, vb, plan);
+  ash::launch_init(plan, L);
   ash_map old = *m;
   m->S = m->tuning.slots_per_bucket;
   m->slots = slots;
@@ -733,8 +762,7 @@ ash_status grow_async(ash_map* m, int64_t new_capacity, cudaStream_t st) {
   m->kb = kb;
   m->heap = heap;
   m->vb = vb;
-  m->K.rebuild(m->S, view_of(m), old.kb, list, c, &m->ctrl->count, 1, 0, L);
-  ash::launch_set_used_from_count(m->ctrl, L);
+  m->K.rebuild(m->S, view_of(m), old.kb, list, c, identity ? ash::kCountTop : ash::kCountListed, 1, 0, L);
   dev_free(m, old.slots, st);
   if (grow) {
     dev_free(m, old.kb, st);
@@ -968,14 +996,15 @@ ash_status ash_create(int key_dim, int64_t capacity, int n_values, const int64_t
   m->snap_seq = rec.seq;
   m->ctrl = static_cast<ash::Ctrl*>(dev_alloc(m, sizeof(ash::Ctrl), st));
   if (!m->ctrl) { ash_destroy(m); return fail(ASH_ERR_OOM, "device allocation failed"); }
-  if (cudaMemsetAsync(m->ctrl, 0, sizeof(ash::Ctrl), st) != cudaSuccess) {
-    ash_destroy(m);
-    return cuda_fail(cudaGetLastError(), "ash_create");
-  }
-  s = alloc_storage(m, capacity, st);
+  ash::InitPlan plan;
+  plan.zero(m->ctrl, sizeof(ash::Ctrl));
   // winner flags for a first insert of up to `capacity` keys, allocated here
   // so that the insert itself allocates nothing
-  if (s == ASH_OK) s = ensure_win_bits(m, capacity, st);
+  s = alloc_win_bits(m, (capacity + 31) / 32 * 4, st);
+  if (s == ASH_OK) {
+    plan.zero(m->win_bits, m->win_bits_bytes);
+    s = alloc_storage(m, capacity, plan, st);
+  }
   if (s != ASH_OK) {
     std::string msg = g_last_error;
     ash_destroy(m);
@@ -1229,9 +1258,11 @@ ash_status ash_clear(ash_map* m, ash_stream stream) {
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   m->last_stream = st;
   const ash::Launch L = launch_of(m, st);
-  ASH_CUDA(cudaMemsetAsync(m->slots, 0xFF, m->n_slots * 8, st));
-  ash::launch_iota(m->heap, 0, m->capacity, L);
-  ash::launch_set_top_used(m->ctrl, 0, 0, L);
+  ash::InitPlan plan;
+  plan.ones(m->slots, m->n_slots * 8);
+  plan.iota(m->heap, 0, m->capacity);
+  plan.word(&m->ctrl->top_used, 0);
+  ash::launch_init(plan, L);
   m->size_ub = 0;
   m->used_ub = 0;
   m->tomb_lb = 0;

@@ -13,7 +13,7 @@ enum KernelKind {
   kKEraseResolve,
   kKRebuild,
   kKListActive,
-  kKIota,
+  kKInit,
   kKScatterRows,
   kKGatherRows,
   kKGatherKeys,
