@@ -14,7 +14,7 @@ namespace ash {
 template <int S>
 static void erase_resolve_s(const TableView& t, int64_t n, const int32_t* slot_in, uint8_t* mask, const Launch& L) {
   TraceScope ts(kKEraseResolve, L.stream);
-  erase_resolve_kernel<S><<<grid_for(n, L), L.block, 0, L.stream>>>(t, n, slot_in, mask);
+  launch_dependent(erase_resolve_kernel<S>, grid_for(n, L), L.block, L.stream, t, n, slot_in, mask);
 }
 
 void launch_erase_resolve(int S, const TableView& t, int64_t n, const int32_t* slot_in, uint8_t* mask, const Launch& L) {
@@ -302,12 +302,13 @@ void launch_init(const InitPlan& plan, const Launch& L) {
 }
 
 __global__ void snapshot_kernel(Ctrl* ctrl, Snap* snap, uint32_t seq) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (threadIdx.x == 0) publish_snapshot(ctrl, snap, seq);
 }
 
 void launch_snapshot(Ctrl* ctrl, Snap* snap, uint32_t seq, const Launch& L) {
   TraceScope ts(kKSetCtrl, L.stream);
-  snapshot_kernel<<<1, 32, 0, L.stream>>>(ctrl, snap, seq);
+  launch_dependent(snapshot_kernel, 1, 32, L.stream, ctrl, snap, seq);
 }
 
 // -------------------------------------------------------------- value rows

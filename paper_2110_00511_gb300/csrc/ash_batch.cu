@@ -6,9 +6,9 @@
 // one persistent kernel over ALL maps of that phase: claim, commit, find,
 // erase-mark and erase-resolve.  Work is cut into tiles of blockDim.x keys that
 // never straddle two operations, so a commit or erase-resolve tile still
-// aggregates its heap atomic over one map.  The five kernels plus the upload of
-// the descriptor table form one CUDA graph, built once per ring slot and
-// replayed: the kernels read everything (maps, pointers, tile counts) from the
+// aggregates its heap atomic over one map.  The five kernels, one that
+// publishes the maps' control-block snapshots, and the upload of the
+// descriptor table form one CUDA graph, built once per ring slot and replayed: the kernels read everything (maps, pointers, tile counts) from the
 // device copy of the table, so a new batch only rewrites the pinned table.
 #include <cuda_runtime.h>
 
@@ -47,11 +47,19 @@ struct BatchPhase {
   int64_t tiles;
 };
 
+// A control-block snapshot that a map asks for after the batch.
+struct BatchSnap {
+  Ctrl* ctrl;
+  Snap* snap;
+  uint32_t seq;
+};
+
 struct BatchTable {
   BatchPhase ph[kPhases];
   int32_t n_ops;
-  int32_t pad;
+  int32_t n_snaps;
   BatchOp ops[kBatchMaxOps];
+  BatchSnap snaps[kBatchMaxOps];
 };
 
 // Loads the tile starts of one phase into shared memory and maps a tile to
@@ -72,20 +80,32 @@ __device__ __forceinline__ int op_of_tile(const int64_t* s_tile0, int count, int
   return lo;
 }
 
-#define ASH_DS_CASES(FN, ...)                                       \
-  switch (op.key_dim * 100 + op.S) {                                \
-    case 104: FN<1, 4>(__VA_ARGS__); break;                         \
-    case 108: FN<1, 8>(__VA_ARGS__); break;                         \
-    case 116: FN<1, 16>(__VA_ARGS__); break;                        \
-    case 204: FN<2, 4>(__VA_ARGS__); break;                         \
-    case 208: FN<2, 8>(__VA_ARGS__); break;                         \
-    case 216: FN<2, 16>(__VA_ARGS__); break;                        \
-    case 304: FN<3, 4>(__VA_ARGS__); break;                         \
-    case 308: FN<3, 8>(__VA_ARGS__); break;                         \
-    case 316: FN<3, 16>(__VA_ARGS__); break;                        \
-    case 404: FN<4, 4>(__VA_ARGS__); break;                         \
-    case 408: FN<4, 8>(__VA_ARGS__); break;                         \
-    default: FN<4, 16>(__VA_ARGS__); break;                         \
+// The kernels exist twice: for batches whose maps all have 4-slot buckets (the
+// default), and for any bucket sizes.  The 16-slot code alone sets the
+// register count of a kernel that holds it (WIDE).
+#define ASH_DS_CASES(WIDE, FN, ...)                                 \
+  if constexpr (!(WIDE)) {                                          \
+    switch (op.key_dim) {                                           \
+      case 1: FN<1, 4>(__VA_ARGS__); break;                         \
+      case 2: FN<2, 4>(__VA_ARGS__); break;                         \
+      case 3: FN<3, 4>(__VA_ARGS__); break;                         \
+      default: FN<4, 4>(__VA_ARGS__); break;                        \
+    }                                                               \
+  } else {                                                          \
+    switch (op.key_dim * 100 + op.S) {                              \
+      case 104: FN<1, 4>(__VA_ARGS__); break;                       \
+      case 108: FN<1, 8>(__VA_ARGS__); break;                       \
+      case 116: FN<1, 16>(__VA_ARGS__); break;                      \
+      case 204: FN<2, 4>(__VA_ARGS__); break;                       \
+      case 208: FN<2, 8>(__VA_ARGS__); break;                       \
+      case 216: FN<2, 16>(__VA_ARGS__); break;                      \
+      case 304: FN<3, 4>(__VA_ARGS__); break;                       \
+      case 308: FN<3, 8>(__VA_ARGS__); break;                       \
+      case 316: FN<3, 16>(__VA_ARGS__); break;                      \
+      case 404: FN<4, 4>(__VA_ARGS__); break;                       \
+      case 408: FN<4, 8>(__VA_ARGS__); break;                       \
+      default: FN<4, 16>(__VA_ARGS__); break;                       \
+    }                                                               \
   }
 
 // In the batched kernels the full per-key protocols are the main path, so
@@ -100,11 +120,12 @@ __device__ __forceinline__ void batch_claim_one(const BatchOp& op, int64_t pos) 
 
 template <int D, int S>
 __device__ __forceinline__ void batch_find_one(const BatchOp& op, int64_t pos) {
-  int32_t k[D];
-  load_input_key<D>(op.keys, pos, k);
-  const int32_t r = find_key<D, S>(op.t, k);
-  op.idx[pos] = r;
-  op.mask[pos] = r >= 0 ? 1 : 0;
+  int32_t k[1][D], r[1];
+  const bool ok[1] = {true};
+  load_input_key<D>(op.keys, pos, k[0]);
+  find_keys<D, S, 1>(op.t, k, ok, r);
+  op.idx[pos] = r[0];
+  op.mask[pos] = r[0] >= 0 ? 1 : 0;
 }
 
 template <int D, int S>
@@ -112,6 +133,7 @@ __device__ __forceinline__ void batch_mark_one(const BatchOp& op, int64_t pos) {
   op.idx[pos] = erase_mark_one<D, S>(op.t, op.keys, pos);
 }
 
+template <bool WIDE>
 __global__ void __launch_bounds__(kBatchThreads) batch_claim_kernel(const BatchTable* __restrict__ tb) {
   __shared__ int64_t s_tile0[kBatchMaxOps];
   load_tile_starts(tb, kPhaseInsert, s_tile0);
@@ -119,7 +141,7 @@ __global__ void __launch_bounds__(kBatchThreads) batch_claim_kernel(const BatchT
   for (int64_t tile = blockIdx.x; tile < ph.tiles; tile += gridDim.x) {
     const BatchOp& op = tb->ops[ph.first + op_of_tile(s_tile0, ph.count, tile)];
     const int64_t pos = (tile - op.tile0) * blockDim.x + threadIdx.x;
-    if (pos < op.n) { ASH_DS_CASES(batch_claim_one, op, pos) }
+    if (pos < op.n) { ASH_DS_CASES(WIDE, batch_claim_one, op, pos) }
   }
 }
 
@@ -147,6 +169,7 @@ __global__ void __launch_bounds__(kBatchThreads) batch_commit_kernel(const Batch
   }
 }
 
+template <bool WIDE>
 __global__ void __launch_bounds__(kBatchThreads) batch_find_kernel(const BatchTable* __restrict__ tb) {
   __shared__ int64_t s_tile0[kBatchMaxOps];
   load_tile_starts(tb, kPhaseFind, s_tile0);
@@ -154,10 +177,11 @@ __global__ void __launch_bounds__(kBatchThreads) batch_find_kernel(const BatchTa
   for (int64_t tile = blockIdx.x; tile < ph.tiles; tile += gridDim.x) {
     const BatchOp& op = tb->ops[ph.first + op_of_tile(s_tile0, ph.count, tile)];
     const int64_t pos = (tile - op.tile0) * blockDim.x + threadIdx.x;
-    if (pos < op.n) { ASH_DS_CASES(batch_find_one, op, pos) }
+    if (pos < op.n) { ASH_DS_CASES(WIDE, batch_find_one, op, pos) }
   }
 }
 
+template <bool WIDE>
 __global__ void __launch_bounds__(kBatchThreads) batch_erase_mark_kernel(const BatchTable* __restrict__ tb) {
   __shared__ int64_t s_tile0[kBatchMaxOps];
   load_tile_starts(tb, kPhaseErase, s_tile0);
@@ -165,10 +189,11 @@ __global__ void __launch_bounds__(kBatchThreads) batch_erase_mark_kernel(const B
   for (int64_t tile = blockIdx.x; tile < ph.tiles; tile += gridDim.x) {
     const BatchOp& op = tb->ops[ph.first + op_of_tile(s_tile0, ph.count, tile)];
     const int64_t pos = (tile - op.tile0) * blockDim.x + threadIdx.x;
-    if (pos < op.n) { ASH_DS_CASES(batch_mark_one, op, pos) }
+    if (pos < op.n) { ASH_DS_CASES(WIDE, batch_mark_one, op, pos) }
   }
 }
 
+template <bool WIDE>
 __global__ void __launch_bounds__(kBatchThreads) batch_erase_resolve_kernel(const BatchTable* __restrict__ tb) {
   __shared__ int64_t s_tile0[kBatchMaxOps];
   __shared__ int s_warp[33];
@@ -179,10 +204,17 @@ __global__ void __launch_bounds__(kBatchThreads) batch_erase_resolve_kernel(cons
   for (int64_t tile = blockIdx.x; tile < ph.tiles; tile += gridDim.x) {
     const BatchOp& op = tb->ops[ph.first + op_of_tile(s_tile0, ph.count, tile)];
     const int64_t base0 = (tile - op.tile0) * blockDim.x;
-    if (op.S == 4) erase_resolve_tile<4>(op.t, op.n, base0, op.idx, op.mask, s_warp, &s_cnt, &s_base);
+    if (!WIDE || op.S == 4) erase_resolve_tile<4>(op.t, op.n, base0, op.idx, op.mask, s_warp, &s_cnt, &s_base);
     else if (op.S == 8) erase_resolve_tile<8>(op.t, op.n, base0, op.idx, op.mask, s_warp, &s_cnt, &s_base);
     else erase_resolve_tile<16>(op.t, op.n, base0, op.idx, op.mask, s_warp, &s_cnt, &s_base);
   }
+}
+
+// Publishes the snapshots of every map that asked for one, once its
+// operations are done.
+__global__ void __launch_bounds__(kBatchMaxOps) batch_snapshot_kernel(const BatchTable* __restrict__ tb) {
+  const int i = threadIdx.x;
+  if (i < tb->n_snaps) publish_snapshot(tb->snaps[i].ctrl, tb->snaps[i].snap, tb->snaps[i].seq);
 }
 
 }  // namespace ash
@@ -197,8 +229,8 @@ struct ash_batch {
   struct Slot {
     BatchTable* h = nullptr;  // pinned
     BatchTable* d = nullptr;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
+    cudaGraph_t graph[2] = {};  // 4-slot buckets only, any bucket sizes
+    cudaGraphExec_t exec[2] = {};
     cudaEvent_t done = nullptr;
     bool used = false;
     int32_t* scratch = nullptr;  // erase slot indices
@@ -210,32 +242,39 @@ struct ash_batch {
 
 namespace {
 
+template <bool WIDE>
 ash_status build_graph(ash_batch* b, ash_batch::Slot& s) {
-  if (cudaGraphCreate(&s.graph, 0) != cudaSuccess) return cuda_fail(cudaGetLastError(), "cudaGraphCreate");
+  cudaGraph_t& graph = s.graph[WIDE];
+  if (graph) cudaGraphDestroy(graph);  // left by an attempt that failed
+  graph = nullptr;
+  if (cudaGraphCreate(&graph, 0) != cudaSuccess) return cuda_fail(cudaGetLastError(), "cudaGraphCreate");
   cudaGraphNode_t copy = nullptr;
-  if (cudaGraphAddMemcpyNode1D(&copy, s.graph, nullptr, 0, s.d, s.h, sizeof(BatchTable), cudaMemcpyHostToDevice) !=
+  if (cudaGraphAddMemcpyNode1D(&copy, graph, nullptr, 0, s.d, s.h, sizeof(BatchTable), cudaMemcpyHostToDevice) !=
       cudaSuccess)
     return cuda_fail(cudaGetLastError(), "cudaGraphAddMemcpyNode1D");
-  void* kernels[5] = {reinterpret_cast<void*>(batch_claim_kernel), reinterpret_cast<void*>(batch_commit_kernel),
-                      reinterpret_cast<void*>(batch_find_kernel), reinterpret_cast<void*>(batch_erase_mark_kernel),
-                      reinterpret_cast<void*>(batch_erase_resolve_kernel)};
+  void* kernels[6] = {reinterpret_cast<void*>(batch_claim_kernel<WIDE>), reinterpret_cast<void*>(batch_commit_kernel),
+                      reinterpret_cast<void*>(batch_find_kernel<WIDE>),
+                      reinterpret_cast<void*>(batch_erase_mark_kernel<WIDE>),
+                      reinterpret_cast<void*>(batch_erase_resolve_kernel<WIDE>),
+                      reinterpret_cast<void*>(batch_snapshot_kernel)};
   cudaGraphNode_t prev = copy;
   const BatchTable* arg = s.d;
   void* args[1] = {&arg};
   for (void* k : kernels) {
     cudaKernelNodeParams p{};
     p.func = k;
-    p.gridDim = dim3(b->grid);
-    p.blockDim = dim3(kBatchThreads);
+    const bool snapshots = k == kernels[5];
+    p.gridDim = dim3(snapshots ? 1 : b->grid);
+    p.blockDim = dim3(snapshots ? kBatchMaxOps : kBatchThreads);
     p.sharedMemBytes = 0;
     p.kernelParams = args;
     p.extra = nullptr;
     cudaGraphNode_t node = nullptr;
-    if (cudaGraphAddKernelNode(&node, s.graph, &prev, 1, &p) != cudaSuccess)
+    if (cudaGraphAddKernelNode(&node, graph, &prev, 1, &p) != cudaSuccess)
       return cuda_fail(cudaGetLastError(), "cudaGraphAddKernelNode");
     prev = node;
   }
-  if (cudaGraphInstantiate(&s.exec, s.graph, 0) != cudaSuccess)
+  if (cudaGraphInstantiate(&s.exec[WIDE], graph, 0) != cudaSuccess)
     return cuda_fail(cudaGetLastError(), "cudaGraphInstantiate");
   return ASH_OK;
 }
@@ -299,8 +338,10 @@ ash_status ash_batch_destroy(ash_batch* b) {
   DeviceGuard g(b->device);
   for (auto& s : b->slot) {
     if (s.done) cudaEventSynchronize(s.done);
-    if (s.exec) cudaGraphExecDestroy(s.exec);
-    if (s.graph) cudaGraphDestroy(s.graph);
+    for (cudaGraphExec_t e : s.exec)
+      if (e) cudaGraphExecDestroy(e);
+    for (cudaGraph_t gr : s.graph)
+      if (gr) cudaGraphDestroy(gr);
     if (s.h) cudaFreeHost(s.h);
     if (s.d) cudaFree(s.d);
     if (s.done) cudaEventDestroy(s.done);
@@ -406,23 +447,32 @@ ash_status ash_batch_run(ash_batch* b, const ash_batch_op* ops, int n_ops, ash_s
     tb->ph[ph].tiles = tiles;
   }
   tb->n_ops = k;
-  if (!sl.exec) {
-    ash_status s = build_graph(b, sl);
+  int wide = 0;
+  for (int i = 0; i < k; ++i) wide |= tb->ops[i].S != 4 ? 1 : 0;
+  if (!sl.exec[wide]) {
+    ash_status s = wide ? build_graph<true>(b, sl) : build_graph<false>(b, sl);
     if (s != ASH_OK) return s;
   }
-  {
-    TraceScope ts(kKBatch, st, 5);
-    if (cudaGraphLaunch(sl.exec, st) != cudaSuccess) return cuda_fail(cudaGetLastError(), "cudaGraphLaunch");
-  }
+  // ---- what the maps' snapshots will report, published by the graph itself
+  std::vector<ash_map*> snapped;
+  tb->n_snaps = 0;
   for (int i = 0; i < n_ops; ++i)
-    if (ops[i].op == ASH_OP_INSERT || ops[i].op == ASH_OP_ACTIVATE) {
-      ops[i].map->pref_placed = false;  // keys placed in slot order
-      maybe_snapshot(ops[i].map, st);
-    } else if (ops[i].op == ASH_OP_ERASE) {
-      ops[i].map->heap_identity = false;
-      ops[i].map->erased_since_snap += ops[i].n;
-      maybe_snapshot(ops[i].map, st);
-    }
+    if (ops[i].op == ASH_OP_ERASE) ops[i].map->erased_since_snap += ops[i].n;
+  for (int i = 0; i < n_ops; ++i) {
+    ash_map* m = ops[i].map;
+    if (ops[i].op == ASH_OP_FIND || std::find(snapped.begin(), snapped.end(), m) != snapped.end()) continue;
+    if (!snapshot_wanted(m, st, 0)) continue;
+    snapped.push_back(m);
+    tb->snaps[tb->n_snaps++] = {m->ctrl, m->snap_dev, m->snap_seq};
+  }
+  {
+    TraceScope ts(kKBatch, st, 6);
+    if (cudaGraphLaunch(sl.exec[wide], st) != cudaSuccess) return cuda_fail(cudaGetLastError(), "cudaGraphLaunch");
+  }
+  for (ash_map* m : snapped) snapshot_issued(m);
+  for (int i = 0; i < n_ops; ++i)
+    if (ops[i].op == ASH_OP_INSERT || ops[i].op == ASH_OP_ACTIVATE) ops[i].map->pref_placed = false;  // keys placed in slot order
+    else if (ops[i].op == ASH_OP_ERASE) ops[i].map->heap_identity = false;
   if (cudaEventRecord(sl.done, st) != cudaSuccess) return cuda_fail(cudaGetLastError(), "cudaEventRecord");
   sl.used = true;
   return ASH_OK;

@@ -419,9 +419,12 @@ __device__ __forceinline__ bool join_claim(const TableView& t, uint64_t* p, uint
 // Order of the EMPTY slots a claim tries (claim_key):
 //   kClaimSlotOrder  slot order, one CAS site per slot (unrolled): the
 //                    fastest form, used out of line as a slow path
-//   kClaimSlotMask   slot order, one CAS site for all slots (a bit-mask
-//                    loop): fewer registers, for the batched kernel that
-//                    inlines the protocol for every key dimension
+//   kClaimSlotMask   slot order, one compare site and one CAS site for all
+//                    slots (bit-mask loops): fewer registers, for the batched
+//                    kernel that inlines the protocol for every key dimension
+//                    and runs it on full warps (claims of 24 maps 32 -> 28
+//                    us; out of line in claim_bucket_kernel the same compares
+//                    made 10^8 ranged keys 5 % slower)
 //   kClaimPrefFirst  the key's preferred slot first in its home bucket, then
 //                    slot order (keeps the preferred-slot invariant)
 constexpr int kClaimSlotOrder = 0;
@@ -446,13 +449,44 @@ __device__ __forceinline__ int32_t claim_key(const TableView& t, const In& keys,
     uint64_t* bp = t.slots + static_cast<size_t>(b) * S;
     uint64_t w[S];
     load_bucket<S, false>(bp, w);
+    if constexpr (ORDER == kClaimSlotMask) {
+      // the first fingerprint match is picked before anything is compared, so
+      // the lanes of a warp wait for one compare, not for one per slot
+      int at = -1, matches = 0;
+      uint64_t seen = 0;
 #pragma unroll
-    for (int s = 0; s < S; ++s) {
-      const int m = claim_match<D, In>(w[s], fp, k, keys, t.kb);
-      if (m == 2) return kClaimExists;
-      if (m == 1)
-        return join_claim<FLAGS>(t, bp + s, lo32(w[s]), mine, static_cast<uint32_t>(pos)) ? static_cast<int32_t>(b * S + s)
-                                                                                    : kClaimJoined;
+      for (int s = S - 1; s >= 0; --s) {
+        if (lo32(w[s]) != kNoIndex && hi32(w[s]) == fp) {
+          at = s;
+          seen = w[s];
+          ++matches;
+        }
+      }
+      while (matches > 0) {
+        const int m = claim_match<D, In>(seen, fp, k, keys, t.kb);
+        if (m == 2) return kClaimExists;
+        if (m == 1)
+          return join_claim<FLAGS>(t, bp + at, lo32(seen), mine, static_cast<uint32_t>(pos)) ? static_cast<int32_t>(b * S + at)
+                                                                                      : kClaimJoined;
+        if (--matches == 0) break;
+        const int after = at;  // another key with this fingerprint: the next match
+#pragma unroll
+        for (int s = S - 1; s >= 0; --s) {
+          if (s > after && lo32(w[s]) != kNoIndex && hi32(w[s]) == fp) {
+            at = s;
+            seen = w[s];
+          }
+        }
+      }
+    } else {
+#pragma unroll
+      for (int s = 0; s < S; ++s) {
+        const int m = claim_match<D, In>(w[s], fp, k, keys, t.kb);
+        if (m == 2) return kClaimExists;
+        if (m == 1)
+          return join_claim<FLAGS>(t, bp + s, lo32(w[s]), mine, static_cast<uint32_t>(pos)) ? static_cast<int32_t>(b * S + s)
+                                                                                      : kClaimJoined;
+      }
     }
     if constexpr (ORDER == kClaimSlotOrder) {
 #pragma unroll
@@ -1127,16 +1161,32 @@ __device__ __forceinline__ int32_t erase_mark_one(const TableView& t, const int3
     uint64_t* bp = t.slots + static_cast<size_t>(b) * S;
     uint64_t w[S];
     load_bucket<S, false>(bp, w);
+    // candidates: committed with an equal fingerprint, or already marked
+    // (fingerprint gone); the former first, each compared by itself, so the
+    // lanes of a warp usually wait for one compare
     bool stop = false;
+    uint32_t same = 0, marked = 0;
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-      stop |= (w[s] == kEmpty);
       const uint32_t lo = lo32(w[s]), hi = hi32(w[s]);
-      // committed with an equal fingerprint, or already marked (fingerprint gone)
-      if (res < 0 && lo < kClaimBit && (hi == fp || hi < kFpBit) && kb_equal<D>(t.kb, lo, k)) {
-        if (hi > static_cast<uint32_t>(pos))
-          atomicMin(reinterpret_cast<unsigned long long*>(bp + s), (static_cast<unsigned long long>(pos) << 32) | lo);
-        res = static_cast<int32_t>(b * S + s);
+      stop |= (w[s] == kEmpty);
+      same |= (lo < kClaimBit && hi == fp ? 1u : 0u) << s;
+      marked |= (lo < kClaimBit && hi < kFpBit ? 1u : 0u) << s;
+    }
+    while (same | marked) {
+      const int at = __ffs(same ? same : marked) - 1;
+      if (same) same &= same - 1;
+      else marked &= marked - 1;
+      uint64_t word = 0;
+#pragma unroll
+      for (int s = 0; s < S; ++s)
+        if (s == at) word = w[s];
+      if (kb_equal<D>(t.kb, lo32(word), k)) {
+        if (hi32(word) > static_cast<uint32_t>(pos))
+          atomicMin(reinterpret_cast<unsigned long long*>(bp + at),
+                    (static_cast<unsigned long long>(pos) << 32) | lo32(word));
+        res = static_cast<int32_t>(b * S + at);
+        break;
       }
     }
     if (stop) break;
@@ -1149,6 +1199,7 @@ template <int D, int S>
 __global__ void __launch_bounds__(256) erase_mark_kernel(TableView t, const int32_t* __restrict__ keys, int64_t n,
                                                          int32_t* __restrict__ slot_out) {
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   for (int64_t pos = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; pos < n; pos += stride)
     slot_out[pos] = erase_mark_one<D, S>(t, keys, pos);
 }
@@ -1220,6 +1271,7 @@ __global__ void __launch_bounds__(256) erase_resolve_kernel(TableView t, int64_t
   __shared__ int s_warp[33];
   __shared__ int s_cnt;
   __shared__ int s_base;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t base = static_cast<int64_t>(blockIdx.x) * blockDim.x; base < n; base += stride)
     erase_resolve_tile<S>(t, n, base, slot_in, mask, s_warp, &s_cnt, &s_base);
@@ -1503,7 +1555,7 @@ struct DimLaunchers {
   template <int S>
   static void erase_mark_s(const TableView& t, const int32_t* keys, int64_t n, int32_t* slot_out, const Launch& L) {
     TraceScope ts(kKEraseMark, L.stream);
-    erase_mark_kernel<D, S><<<grid_for(n, L), L.block, 0, L.stream>>>(t, keys, n, slot_out);
+    launch_dependent(erase_mark_kernel<D, S>, grid_for(n, L), L.block, L.stream, t, keys, n, slot_out);
   }
   static void erase_mark(int S, const TableView& t, const int32_t* keys, int64_t n, int32_t* slot_out, const Launch& L) {
     if (S == 4) erase_mark_s<4>(t, keys, n, slot_out, L);
