@@ -1644,7 +1644,7 @@ def per_op_figures(args, device, hbm_peak):
 def batched_figures(args, device, reps=15):
     """Many maps, one mixed batch each (key_dim 2-4, capacities log-uniform in
     2^10..2^21, 30/60/10 insert/find/erase, rho ~ U(0.2, 1)), serviced (a) as
-    ONE graph launch of the batched kernels and (b) as plain per-map calls
+    ONE run of the batched kernels and (b) as plain per-map calls
     (insert, find, erase for each map) through the same binding.  Maps are
     cleared between repetitions (untimed); each repetition is timed with CUDA
     events around the whole service."""

@@ -330,7 +330,7 @@ ash_status ash_set_tuning(ash_map* map, const ash_tuning* tuning_host);
 ash_status ash_sync_status(ash_map* map, ash_stream stream);
 
 /* ---------------------------------------------------------------------------
- * Batched execution: one CUDA-graph launch services many maps (the paper has
+ * Batched execution: one chain of launches services many maps (the paper has
  * no batched form; it applies the per-map operations above to many maps at
  * once).  Phases run in the order insert/activate -> find -> erase, each as
  * one persistent kernel over all maps of the batch, so a map with an insert
@@ -381,7 +381,7 @@ ash_status ash_autotune(int key_dim, int64_t capacity, float rho, int device, as
  * live/capacity ratio past max_load (and rebuilds its table when erased
  * slots would pass the map's max_used_fraction) on a growth stream, leaving
  * that tenant out of batches until the growth finishes, and runs each batch
- * as one ash_batch_run graph between an upload and a download on separate
+ * as one ash_batch_run between an upload and a download on separate
  * streams.
  * Requests that arrive while batches are on the GPU join the next batch.
  *   ash_server_wait: blocks until the request's outputs are on the host,

@@ -456,7 +456,7 @@ def ash_batch_run(handle, ops, stream=None):
 
 
 class Batch:
-    """One batched-execution context (a ring of CUDA graphs).  `run` takes
+    """One batched-execution context (a ring of descriptor tables).  `run` takes
     (HashMap, op, keys, values) tuples and returns [(buf_indices, masks)]."""
 
     def __init__(self, device=0):

@@ -1,4 +1,4 @@
-// Batched execution: one CUDA-graph launch services many maps.
+// Batched execution: one short chain of launches services many maps.
 //
 // A batch is a list of operations, at most one per (map, phase), on maps of
 // key dimension 1..4.  Phases run in the order insert/activate -> find ->
@@ -6,10 +6,14 @@
 // one persistent kernel over ALL maps of that phase: claim, commit, find,
 // erase-mark and erase-resolve.  Work is cut into tiles of blockDim.x keys that
 // never straddle two operations, so a commit or erase-resolve tile still
-// aggregates its heap atomic over one map.  The five kernels, one that
-// publishes the maps' control-block snapshots, and the upload of the
-// descriptor table form one CUDA graph, built once per ring slot and replayed: the kernels read everything (maps, pointers, tile counts) from the
-// device copy of the table, so a new batch only rewrites the pinned table.
+// aggregates its heap atomic over one map.  The kernels read everything (maps,
+// pointers, tile counts) from a descriptor table that the first launch copies
+// from a pinned ring slot; a last one publishes the maps' control-block
+// snapshots.  All are programmatic dependents of the one before, and a phase
+// without work is not launched.  (As a CUDA graph of a table copy and six
+// kernels the same work took 255 against 237 us for 24 maps, and 96 against
+// 81 us when it held finds only: a graph runs its empty phases, copies the
+// whole table and has no programmatic edges.)
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -58,13 +62,22 @@ struct BatchTable {
   BatchPhase ph[kPhases];
   int32_t n_ops;
   int32_t n_snaps;
-  BatchOp ops[kBatchMaxOps];
   BatchSnap snaps[kBatchMaxOps];
+  BatchOp ops[kBatchMaxOps];  // last: only the part in use is copied
 };
+
+// Copies the table's part in use from pinned host memory (the SMs read it
+// over the CPU-GPU link).
+__global__ void __launch_bounds__(1024) batch_upload_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst,
+                                                            int units) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < units; i += gridDim.x * blockDim.x) dst[i] = src[i];
+}
 
 // Loads the tile starts of one phase into shared memory and maps a tile to
 // its operation (binary search over at most kBatchMaxOps entries).
 __device__ __forceinline__ void load_tile_starts(const BatchTable* tb, int phase, int64_t* s_tile0) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // every batch kernel is a programmatic dependent
   const BatchPhase ph = tb->ph[phase];
   for (int i = threadIdx.x; i < ph.count; i += blockDim.x) s_tile0[i] = tb->ops[ph.first + i].tile0;
   __syncthreads();
@@ -213,6 +226,7 @@ __global__ void __launch_bounds__(kBatchThreads) batch_erase_resolve_kernel(cons
 // Publishes the snapshots of every map that asked for one, once its
 // operations are done.
 __global__ void __launch_bounds__(kBatchMaxOps) batch_snapshot_kernel(const BatchTable* __restrict__ tb) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int i = threadIdx.x;
   if (i < tb->n_snaps) publish_snapshot(tb->snaps[i].ctrl, tb->snaps[i].snap, tb->snaps[i].seq);
 }
@@ -229,8 +243,6 @@ struct ash_batch {
   struct Slot {
     BatchTable* h = nullptr;  // pinned
     BatchTable* d = nullptr;
-    cudaGraph_t graph[2] = {};  // 4-slot buckets only, any bucket sizes
-    cudaGraphExec_t exec[2] = {};
     cudaEvent_t done = nullptr;
     bool used = false;
     int32_t* scratch = nullptr;  // erase slot indices
@@ -242,41 +254,29 @@ struct ash_batch {
 
 namespace {
 
+// The batch's kernels on st, empty phases left out.
 template <bool WIDE>
-ash_status build_graph(ash_batch* b, ash_batch::Slot& s) {
-  cudaGraph_t& graph = s.graph[WIDE];
-  if (graph) cudaGraphDestroy(graph);  // left by an attempt that failed
-  graph = nullptr;
-  if (cudaGraphCreate(&graph, 0) != cudaSuccess) return cuda_fail(cudaGetLastError(), "cudaGraphCreate");
-  cudaGraphNode_t copy = nullptr;
-  if (cudaGraphAddMemcpyNode1D(&copy, graph, nullptr, 0, s.d, s.h, sizeof(BatchTable), cudaMemcpyHostToDevice) !=
-      cudaSuccess)
-    return cuda_fail(cudaGetLastError(), "cudaGraphAddMemcpyNode1D");
-  void* kernels[6] = {reinterpret_cast<void*>(batch_claim_kernel<WIDE>), reinterpret_cast<void*>(batch_commit_kernel),
-                      reinterpret_cast<void*>(batch_find_kernel<WIDE>),
-                      reinterpret_cast<void*>(batch_erase_mark_kernel<WIDE>),
-                      reinterpret_cast<void*>(batch_erase_resolve_kernel<WIDE>),
-                      reinterpret_cast<void*>(batch_snapshot_kernel)};
-  cudaGraphNode_t prev = copy;
-  const BatchTable* arg = s.d;
-  void* args[1] = {&arg};
-  for (void* k : kernels) {
-    cudaKernelNodeParams p{};
-    p.func = k;
-    const bool snapshots = k == kernels[5];
-    p.gridDim = dim3(snapshots ? 1 : b->grid);
-    p.blockDim = dim3(snapshots ? kBatchMaxOps : kBatchThreads);
-    p.sharedMemBytes = 0;
-    p.kernelParams = args;
-    p.extra = nullptr;
-    cudaGraphNode_t node = nullptr;
-    if (cudaGraphAddKernelNode(&node, graph, &prev, 1, &p) != cudaSuccess)
-      return cuda_fail(cudaGetLastError(), "cudaGraphAddKernelNode");
-    prev = node;
+void launch_batch(const ash_batch* b, const ash_batch::Slot& s, cudaStream_t st) {
+  const BatchTable* tb = s.h;
+  const BatchTable* d = s.d;
+  auto grid = [&](int phase) {
+    const int64_t tiles = tb->ph[phase].tiles;
+    return static_cast<int>(tiles < b->grid ? tiles : b->grid);
+  };
+  const int units = static_cast<int>((offsetof(BatchTable, ops) + sizeof(BatchOp) * tb->n_ops + 15) / 16);
+  launch_dependent(batch_upload_kernel, (units + 1023) / 1024, 1024, st, reinterpret_cast<const uint4*>(s.h),
+                   reinterpret_cast<uint4*>(s.d), units);
+  if (tb->ph[kPhaseInsert].tiles > 0) {
+    launch_dependent(batch_claim_kernel<WIDE>, grid(kPhaseInsert), kBatchThreads, st, d);
+    launch_dependent(batch_commit_kernel, grid(kPhaseInsert), kBatchThreads, st, d);
   }
-  if (cudaGraphInstantiate(&s.exec[WIDE], graph, 0) != cudaSuccess)
-    return cuda_fail(cudaGetLastError(), "cudaGraphInstantiate");
-  return ASH_OK;
+  if (tb->ph[kPhaseFind].tiles > 0)
+    launch_dependent(batch_find_kernel<WIDE>, grid(kPhaseFind), kBatchThreads, st, d);
+  if (tb->ph[kPhaseErase].tiles > 0) {
+    launch_dependent(batch_erase_mark_kernel<WIDE>, grid(kPhaseErase), kBatchThreads, st, d);
+    launch_dependent(batch_erase_resolve_kernel<WIDE>, grid(kPhaseErase), kBatchThreads, st, d);
+  }
+  if (tb->n_snaps > 0) launch_dependent(batch_snapshot_kernel, 1, kBatchMaxOps, st, d);
 }
 
 void* batch_alloc(ash_batch* b, size_t bytes, cudaStream_t st) {
@@ -338,10 +338,6 @@ ash_status ash_batch_destroy(ash_batch* b) {
   DeviceGuard g(b->device);
   for (auto& s : b->slot) {
     if (s.done) cudaEventSynchronize(s.done);
-    for (cudaGraphExec_t e : s.exec)
-      if (e) cudaGraphExecDestroy(e);
-    for (cudaGraph_t gr : s.graph)
-      if (gr) cudaGraphDestroy(gr);
     if (s.h) cudaFreeHost(s.h);
     if (s.d) cudaFree(s.d);
     if (s.done) cudaEventDestroy(s.done);
@@ -447,13 +443,9 @@ ash_status ash_batch_run(ash_batch* b, const ash_batch_op* ops, int n_ops, ash_s
     tb->ph[ph].tiles = tiles;
   }
   tb->n_ops = k;
-  int wide = 0;
-  for (int i = 0; i < k; ++i) wide |= tb->ops[i].S != 4 ? 1 : 0;
-  if (!sl.exec[wide]) {
-    ash_status s = wide ? build_graph<true>(b, sl) : build_graph<false>(b, sl);
-    if (s != ASH_OK) return s;
-  }
-  // ---- what the maps' snapshots will report, published by the graph itself
+  bool wide = false;
+  for (int i = 0; i < k; ++i) wide |= tb->ops[i].S != 4;
+  // ---- the snapshots that the maps ask for, published by the batch's last kernel
   std::vector<ash_map*> snapped;
   tb->n_snaps = 0;
   for (int i = 0; i < n_ops; ++i)
@@ -465,9 +457,12 @@ ash_status ash_batch_run(ash_batch* b, const ash_batch_op* ops, int n_ops, ash_s
     snapped.push_back(m);
     tb->snaps[tb->n_snaps++] = {m->ctrl, m->snap_dev, m->snap_seq};
   }
-  {
-    TraceScope ts(kKBatch, st, 6);
-    if (cudaGraphLaunch(sl.exec[wide], st) != cudaSuccess) return cuda_fail(cudaGetLastError(), "cudaGraphLaunch");
+  if (k > 0) {
+    TraceScope ts(kKBatch, st, 7);
+    if (wide) launch_batch<true>(b, sl, st);
+    else launch_batch<false>(b, sl, st);
+    ash_status s = check_launch("batch_run");
+    if (s != ASH_OK) return s;
   }
   for (ash_map* m : snapped) snapshot_issued(m);
   for (int i = 0; i < n_ops; ++i)

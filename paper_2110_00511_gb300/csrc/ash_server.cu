@@ -11,7 +11,7 @@
 //   3. forms a batch of at most one admitted request per tenant (so each
 //      tenant's requests run in arrival order), grows a tenant map x2 before
 //      an insert would push its live/capacity ratio past max_load,
-//   4. uploads the batch on a copy stream, runs it as ONE ash_batch_run graph
+//   4. uploads the batch on a copy stream, runs it as ONE ash_batch_run
 //      on the compute stream, downloads its outputs on a second copy stream
 //      and marks the requests done from a host callback.
 // The worker does not wait for a batch before launching the next one, so
@@ -453,7 +453,7 @@ void worker_loop(ash_server* s) {
       lk.lock();
       continue;
     }
-    // 4) launch: upload, one batched graph, download, host callback
+    // 4) launch: upload, one batched run, download, host callback
     std::vector<ash_batch_op> ops;
     if (st == ASH_OK) {
       for (Request* r : pick) {

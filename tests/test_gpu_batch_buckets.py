@@ -1,5 +1,5 @@
 """One batch context serving maps of 4-slot buckets only, wider ones only and
-both in turn (its two kinds of graph on the same ring slots), over more rounds
+both in turn (its two sets of kernels, on the same ring slots), over more rounds
 than the ring has slots: masks and values equal those of plain calls."""
 import pytest
 import torch
