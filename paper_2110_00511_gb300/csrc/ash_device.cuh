@@ -81,6 +81,7 @@ struct TableView {
   uint32_t max_probes;
   int32_t capacity;
   int32_t flags;        // kViewHeapIdentity | kViewPrefPlaced
+  int32_t key_dim;
   // Winner flags of one insert (one bit per input position, zero before the
   // claim kernel), or null.  A position that displaces an equal key's claim
   // with a lower position sets the displaced position's bit, so after the
@@ -228,6 +229,17 @@ __device__ __forceinline__ bool input_key_equal(const In& keys, int64_t pos, con
 #pragma unroll
   for (int j = 0; j < D; ++j) eq &= (o[j] == k[j]);
   return eq;
+}
+
+// Home bucket of kB row i, for the kernels that are not compiled per key
+// dimension (same hash as hash_key).
+__device__ __forceinline__ uint32_t home_of_row(const int32_t* kb, int d, uint32_t n_buckets, uint32_t i) {
+  const int ks = d <= 1 ? 1 : (d <= 2 ? 2 : (d <= 4 ? 4 : 8));
+  const int32_t* row = kb + static_cast<size_t>(i) * ks;
+  uint64_t h = static_cast<uint64_t>(d);
+#pragma unroll 1
+  for (int j = 0; j < d; ++j) h += static_cast<uint64_t>(static_cast<uint32_t>(__ldg(row + j))) * coord_mult(j);
+  return home_bucket(mix64(h), n_buckets);
 }
 
 // Loads row i of kB into o (KS values; the first D are the key).

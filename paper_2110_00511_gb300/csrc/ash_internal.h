@@ -59,10 +59,9 @@ struct ash_map {
   uint32_t snap_seq = 0;           // number of the last snapshot requested
   int snap_state = 0;              // 0 idle, 1 in flight, 2 in flight but stale
   int64_t added_since_snap = 0;    // insert/activate keys issued after the snapshot's copy
-  // Lower bound on tombstones (used - live of the last landed snapshot):
-  // inserts never reuse a tombstone, so the count only grows until a rebuild
-  // (which resets it).  Drives the clean-up rebuilds (tombstones_need_rebuild).
-  int64_t tomb_lb = 0;
+  // Tombstones (used - live) when the control block was last seen by the
+  // host.  Drives the clean-up rebuilds (tombstones_need_rebuild).
+  int64_t tombs = 0;
   int64_t erased_since_snap = 0;   // erase keys issued after the last snapshot (tombstones may have formed)
   // Snapshots are taken only while every insert/activate of the map has come
   // on one stream (then stream order makes "snapshot + keys issued since" an

@@ -12,7 +12,9 @@
 //                 (claim_pref_kernel, while the table fits in L2; keys that
 //                 find it taken are queued per warp and claimed from their
 //                 buckets in dense rounds), or the first EMPTY slot of the
-//                 loaded home bucket (claim_bucket_kernel).  A thread that
+//                 loaded home bucket (claim_bucket_kernel).  A key whose home
+//                 bucket is full walks its chain (claim_key) and may take a
+//                 tombstone on it.  A thread that
 //                 meets a claimed slot compares its key with the READ-ONLY
 //                 input row of the claimant (never with a half-written kB
 //                 row, which removes the torn-copy race of Sec. 4.4.2) and,
@@ -30,9 +32,9 @@
 // erase           two kernels: mark (atomicMin of the input position into the
 //                 slot's high word, keeping the buffer index) and resolve (the
 //                 lowest position wins, frees the index with one atomic per
-//                 block, and empties the slot, or leaves a tombstone when its
-//                 bucket holds no EMPTY slot or, under the preferred-slot
-//                 invariant, another live key prefers it).  Allocation and
+//                 block, and empties the slot, or leaves a tombstone when a
+//                 probe chain may pass its bucket or, under the preferred-
+//                 slot invariant, another live key prefers it).  Allocation and
 //                 free never run in the same kernel (the atomicAdd/atomicSub
 //                 conflict that Sec. 4.3.1 warns about).
 // rebuild         inserts already-unique keys (rehash, Sec. 4.5) into an empty
@@ -416,14 +418,13 @@ __device__ __forceinline__ bool join_claim(const TableView& t, uint64_t* p, uint
   return true;
 }
 
-// Order of the EMPTY slots a claim tries (claim_key):
-//   kClaimSlotOrder  slot order, one CAS site per slot (unrolled): the
-//                    fastest form, used out of line as a slow path
-//   kClaimSlotMask   slot order, one compare site and one CAS site for all
-//                    slots (bit-mask loops): fewer registers, for the batched
-//                    kernel that inlines the protocol for every key dimension
-//                    and runs it on full warps (claims of 24 maps 32 -> 28
-//                    us; out of line in claim_bucket_kernel the same compares
+// Order in which a claim takes the EMPTY slots of a bucket (claim_key):
+//   kClaimSlotOrder  slot order, used out of line as a slow path
+//   kClaimSlotMask   slot order, one compare site for all slots (a loop over
+//                    the matches): fewer registers, for the batched kernel
+//                    that inlines the protocol for every key dimension and
+//                    runs it on full warps (claims of 24 maps 32 -> 28 us;
+//                    out of line in claim_bucket_kernel the same compares
 //                    made 10^8 ranged keys 5 % slower)
 //   kClaimPrefFirst  the key's preferred slot first in its home bucket, then
 //                    slot order (keeps the preferred-slot invariant)
@@ -431,12 +432,31 @@ constexpr int kClaimSlotOrder = 0;
 constexpr int kClaimSlotMask = 1;
 constexpr int kClaimPrefFirst = 2;
 
-// The full claim protocol for one key, from its home bucket: 1) any slot of
-// the bucket holding an equal key ends the search; 2) otherwise the EMPTY
-// slots are claimed in the order ORDER gives, and a lost CAS re-checks the
-// winner's word for an equal key; 3) a bucket without EMPTY slots sends the
-// key to the next bucket.  FLAGS: winner flags may be set (t.lost); the
-// batched kernel, which has none, compiles without them.
+// The full claim protocol for one key, a walk from its home bucket: 1) any
+// slot holding an equal key ends the search; 2) the walk ends at the first
+// bucket with an EMPTY slot, where the key is known to be absent; 3) the key
+// takes the first TOMBSTONE of the buckets without an EMPTY slot that it
+// walked past, else an EMPTY slot of the last bucket.  A lost CAS compares
+// with the winner's word and starts the walk again.
+//
+// Equal keys of one batch cannot take two slots.  A slot only goes from free
+// (EMPTY or TOMBSTONE, and of one kind while it is free) to taken during an
+// insert, and every path prefers free slots in one order: by bucket along the
+// chain, within a bucket EMPTY before TOMBSTONE, then by position.  Had two
+// equal keys taken slots x and then y, both slots were free in both walks
+// (the second walk passed x before it was taken, else it would have met the
+// equal key there; y was free until taken last), and the walks preferred
+// them differently.
+//
+// Reusing tombstones keeps the runs of full buckets from growing: a run of
+// length L collects the keys that hash into it, and when these could only be
+// placed past its end, every insert / erase cycle of a sliding window left
+// the run longer by a share of L, until the tombstone count called for a
+// rebuild.  GB300: a window of 262k keys over 1M entries 101 -> 69 us a pass
+// (no rebuild in 1200 passes, 19 before), 24 maps in one batch 514 -> 118 us.
+//
+// FLAGS: winner flags may be set (t.lost); the batched kernel, which has
+// none, compiles without them.
 template <int D, int S, class In, int ORDER, bool FLAGS = true>
 __device__ __forceinline__ int32_t claim_key(const TableView& t, const In& keys, int64_t pos) {
   int32_t k[D];
@@ -444,8 +464,10 @@ __device__ __forceinline__ int32_t claim_key(const TableView& t, const In& keys,
   const uint64_t h = hash_key<D>(k);
   const uint32_t fp = fingerprint(h);
   const uint64_t mine = (static_cast<uint64_t>(fp) << 32) | (kClaimBit | static_cast<uint32_t>(pos));
-  uint32_t b = home_bucket(h, t.n_buckets);
-  for (uint32_t probe = 0; probe < t.max_probes; ++probe) {
+  const uint32_t home = home_bucket(h, t.n_buckets);
+  uint32_t b = home;
+  uint32_t tomb = kNoIndex;  // first tombstone passed, as a slot index
+  for (uint32_t probe = 0; probe < t.max_probes;) {
     uint64_t* bp = t.slots + static_cast<size_t>(b) * S;
     uint64_t w[S];
     load_bucket<S, false>(bp, w);
@@ -488,40 +510,41 @@ __device__ __forceinline__ int32_t claim_key(const TableView& t, const In& keys,
                                                                                       : kClaimJoined;
       }
     }
-    if constexpr (ORDER == kClaimSlotOrder) {
+    uint32_t empty = 0, tombs = 0;
 #pragma unroll
-      for (int s = 0; s < S; ++s) {
-        if (w[s] == kEmpty) {
-          const uint64_t old = atomicCAS(reinterpret_cast<unsigned long long*>(bp + s),
-                                         static_cast<unsigned long long>(kEmpty), static_cast<unsigned long long>(mine));
-          if (old == kEmpty) return static_cast<int32_t>(b * S + s);
-          const int m = claim_match<D, In>(old, fp, k, keys, t.kb);
-          if (m == 2) return kClaimExists;
-          if (m == 1)
-            return join_claim<FLAGS>(t, bp + s, lo32(old), mine, static_cast<uint32_t>(pos)) ? static_cast<int32_t>(b * S + s)
-                                                                                      : kClaimJoined;
-        }
-      }
-    } else {
-      // EMPTY slots of the snapshot as a bit mask (one CAS site for all)
-      uint32_t emask = 0;
-#pragma unroll
-      for (int s = 0; s < S; ++s) emask |= (w[s] == kEmpty ? 1u : 0u) << s;
-      const uint32_t pbit = ORDER == kClaimPrefFirst && probe == 0 ? 1u << pref_slot<S>(fp) : 0u;
-      while (emask) {
-        const int s = (emask & pbit) ? static_cast<int>(pref_slot<S>(fp)) : __ffs(emask) - 1;
-        emask &= ~(1u << s);
-        const uint64_t old = atomicCAS(reinterpret_cast<unsigned long long*>(bp + s),
-                                       static_cast<unsigned long long>(kEmpty), static_cast<unsigned long long>(mine));
-        if (old == kEmpty) return static_cast<int32_t>(b * S + s);
-        const int m = claim_match<D, In>(old, fp, k, keys, t.kb);
-        if (m == 2) return kClaimExists;
-        if (m == 1)
-          return join_claim<FLAGS>(t, bp + s, lo32(old), mine, static_cast<uint32_t>(pos)) ? static_cast<int32_t>(b * S + s)
-                                                                                    : kClaimJoined;
-      }
+    for (int s = 0; s < S; ++s) {
+      empty |= (w[s] == kEmpty ? 1u : 0u) << s;
+      tombs |= (w[s] == kTombstone ? 1u : 0u) << s;
     }
-    b = next_bucket(b, t.n_buckets);
+    if (!empty) {
+      if (tomb == kNoIndex && tombs) tomb = b * S + __ffs(tombs) - 1;
+      b = next_bucket(b, t.n_buckets);
+      ++probe;
+      if (probe < t.max_probes || tomb == kNoIndex) continue;
+      // no EMPTY slot within max_probes buckets, but a tombstone
+    }
+    uint32_t slot = tomb;
+    uint64_t free_word = kTombstone;
+    if (tomb == kNoIndex) {
+      const uint32_t pref = pref_slot<S>(fp);
+      slot = b * S + (ORDER == kClaimPrefFirst && probe == 0 && ((empty >> pref) & 1u) ? pref : __ffs(empty) - 1);
+      free_word = kEmpty;
+    }
+    const uint64_t old = atomicCAS(reinterpret_cast<unsigned long long*>(t.slots + slot),
+                                   static_cast<unsigned long long>(free_word), static_cast<unsigned long long>(mine));
+    if (old == free_word) {
+      // the commit counts every winner's slot as newly used
+      if (free_word == kTombstone) atomicAdd(&t.ctrl->top_used, 0ull - (1ull << 32));
+      return static_cast<int32_t>(slot);
+    }
+    const int m = claim_match<D, In>(old, fp, k, keys, t.kb);
+    if (m == 2) return kClaimExists;
+    if (m == 1)
+      return join_claim<FLAGS>(t, t.slots + slot, lo32(old), mine, static_cast<uint32_t>(pos)) ? static_cast<int32_t>(slot)
+                                                                                        : kClaimJoined;
+    b = home;  // another key was faster
+    tomb = kNoIndex;
+    probe = 0;
   }
   atomicOr(&t.ctrl->status, kStatusTableFull);
   return kClaimFailed;
@@ -1205,6 +1228,26 @@ __global__ void __launch_bounds__(256) erase_mark_kernel(TableView t, const int3
 }
 
 // ------------------------------------------------------------ erase: resolve
+// Whether no key that stays in the table probes on past bucket b: such a key
+// would have to sit in the next bucket (which holds an EMPTY slot, so none of
+// its chains goes further) with another home bucket.  Marked words leave the
+// table in this kernel, so they do not count; a slot of the next bucket that
+// another thread empties meanwhile only makes the answer truer.
+template <int S>
+__device__ __noinline__ bool nobody_probes_past(const uint64_t* slots, const int32_t* kb, uint32_t n_buckets,
+                                                int key_dim, uint32_t b) {
+  const uint32_t nb = next_bucket(b, n_buckets);
+  if (nb == b) return false;
+  bool empty = false;
+#pragma unroll 1
+  for (int j = 0; j < S; ++j) {
+    const uint64_t w = load_slot_relaxed(slots + static_cast<size_t>(nb) * S + j);
+    empty |= (w == kEmpty);
+    if (is_committed(w) && home_of_row(kb, key_dim, n_buckets, lo32(w)) != nb) return false;
+  }
+  return empty;
+}
+
 // One tile of blockDim.x positions starting at base0.  Every thread of the
 // block must call it (block-wide scan and barriers).
 template <int S>
@@ -1220,12 +1263,12 @@ __device__ __forceinline__ void erase_resolve_tile(const TableView& t, int64_t n
     w = load_slot_relaxed(t.slots + s);
     win = hi32(w) == static_cast<uint32_t>(pos);
     if (win) {
-      // EMPTY only when the bucket already has an EMPTY slot (no probe chain
-      // passes through it) and, while the map keeps the preferred-slot
-      // invariant, no other live key of the bucket prefers the freed slot; a
-      // TOMBSTONE otherwise (the freed slot itself holds a marked word, which
-      // never counts).  The bucket is read 32 bytes at a time to keep few
-      // words live.
+      // EMPTY only when no probe chain passes through the bucket (it already
+      // has an EMPTY slot, or nobody_probes_past it) and, while the map keeps
+      // the preferred-slot invariant, no other live key of the bucket prefers
+      // the freed slot; a TOMBSTONE otherwise (the freed slot itself holds a
+      // marked word, which never counts).  The bucket is read 32 bytes at a
+      // time to keep few words live.
       const uint64_t* bp = t.slots + static_cast<size_t>(s / S) * S;
       const uint32_t own = static_cast<uint32_t>(s) & (S - 1);
       bool preferred = false;
@@ -1239,7 +1282,9 @@ __device__ __forceinline__ void erase_resolve_tile(const TableView& t, int64_t n
           preferred |= is_committed(cw[j]) && pref_slot<S>(hi32(cw[j])) == own;
         }
       }
-      to_empty &= !(preferred && (t.flags & kViewPrefPlaced));
+      preferred &= (t.flags & kViewPrefPlaced) != 0;
+      if (!to_empty && !preferred) to_empty = nobody_probes_past<S>(t.slots, t.kb, t.n_buckets, t.key_dim, static_cast<uint32_t>(s) / S);
+      to_empty &= !preferred;
     }
   }
   int rank, total;

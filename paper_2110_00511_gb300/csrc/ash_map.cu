@@ -333,6 +333,7 @@ ash::TableView view_of(const ash_map* m) {
                      : m->n_buckets;
   t.capacity = static_cast<int32_t>(m->capacity);
   t.flags = (m->heap_identity ? ash::kViewHeapIdentity : 0) | (m->pref_placed ? ash::kViewPrefPlaced : 0);
+  t.key_dim = m->key_dim;
   t.lost = nullptr;
   t.snap = nullptr;
   t.snap_seq = 0;
@@ -387,7 +388,7 @@ ash_status refresh(ash_map* m, cudaStream_t st, int64_t* top, int64_t* used, int
   tighten_bounds(m);  // folds in a snapshot that has landed
   m->size_ub = *top;
   m->used_ub = *used;
-  if (*used - *top > m->tomb_lb) m->tomb_lb = *used - *top;  // exact now
+  m->tombs = *used - *top;
   return ASH_OK;
 }
 
@@ -401,21 +402,21 @@ void tighten_bounds(ash_map* m) {
     const int64_t used = snap_used + m->added_since_snap;
     if (top < m->size_ub) m->size_ub = top;
     if (used < m->used_ub) m->used_ub = used;
-    if (snap_used - snap_top > m->tomb_lb) m->tomb_lb = snap_used - snap_top;
+    m->tombs = snap_used - snap_top;
   }
   m->snap_state = 0;
 }
 
-// Erased slots whose bucket has no EMPTY slot stay tombstones, and inserts
-// claim only EMPTY slots, so under insert/erase churn the runs of full
-// buckets lengthen: measured on a 2^24-capacity map, a find of 1M keys took
-// 3x as long as on a rebuilt table with tombstones at 0.3 of the live count,
-// 14x at 1.3 and 27x at 2.0, with the used slots (0.29-0.55 of the table)
-// still below max_used_fraction.  A table whose known tombstones pass a
-// quarter of its live entries (and 1/64 of its slots) is rebuilt.
+// Erase leaves a tombstone where a probe chain may pass (or another key
+// prefers the slot), and claims reuse only those of buckets without an EMPTY
+// slot, so tombstones can gather and lengthen the chains: when no claim reused
+// any, a find of 1M keys on a 2^24-capacity map took 3x as long as on a
+// rebuilt table with tombstones at 0.3 of the live count, 14x at 1.3 and 27x
+// at 2.0.  A table whose known tombstones pass a quarter of its live entries
+// (and 1/64 of its slots) is rebuilt.
 bool tombstones_need_rebuild(const ash_map* m) {
   const int64_t live = m->size_ub;
-  return m->tomb_lb > m->n_slots / 64 && 4 * m->tomb_lb > live;
+  return m->tombs > m->n_slots / 64 && 4 * m->tombs > live;
 }
 
 void invalidate_snapshot(ash_map* m) {
@@ -690,7 +691,7 @@ ash_status rebuild_to(ash_map* m, int64_t new_capacity, int64_t size, cudaStream
   dev_free(m, list, st);
   m->size_ub = size;
   m->used_ub = size;
-  m->tomb_lb = 0;
+  m->tombs = 0;
   invalidate_snapshot(m);
   return check_launch("rehash");
 }
@@ -771,7 +772,7 @@ ash_status grow_async(ash_map* m, int64_t new_capacity, cudaStream_t st) {
   }
   dev_free(m, list, st);
   m->used_ub = m->size_ub;
-  m->tomb_lb = 0;
+  m->tombs = 0;
   invalidate_snapshot(m);  // a snapshot taken before the rebuild would report its tombstones
   return check_launch("grow_async");
 }
@@ -1265,7 +1266,7 @@ ash_status ash_clear(ash_map* m, ash_stream stream) {
   ash::launch_init(plan, L);
   m->size_ub = 0;
   m->used_ub = 0;
-  m->tomb_lb = 0;
+  m->tombs = 0;
   m->pref_placed = true;
   m->heap_identity = true;
   invalidate_snapshot(m);
