@@ -563,11 +563,12 @@ __device__ __noinline__ int32_t claim_one(const TableView t, const In keys, int6
 // compare once (claimant's input row or kB row); on no match, CAS the first
 // EMPTY slot (PrefFirst: the preferred slot when it is EMPTY).  The loads,
 // compares and CASes of the DK keys are issued back to back.  Anything else
-// (several fingerprint matches, a lost CAS, a full bucket) runs claim_one,
-// which is safe because this path changed nothing then.
+// (several fingerprint matches, a lost CAS, a full bucket) is left to
+// claim_one (slow[q]), which is safe because this path changed nothing then.
 template <int D, int S, int DK, class In, bool PrefFirst>
 __device__ __forceinline__ void claim_from_bucket(const TableView& t, const In& keys, const int64_t (&pos)[DK],
-                                                  const bool (&v)[DK], int32_t* __restrict__ slot_out) {
+                                                  const bool (&v)[DK], int32_t* __restrict__ slot_out,
+                                                  bool (&slow)[DK]) {
   constexpr int KS = KeyStride<D>::value;
   int32_t k[DK][D];
   uint32_t fp[DK], b[DK];
@@ -627,7 +628,7 @@ __device__ __forceinline__ void claim_from_bucket(const TableView& t, const In& 
     }
   }
   int32_t res[DK];
-  bool cas[DK], slow[DK];
+  bool cas[DK];
 #pragma unroll
   for (int q = 0; q < DK; ++q) {
     res[q] = kClaimFailed;
@@ -670,33 +671,77 @@ __device__ __forceinline__ void claim_from_bucket(const TableView& t, const In& 
       if (old[q] == kEmpty) res[q] = static_cast<int32_t>(b[q] * S + es[q]);
       else slow[q] = true;
     }
-    if (slow[q]) res[q] = claim_one<D, S, In, PrefFirst>(t, keys, pos[q]);  // rare
-    if (v[q]) slot_out[pos[q]] = res[q];
+    if (v[q] && !slow[q]) slot_out[pos[q]] = res[q];
   }
+}
+
+// A warp's list in shared memory of positions put off to a round of their
+// own, so that slower paths run on full warps instead of stalling every warp
+// for a few lanes.  Every lane of the warp calls push and take.
+struct WarpList {
+  int32_t* at;
+  int n = 0;  // warp-uniform
+  __device__ explicit WarpList(int32_t* storage) : at(storage) {}
+  __device__ __forceinline__ void push(bool mine, int64_t pos) {
+    const int lane = threadIdx.x & 31;
+    const unsigned bal = __ballot_sync(0xFFFFFFFFu, mine);
+    if (mine) at[n + __popc(bal & ((1u << lane) - 1u))] = static_cast<int32_t>(pos);
+    n += __popc(bal);
+    __syncwarp();
+  }
+  // Removes the last 32 entries (or what there is): this lane's, -1 for none.
+  __device__ __forceinline__ int64_t take() {
+    const int lane = threadIdx.x & 31;
+    const int from = n > 32 ? n - 32 : 0;
+    const int64_t pos = from + lane < n ? at[from + lane] : -1;
+    __syncwarp();
+    n = from;
+    return pos;
+  }
+};
+
+// Claims a round of put-off positions by the full protocol.
+template <int D, int S, class In, bool PrefFirst>
+__device__ __forceinline__ void claim_slow_round(const TableView& t, const In& keys, WarpList& list,
+                                                 int32_t* __restrict__ slot_out) {
+  const int64_t pos = list.take();
+  if (pos >= 0) slot_out[pos] = claim_one<D, S, In, PrefFirst>(t, keys, pos);
+  __syncwarp();
 }
 
 // Claim kernel, bucket load first: KPT keys per thread, each claimed from its
 // loaded home bucket (two dependent accesses per key: bucket load, CAS) in
-// slot order.  The better choice when the table does not stay in L2: the
-// loads bring the buckets in with deep miss queues and the CASes then hit L2.
-// Slot order does not keep the preferred-slot invariant (preferred-first
-// placement measured 5-10 % slower here), so the host clears the map's flag.
+// slot order; keys that need the full protocol (mostly full home buckets) are
+// queued per warp and claimed 32 at a time: though 2 % of the keys, most
+// warps have one, and running the protocol for it at once cost more than all
+// its other keys' CASes (GB300, 10^8 keys by ranges: activate and find 9.18 ->
+// 8.56 ms).  The better choice when the table does not stay in L2: the loads bring the buckets in with deep miss queues
+// and the CASes then hit L2.  Slot order does not keep the preferred-slot
+// invariant (preferred-first placement measured 5-10 % slower here), so the
+// host clears the map's flag.
 template <int D, int S, int KPT, class In = const int32_t*>
 __global__ void __launch_bounds__(256) claim_bucket_kernel(TableView t, const In keys, int64_t n,
                                                            int32_t* __restrict__ slot_out) {
   // a programmatic dependent of the previous kernel: wait for its grid (a no-op otherwise)
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  __shared__ int32_t s_slow[8][32 + 32 * KPT];
+  WarpList slow(s_slow[threadIdx.x >> 5]);
+  const int lane = threadIdx.x & 31;
   const int64_t step = static_cast<int64_t>(gridDim.x) * blockDim.x * KPT;
-  for (int64_t base = static_cast<int64_t>(blockIdx.x) * blockDim.x * KPT + threadIdx.x; base < n; base += step) {
+  for (int64_t base = static_cast<int64_t>(blockIdx.x) * blockDim.x * KPT + threadIdx.x; base - lane < n; base += step) {
     int64_t p[KPT];
-    bool v[KPT];
+    bool v[KPT], put_off[KPT];
 #pragma unroll
     for (int q = 0; q < KPT; ++q) {
       p[q] = base + static_cast<int64_t>(q) * blockDim.x;
       v[q] = p[q] < n;
     }
-    claim_from_bucket<D, S, KPT, In, false>(t, keys, p, v, slot_out);
+    claim_from_bucket<D, S, KPT, In, false>(t, keys, p, v, slot_out, put_off);
+#pragma unroll
+    for (int q = 0; q < KPT; ++q) slow.push(put_off[q], p[q]);
+    while (slow.n >= 32) claim_slow_round<D, S, In, false>(t, keys, slow, slot_out);
   }
+  if (slow.n > 0) claim_slow_round<D, S, In, false>(t, keys, slow, slot_out);
 }
 
 // Claim kernel, preferred slot first.  Each warp takes 32 * KPT consecutive
@@ -709,10 +754,11 @@ __global__ void __launch_bounds__(256) claim_bucket_kernel(TableView t, const In
 // in the warp's shared-memory list; whenever the list holds 32 * kDL keys the
 // warp claims them from their buckets together, kDL per lane
 // (claim_from_bucket), so the slower path runs on dense warps instead of
-// stalling every warp for a few lanes.  A CAS that misses L2 waits on DRAM
+// stalling every warp for a few lanes (a second queue for those that then
+// need the full protocol cost registers and 3 % at 4M keys).  A CAS that misses L2 waits on DRAM
 // inside the atomic unit, so this path pays off while the table stays in L2.
 template <int D, int S, int KPT, class In = const int32_t*>
-__global__ void __launch_bounds__(256) claim_pref_kernel(TableView t, const In keys, int64_t n,
+__global__ void __launch_bounds__(256, S == 4 && D <= 4 ? 6 : 1) claim_pref_kernel(TableView t, const In keys, int64_t n,
                                                          int32_t* __restrict__ slot_out) {
   // a programmatic dependent of the previous kernel: wait for its grid (a no-op otherwise)
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -803,7 +849,7 @@ __global__ void __launch_bounds__(256) claim_pref_kernel(TableView t, const In k
     __syncwarp();
     while (qn >= kDrain) {
       int64_t p[kDL];
-      bool v[kDL];
+      bool v[kDL], slow[kDL];
 #pragma unroll
       for (int r = 0; r < kDL; ++r) {
         v[r] = true;
@@ -811,19 +857,25 @@ __global__ void __launch_bounds__(256) claim_pref_kernel(TableView t, const In k
       }
       __syncwarp();
       qn -= kDrain;
-      claim_from_bucket<D, S, kDL, In, true>(t, keys, p, v, slot_out);
+      claim_from_bucket<D, S, kDL, In, true>(t, keys, p, v, slot_out, slow);
+#pragma unroll
+      for (int r = 0; r < kDL; ++r)
+        if (slow[r]) slot_out[p[r]] = claim_one<D, S, In, true>(t, keys, p[r]);
     }
   }
   __syncwarp();
   if (qn > 0) {
     int64_t p[kDL];
-    bool v[kDL];
+    bool v[kDL], slow[kDL];
 #pragma unroll
     for (int r = 0; r < kDL; ++r) {
       v[r] = r * 32 + lane < qn;
       p[r] = v[r] ? queue[r * 32 + lane] : 0;
     }
-    claim_from_bucket<D, S, kDL, In, true>(t, keys, p, v, slot_out);
+    claim_from_bucket<D, S, kDL, In, true>(t, keys, p, v, slot_out, slow);
+#pragma unroll
+    for (int r = 0; r < kDL; ++r)
+      if (slow[r]) slot_out[p[r]] = claim_one<D, S, In, true>(t, keys, p[r]);
   }
 }
 
