@@ -755,8 +755,10 @@ __global__ void __launch_bounds__(256) claim_bucket_kernel(TableView t, const In
 // warp claims them from their buckets together, kDL per lane
 // (claim_from_bucket), so the slower path runs on dense warps instead of
 // stalling every warp for a few lanes (a second queue for those that then
-// need the full protocol cost registers and 3 % at 4M keys).  A CAS that misses L2 waits on DRAM
-// inside the atomic unit, so this path pays off while the table stays in L2.
+// need the full protocol cost registers and 3 % at 4M keys).  A CAS that
+// misses L2 waits on DRAM inside the atomic unit, so this path pays off while
+// the table stays in L2.  Six blocks per SM for 4-slot buckets (40 registers):
+// 4M claims 90 us, against 107 with four blocks and 105 with eight.
 template <int D, int S, int KPT, class In = const int32_t*>
 __global__ void __launch_bounds__(256, S == 4 && D <= 4 ? 6 : 1) claim_pref_kernel(TableView t, const In keys, int64_t n,
                                                          int32_t* __restrict__ slot_out) {

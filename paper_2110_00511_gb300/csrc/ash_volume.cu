@@ -246,62 +246,101 @@ __global__ void __launch_bounds__(kThreads) integrate_kernel(const int32_t* __re
 // every listed cell read missing blocks, which are invalid.
 constexpr int kRangeTile = 8;
 
-__global__ void range_reset_kernel(unsigned int* __restrict__ zmin, unsigned int* __restrict__ zmax, int n_tiles) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n_tiles) {
+// Occupancy of the block lattice, wrapped to 128 blocks per axis (one bit per
+// block), and of its cells of 4 x 4 x 4 blocks.  A clear bit proves a block (or
+// a whole cell) missing; a set one may stand for another block 128 away.
+constexpr int kOccBits = 7;
+constexpr int kOccCell = 2;  // log2 blocks per cell edge
+constexpr int kOccFineWords = 1 << (3 * kOccBits - 5);
+constexpr int kOccWords = kOccFineWords + (1 << (3 * (kOccBits - kOccCell) - 5));
+
+template <int BITS>
+__device__ __forceinline__ uint32_t occ_bit(int32_t x, int32_t y, int32_t z) {
+  constexpr uint32_t M = (1u << BITS) - 1u;
+  return (((static_cast<uint32_t>(z) & M) << BITS | (static_cast<uint32_t>(y) & M)) << BITS) | (static_cast<uint32_t>(x) & M);
+}
+
+__device__ __forceinline__ uint32_t fine_bit(const int32_t (&K)[3]) { return occ_bit<kOccBits>(K[0], K[1], K[2]); }
+
+__device__ __forceinline__ uint32_t cell_bit(const int32_t (&K)[3]) {
+  return 32u * kOccFineWords + occ_bit<kOccBits - kOccCell>(K[0] >> kOccCell, K[1] >> kOccCell, K[2] >> kOccCell);
+}
+
+__global__ void range_reset_kernel(unsigned int* __restrict__ zmin, unsigned int* __restrict__ zmax, int n_tiles,
+                                   uint32_t* __restrict__ occupied, unsigned long long* __restrict__ next_chunk) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+  const int stride = gridDim.x * blockDim.x;
+  if (tid == 0) *next_chunk = 0ull;
+  for (int i = tid; i < kOccWords / 4; i += stride) reinterpret_cast<uint4*>(occupied)[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (int i = tid; i < n_tiles; i += stride) {
     zmin[i] = 0x7F800000u;  // +inf: no block over this tile yet
     zmax[i] = 0u;
   }
 }
 
-// Thread per live block (grid-stride over at most n_max entries of `live`,
-// the first *count_dev of which are valid).  Depths are positive, so their
-// float bit patterns order like the values and integer atomics keep the
-// extremes.
+__device__ __forceinline__ float min_of_8(float v) {
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o, 8));
+  return v;
+}
+
+__device__ __forceinline__ float max_of_8(float v) {
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o, 8));
+  return v;
+}
+
+// Warp per live block: lane c (mod 8) projects corner c, then the lanes share
+// out the tiles under the block.  live == nullptr: the live blocks are kB rows
+// 0..t-1 (identity heap), else the first *count_dev entries of `live`, n_max
+// at most.  Depths are positive, so their float bit patterns order like the
+// values and integer atomics keep the extremes.  Each block also sets its
+// occupancy bits; zmin == nullptr: nothing else.  (A thread per block, going
+// through corners and tiles one after the other, took 11.5 us for 2000 blocks
+// and few of the chip's warps.)
 __global__ void __launch_bounds__(kThreads) block_range_kernel(const int32_t* __restrict__ kb, int ks, int ell,
+                                                               const Ctrl* __restrict__ ctrl,
                                                                const int32_t* __restrict__ live, int64_t n_max,
                                                                const int64_t* __restrict__ count_dev, Cam cam,
                                                                float voxel, int32_t width, int32_t height,
                                                                int tiles_x, int tiles_y, unsigned int* __restrict__ zmin,
-                                                               unsigned int* __restrict__ zmax) {
-  int64_t n = *count_dev;
+                                                               unsigned int* __restrict__ zmax,
+                                                               uint32_t* __restrict__ occupied) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  int64_t n = live ? *count_dev : static_cast<int64_t>(static_cast<uint32_t>(ctrl->top_used));
   if (n > n_max) n = n_max;
-  for (int64_t r = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; r < n;
-       r += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int32_t* key = kb + static_cast<int64_t>(__ldg(live + r)) * ks;
-    float lo[3], hi[3];
+  const int lane = threadIdx.x & 31;
+  const int64_t n_warps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
+  for (int64_t r = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); r < n; r += n_warps) {
+    const int32_t* key = kb + (live ? static_cast<int64_t>(__ldg(live + r)) : r) * ks;
     bool far_out = false;  // beyond |g| < 2^18 the margins are not proven: cover everything
+    const int32_t K[3] = {__ldg(key), __ldg(key + 1), __ldg(key + 2)};
+    if (lane < 2) {
+      const uint32_t bit = lane == 0 ? fine_bit(K) : cell_bit(K);
+      atomicOr(occupied + (bit >> 5), 1u << (bit & 31));
+    }
+    if (zmin == nullptr) continue;
+    float at[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const int32_t kk = __ldg(key + a);
+      const int32_t kk = K[a];
       far_out |= (kk >= (1 << 18) / ell || kk <= -(1 << 18) / ell);
       const float k = static_cast<float>(kk) * static_cast<float>(ell);
-      lo[a] = (k - 1.0f) * voxel;
-      hi[a] = (k + static_cast<float>(ell)) * voxel;
+      at[a] = (lane >> a) & 1 ? (k + static_cast<float>(ell)) * voxel : (k - 1.0f) * voxel;
     }
-    float z_lo = 3.0e38f, z_hi = -3.0e38f, u_lo = 3.0e38f, u_hi = -3.0e38f, v_lo = 3.0e38f, v_hi = -3.0e38f;
-    bool behind = false;
-#pragma unroll
-    for (int corner = 0; corner < 8; ++corner) {
-      const float x = (corner & 1) ? hi[0] : lo[0];
-      const float y = (corner & 2) ? hi[1] : lo[1];
-      const float z = (corner & 4) ? hi[2] : lo[2];
-      const float xc = cam.e[0] * x + cam.e[1] * y + cam.e[2] * z + cam.e[3];
-      const float yc = cam.e[4] * x + cam.e[5] * y + cam.e[6] * z + cam.e[7];
-      const float zc = cam.e[8] * x + cam.e[9] * y + cam.e[10] * z + cam.e[11];
-      z_lo = fminf(z_lo, zc);
-      z_hi = fmaxf(z_hi, zc);
-      if (zc <= 1.0e-6f) {
-        behind = true;
-      } else {
-        const float u = cam.fx * (xc / zc) + cam.cx;
-        const float v = cam.fy * (yc / zc) + cam.cy;
-        u_lo = fminf(u_lo, u);
-        u_hi = fmaxf(u_hi, u);
-        v_lo = fminf(v_lo, v);
-        v_hi = fmaxf(v_hi, v);
-      }
-    }
+    const float xc = cam.e[0] * at[0] + cam.e[1] * at[1] + cam.e[2] * at[2] + cam.e[3];
+    const float yc = cam.e[4] * at[0] + cam.e[5] * at[1] + cam.e[6] * at[2] + cam.e[7];
+    const float zc = cam.e[8] * at[0] + cam.e[9] * at[1] + cam.e[10] * at[2] + cam.e[11];
+    const bool corner_behind = zc <= 1.0e-6f;
+    const float u = cam.fx * (xc / zc) + cam.cx, v = cam.fy * (yc / zc) + cam.cy;
+    const float z_lo = min_of_8(fminf(3.0e38f, zc));
+    float z_hi = max_of_8(fmaxf(-3.0e38f, zc));
+    const float u_lo = min_of_8(corner_behind ? 3.0e38f : fminf(3.0e38f, u));
+    const float u_hi = max_of_8(corner_behind ? -3.0e38f : fmaxf(-3.0e38f, u));
+    const float v_lo = min_of_8(corner_behind ? 3.0e38f : fminf(3.0e38f, v));
+    const float v_hi = max_of_8(corner_behind ? -3.0e38f : fmaxf(-3.0e38f, v));
+    const bool behind = __any_sync(0xFFFFFFFFu, corner_behind);
     if (!far_out && !(z_hi > 0.0f)) continue;  // wholly behind the camera: no sample (t > 0) reaches it
     int tx0, tx1, ty0, ty1;
     unsigned int zl;
@@ -323,11 +362,13 @@ __global__ void __launch_bounds__(kThreads) block_range_kernel(const int32_t* __
       zl = __float_as_uint(fmaxf(z_lo, 0.0f));
     }
     const unsigned int zh = __float_as_uint(z_hi);
-    for (int ty = ty0; ty <= ty1; ++ty)
-      for (int tx = tx0; tx <= tx1; ++tx) {
-        atomicMin(zmin + ty * tiles_x + tx, zl);
-        atomicMax(zmax + ty * tiles_x + tx, zh);
-      }
+    const int nx = tx1 - tx0 + 1;
+    const int n_over = nx * (ty1 - ty0 + 1);
+    for (int j = lane; j < n_over; j += 32) {
+      const int tile = (ty0 + j / nx) * tiles_x + tx0 + j % nx;
+      atomicMin(zmin + tile, zl);
+      atomicMax(zmax + tile, zh);
+    }
   }
 }
 
@@ -342,14 +383,44 @@ __global__ void __launch_bounds__(kThreads) block_range_kernel(const int32_t* __
 // local index map, K is looked up there and its int32 value row names the
 // block's index in the volume's buffers.
 //
-// Two shortcuts leave the result unchanged.  The last block's lookup is kept,
-// so consecutive samples in one block cost one probe.  And every rounding
-// step of the sample arithmetic is monotone, so each coordinate of g, and of
-// K, is monotone in i: if samples i and m > i fall in the same block, so do
-// all samples between them.  When a block is missing, the kernel estimates
-// the last sample m inside its cell from the ray's exit, recomputes sample m
-// exactly as above, and when it still falls in the block jumps over the
-// samples up to m (all invalid by definition).
+// Two shortcuts leave the result unchanged.  A block is looked up once for all
+// consecutive samples in it.  And every rounding step of the sample arithmetic
+// is monotone, so each coordinate of g, of K and of K's 4 x 4 x 4 cell is
+// monotone in i: if samples i and m > i fall in the same block (or cell), so
+// do all samples between them.  When the occupancy bits or the lookup show
+// that the block or its cell is missing, the kernel estimates the last sample
+// m inside it from the ray's exit, recomputes sample m exactly as above, and
+// when it still falls there jumps over the samples up to m (all invalid by
+// definition).
+//
+// What bounds it: the serial chain of each ray (sample -> block -> voxel
+// loads), few rays being much longer than the rest, and the issue slots of
+// the sample arithmetic.  So a ray takes kRaySamples consecutive samples at
+// once, loads the voxels of those that share the first one's block together
+// and looks at them in order; the division by the voxel size, three per
+// sample, is three instructions (divide_by_voxel); and a warp takes 8 x 4
+// pixels, whose rays pass much the same blocks under one depth range.  Empty
+// space is passed by occupancy bits (two loads that mostly hit L1, no hash),
+// a cell of blocks at a time where it is empty: rays past a sphere's edge made
+// 40-70 lookups each and set the kernel's time.  GB300, 640 x 480 rays, 2000
+// live blocks, up to 850 samples per ray: 164 us -> 117 (tiles, division,
+// samples together) -> 73 (occupancy); 2, 3, 6 samples at once 75, 75, 83.
+//
+// x / b correctly rounded from y = 1 / b correctly rounded (Markstein, IBM J.
+// Res. Dev. 34, 1990): q = x y is within an ulp of the quotient, the remainder
+// x - b q is exact in one fused multiply-add, and q + remainder * y rounds to
+// the quotient, unless something over- or underflows.  Here it may: only
+// floor(q + 1/2) is used, which is 0 for every tiny quotient, and a quotient
+// past the range is refused whether it is huge, infinite or NaN.  y itself has
+// to be a normal number: for voxel sizes outside [2^-60, 2^60] the division is
+// made by __fdiv_rn (MUL false).
+template <bool MUL>
+__device__ __forceinline__ float divide_by_voxel(float x, float voxel, float inv_voxel) {
+  if constexpr (!MUL) return __fdiv_rn(x, voxel);
+  const float q = __fmul_rn(x, inv_voxel);
+  return __fmaf_rn(__fmaf_rn(-q, voxel, x), inv_voxel, q);
+}
+
 struct RaySample {
   int32_t g[3];
   bool in_range;
@@ -357,31 +428,33 @@ struct RaySample {
 
 // i < 2^24, so the conversion to float32 is exact (and int32 keeps it off the
 // 64-bit conversion path).
+template <bool MUL>
 __device__ __forceinline__ RaySample ray_sample(const float (&c)[3], const float (&dw)[3], float depth_min,
-                                                float step, float voxel, int32_t i) {
+                                                float step, float voxel, float inv_voxel, int32_t i) {
   RaySample r;
   r.in_range = true;
   const float t = __fadd_rn(depth_min, __fmul_rn(__int2float_rn(i), step));
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const float gf = floorf(__fadd_rn(__fdiv_rn(__fadd_rn(c[a], __fmul_rn(t, dw[a])), voxel), 0.5f));
-    r.in_range &= (gf > -1.0e9f && gf < 1.0e9f);
+    const float gf = floorf(__fadd_rn(divide_by_voxel<MUL>(__fadd_rn(c[a], __fmul_rn(t, dw[a])), voxel, inv_voxel), 0.5f));
+    r.in_range &= fabsf(gf) < 1.0e9f;
     r.g[a] = r.in_range ? static_cast<int32_t>(gf) : 0;
   }
   return r;
 }
 
-template <int ELL, int S>
+constexpr int kRaySamples = 4;
+
+template <int ELL, int S, bool MUL>
 __device__ __forceinline__ float cast_ray(const TableView& tv, const TableView& local_tv,
                                           const int32_t* __restrict__ local_values, int use_local,
                                           const float* __restrict__ tsdf, const float* __restrict__ weight,
-                                          int32_t volume_capacity, const Cam& cam, int32_t width, int64_t pid,
-                                          float voxel, float depth_min, float step, float inv_step,
+                                          const uint32_t* __restrict__ occupied,
+                                          int32_t volume_capacity, const Cam& cam, int32_t px, int32_t py,
+                                          float voxel, float inv_voxel, float depth_min, float step, float inv_step,
                                           int32_t i_begin, int32_t n_steps) {
   constexpr int kVox = ELL * ELL * ELL;
   constexpr int kShift = ELL == 8 ? 3 : 4;
-  const int32_t py = static_cast<int32_t>(pid / width);
-  const int32_t px = static_cast<int32_t>(pid - static_cast<int64_t>(py) * width);
   float c[3];
   camera_centre(cam, c);
   const float dcx = __fdiv_rn(__fsub_rn(static_cast<float>(px), cam.cx), cam.fx);
@@ -393,49 +466,43 @@ __device__ __forceinline__ float cast_ray(const TableView& tv, const TableView& 
     inv_dw[a] = __fdividef(1.0f, dw[a]);  // only for the skip estimate
   }
 
-  int32_t last[3] = {0, 0, 0};
-  int32_t last_bi = -1;
-  bool have_last = false;
+  int32_t K[3] = {0, 0, 0};
+  int32_t bi = -1;  // block K's index in the volume, -1 until a block was found
   bool prev_valid = false;
-  float prev_d = 0.0f, prev_t = 0.0f;
-  float out = 0.0f;
-  for (int32_t i = i_begin; i < n_steps; ++i) {
-    const float t = __fadd_rn(depth_min, __fmul_rn(__int2float_rn(i), step));
-    const RaySample r = ray_sample(c, dw, depth_min, step, voxel, i);
-    bool valid = false;
-    float dcur = 0.0f;
-    if (r.in_range) {
-      const int32_t K[3] = {r.g[0] >> kShift, r.g[1] >> kShift, r.g[2] >> kShift};
-      if (!have_last || K[0] != last[0] || K[1] != last[1] || K[2] != last[2]) {
-        if (use_local) {
-          const int32_t li = find_key<3, S>(local_tv, K);
-          last_bi = li >= 0 ? __ldg(local_values + li) : -1;
-        } else {
-          last_bi = find_key<3, S>(tv, K);
+  float prev_d = 0.0f;
+  int32_t i = i_begin;
+  while (true) {
+    // 1. on to the next sample in a block that exists
+    while (i < n_steps) {
+      const RaySample r = ray_sample<MUL>(c, dw, depth_min, step, voxel, inv_voxel, i);
+      if (r.in_range) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) K[a] = r.g[a] >> kShift;
+        // missing: K's cell of blocks, or only K itself
+        int shift = kShift + kOccCell;
+        uint32_t bit = cell_bit(K);
+        if ((__ldg(occupied + (bit >> 5)) >> (bit & 31)) & 1u) {
+          shift = kShift;
+          bit = fine_bit(K);
+          if ((__ldg(occupied + (bit >> 5)) >> (bit & 31)) & 1u) {
+            if (use_local) {
+              const int32_t li = find_key<3, S>(local_tv, K);
+              bi = li >= 0 ? __ldg(local_values + li) : -1;
+            } else {
+              bi = find_key<3, S>(tv, K);
+            }
+            if (bi >= 0 && bi < volume_capacity) break;
+          }
         }
-        last[0] = K[0];
-        last[1] = K[1];
-        last[2] = K[2];
-        have_last = true;
-      }
-      if (last_bi >= 0 && last_bi < volume_capacity) {
-        const int v = ((r.g[2] & (ELL - 1)) * ELL + (r.g[1] & (ELL - 1))) * ELL + (r.g[0] & (ELL - 1));
-        const int64_t at = static_cast<int64_t>(last_bi) * kVox + v;
-        const float w = __ldg(weight + at);
-        const float d = __ldg(tsdf + at);
-        if (w > 0.0f) {
-          valid = true;
-          dcur = d;
-        }
-      } else {
-        // missing block: the ray's exit from the cell of samples that map to K
+        // the ray's exit from what is missing: the lattice points [lo, lo + 2^shift) per axis
+        const float t = __fadd_rn(depth_min, __fmul_rn(__int2float_rn(i), step));
+        const float edge = static_cast<float>(1 << shift);
         float t_exit = 3.0e38f;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-          const float lo = (static_cast<float>(K[a]) * ELL - 0.5f) * voxel;
-          const float hi = (static_cast<float>(K[a]) * ELL + (ELL - 0.5f)) * voxel;
-          if (dw[a] > 0.0f) t_exit = fminf(t_exit, (hi - c[a]) * inv_dw[a]);
-          else if (dw[a] < 0.0f) t_exit = fminf(t_exit, (lo - c[a]) * inv_dw[a]);
+          const float lo = static_cast<float>((r.g[a] >> shift) << shift) - 0.5f;
+          const float face = dw[a] > 0.0f ? lo + edge : lo;
+          if (dw[a] != 0.0f) t_exit = fminf(t_exit, (face * voxel - c[a]) * inv_dw[a]);
         }
         const float est = floorf((t_exit - t) * inv_step);
         if (est >= 1.0f) {
@@ -444,78 +511,109 @@ __device__ __forceinline__ float cast_ray(const TableView& tv, const TableView& 
           // confirm with the exact sample arithmetic; one step back if the
           // estimate crossed the face
           for (int tries = 0; tries < 2 && m > i; ++tries, --m) {
-            const RaySample rm = ray_sample(c, dw, depth_min, step, voxel, m);
-            if (rm.in_range && (rm.g[0] >> kShift) == K[0] && (rm.g[1] >> kShift) == K[1] &&
-                (rm.g[2] >> kShift) == K[2]) {
-              i = m;  // samples i+1..m are in the missing block
+            const RaySample rm = ray_sample<MUL>(c, dw, depth_min, step, voxel, inv_voxel, m);
+            if (rm.in_range && (rm.g[0] >> shift) == (r.g[0] >> shift) && (rm.g[1] >> shift) == (r.g[1] >> shift) &&
+                (rm.g[2] >> shift) == (r.g[2] >> shift)) {
+              i = m;  // samples i+1..m are in the missing part
               break;
             }
           }
         }
       }
+      prev_valid = false;
+      ++i;
     }
-    if (valid && prev_valid && prev_d > 0.0f && dcur <= 0.0f) {
-      out = __fadd_rn(prev_t, __fmul_rn(step, __fdiv_rn(prev_d, __fsub_rn(prev_d, dcur))));
-      break;
+    if (i >= n_steps) return 0.0f;
+    // 2. its samples in that block, kRaySamples at a time
+    const float* w_row = weight + static_cast<int64_t>(bi) * kVox;
+    const float* d_row = tsdf + static_cast<int64_t>(bi) * kVox;
+    int m = kRaySamples;
+    while (m == kRaySamples) {
+      int at[kRaySamples];
+      m = 0;
+#pragma unroll
+      for (int q = 0; q < kRaySamples; ++q) {
+        const RaySample r = ray_sample<MUL>(c, dw, depth_min, step, voxel, inv_voxel, i + q);
+        at[q] = ((r.g[2] & (ELL - 1)) * ELL + (r.g[1] & (ELL - 1))) * ELL + (r.g[0] & (ELL - 1));
+        const bool same = i + q < n_steps && r.in_range && (r.g[0] >> kShift) == K[0] && (r.g[1] >> kShift) == K[1] &&
+                          (r.g[2] >> kShift) == K[2];
+        if (same && m == q) m = q + 1;
+      }
+      float w[kRaySamples], d[kRaySamples];
+#pragma unroll
+      for (int q = 0; q < kRaySamples; ++q) {
+        w[q] = q < m ? __ldg(w_row + at[q]) : 0.0f;
+        d[q] = q < m ? __ldg(d_row + at[q]) : 0.0f;
+      }
+#pragma unroll
+      for (int q = 0; q < kRaySamples; ++q) {
+        if (q < m) {
+          const bool valid = w[q] > 0.0f;
+          if (valid && prev_valid && prev_d > 0.0f && d[q] <= 0.0f) {
+            const float prev_t = __fadd_rn(depth_min, __fmul_rn(__int2float_rn(i + q - 1), step));
+            return __fadd_rn(prev_t, __fmul_rn(step, __fdiv_rn(prev_d, __fsub_rn(prev_d, d[q]))));
+          }
+          prev_valid = valid;
+          prev_d = d[q];
+        }
+      }
+      i += m;
     }
-    prev_valid = valid;
-    prev_d = dcur;
-    prev_t = t;
   }
-  return out;
 }
 
-// Persistent grid; each warp takes the next 32 pixels from a counter, so rays
-// of uneven length do not leave the tail of the launch idle.  Each ray
-// samples only i in [i_begin, i_end) from its tile's depth range, widened by
-// two steps on either side; the sample before i_begin lies outside every
-// listed cell, so starting there with no valid predecessor is the same as
-// marching from 0.
-template <int ELL, int S>
+// Persistent grid; each warp takes the next 8 x 4 pixels (half a range tile)
+// from a counter, so rays of uneven length do not leave the tail of the
+// launch idle.  Each ray samples only i in [i_begin, i_end) from its tile's
+// depth range, widened by two steps on either side; the sample before i_begin
+// lies outside every listed cell, so starting there with no valid predecessor
+// is the same as marching from 0.
+template <int ELL, int S, bool MUL>
 __global__ void __launch_bounds__(kThreads) raycast_kernel(TableView tv, TableView local_tv,
                                                            const int32_t* __restrict__ local_values, int use_local,
                                                            const float* __restrict__ tsdf,
-                                                           const float* __restrict__ weight, int32_t volume_capacity,
-                                                           Cam cam, int32_t width, int64_t n_pixels, float voxel,
-                                                           float depth_min, float step,
+                                                           const float* __restrict__ weight,
+                                                           const uint32_t* __restrict__ occupied,
+                                                           int32_t volume_capacity,
+                                                           Cam cam, int32_t width, int32_t height, float voxel,
+                                                           float inv_voxel, float depth_min, float step,
                                                            float inv_step, int32_t n_steps,
                                                            const unsigned int* __restrict__ zmin,
                                                            const unsigned int* __restrict__ zmax, int tiles_x,
-                                                           int use_range, unsigned long long* __restrict__ next_chunk,
+                                                           int tiles_y, int use_range,
+                                                           unsigned long long* __restrict__ next_chunk,
                                                            float* __restrict__ depth_out) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int lane = threadIdx.x & 31;
-  const uint64_t n_chunks = static_cast<uint64_t>((n_pixels + 31) / 32);
+  const uint64_t n_chunks = static_cast<uint64_t>(tiles_x) * static_cast<uint64_t>(tiles_y) * 2u;
   while (true) {
     unsigned long long chunk = 0;
     if (lane == 0) chunk = atomicAdd(next_chunk, 1ull);
     chunk = __shfl_sync(0xFFFFFFFFu, chunk, 0);
     if (chunk >= n_chunks) break;
-    const int64_t pid = static_cast<int64_t>(chunk) * 32 + lane;
-    if (pid < n_pixels) {
-      const int32_t py = static_cast<int32_t>(pid / width);
-      const int32_t px = static_cast<int32_t>(pid - static_cast<int64_t>(py) * width);
-      int32_t i0 = 0, i1 = n_steps;
-      if (use_range) {
-        const int tile = (py / kRangeTile) * tiles_x + px / kRangeTile;
-        const float z0 = __uint_as_float(__ldg(zmin + tile));
-        const float z1 = __uint_as_float(__ldg(zmax + tile));
-        if (z0 <= z1) {
-          const float f0 = floorf((z0 - depth_min) * inv_step) - 2.0f;
-          const float f1 = ceilf((z1 - depth_min) * inv_step) + 2.0f;
-          i0 = f0 <= 0.0f ? 0 : (f0 >= static_cast<float>(n_steps) ? n_steps : static_cast<int32_t>(f0));
-          i1 = f1 >= static_cast<float>(n_steps) ? n_steps : (f1 <= 0.0f ? 0 : static_cast<int32_t>(f1));
-        } else {
-          i1 = 0;  // no listed block over this tile
-        }
+    const uint32_t tile = static_cast<uint32_t>(chunk >> 1);
+    const int32_t ty = static_cast<int32_t>(tile / static_cast<uint32_t>(tiles_x));
+    const int32_t tx = static_cast<int32_t>(tile) - ty * tiles_x;
+    const int32_t px = tx * kRangeTile + (lane & 7);
+    const int32_t py = ty * kRangeTile + static_cast<int32_t>(chunk & 1u) * 4 + (lane >> 3);
+    int32_t i0 = 0, i1 = n_steps;
+    if (use_range) {
+      const float z0 = __uint_as_float(__ldg(zmin + tile));
+      const float z1 = __uint_as_float(__ldg(zmax + tile));
+      if (z0 <= z1) {
+        const float f0 = floorf((z0 - depth_min) * inv_step) - 2.0f;
+        const float f1 = ceilf((z1 - depth_min) * inv_step) + 2.0f;
+        i0 = f0 <= 0.0f ? 0 : (f0 >= static_cast<float>(n_steps) ? n_steps : static_cast<int32_t>(f0));
+        i1 = f1 >= static_cast<float>(n_steps) ? n_steps : (f1 <= 0.0f ? 0 : static_cast<int32_t>(f1));
+      } else {
+        i1 = 0;  // no listed block over this tile
       }
-      float out = 0.0f;
-      {
-        if (i0 < i1)
-          out = cast_ray<ELL, S>(tv, local_tv, local_values, use_local, tsdf, weight, volume_capacity, cam, width, pid,
-                                 voxel, depth_min, step, inv_step, i0, i1);
-      }
-      depth_out[pid] = out;
     }
+    if (px < width && py < height)
+      depth_out[static_cast<int64_t>(py) * width + px] =
+          cast_ray<ELL, S, MUL>(tv, local_tv, local_values, use_local, tsdf, weight, occupied, volume_capacity, cam, px, py, voxel,
+                           inv_voxel, depth_min, step, inv_step, i0, i1);
+    __syncwarp();
   }
 }
 
@@ -748,40 +846,52 @@ ash_status ash_tsdf_raycast(ash_map* blocks, int tsdf_buffer, int weight_buffer,
   const int32_t cap = static_cast<int32_t>(blocks->capacity);
   const int use_local = local_index_map ? 1 : 0;
   const float inv_step = 1.0f / step;
-  // scratch: chunk counter | live count | tile zmin | tile zmax | live indices
+  // Markstein's division needs a normal reciprocal (divide_by_voxel)
+  const bool mul = voxel_size >= 0x1p-60f && voxel_size <= 0x1p60f;
+  const float inv_voxel = mul ? 1.0f / voxel_size : 0.0f;
+  // scratch: chunk counter | live count | occupancy bits | tile zmin | tile
+  // zmax | live indices (only listed when the live blocks are not simply rows
+  // 0..t-1)
   ash_map* lookup = local_index_map ? local_index_map : blocks;
   const int tiles_x = (width + ash::vol::kRangeTile - 1) / ash::vol::kRangeTile;
   const int tiles_y = (height + ash::vol::kRangeTile - 1) / ash::vol::kRangeTile;
   const int n_tiles = tiles_x * tiles_y;
-  const size_t off_tiles = 16, off_live = off_tiles + ((8 * static_cast<size_t>(n_tiles) + 15) / 16) * 16;
-  char* scratch = static_cast<char*>(ash::vol::scratch_alloc(off_live + 4 * static_cast<size_t>(lookup->capacity), st));
+  const bool listed = !lookup->heap_identity;
+  lookup->last_stream = st;
+  const size_t off_tiles = 16 + 4 * static_cast<size_t>(ash::vol::kOccWords), off_live = off_tiles + ((8 * static_cast<size_t>(n_tiles) + 15) / 16) * 16;
+  char* scratch = static_cast<char*>(
+      ash::vol::scratch_alloc(off_live + (listed ? 4 * static_cast<size_t>(lookup->capacity) : 0), st));
   if (!scratch) return fail(ASH_ERR_OOM, "scratch allocation failed");
   unsigned long long* counter = reinterpret_cast<unsigned long long*>(scratch);
   int64_t* live_count = reinterpret_cast<int64_t*>(scratch + 8);
+  uint32_t* occupied = reinterpret_cast<uint32_t*>(scratch + 16);
   unsigned int* zmin = reinterpret_cast<unsigned int*>(scratch + off_tiles);
   unsigned int* zmax = zmin + n_tiles;
-  int32_t* live = reinterpret_cast<int32_t*>(scratch + off_live);
-  cudaMemsetAsync(counter, 0, sizeof(unsigned long long), st);
+  int32_t* live = listed ? reinterpret_cast<int32_t*>(scratch + off_live) : nullptr;
   // the per-tile depth range (Sec. 6.2's min-max estimate) needs samples at t > 0
   const int use_range = depth_min > 0.0f ? 1 : 0;
-  if (use_range) {
+  if (listed) {
     ash_status ls = ash_get_active_indices_async(lookup, live, lookup->capacity, live_count, stream);
     if (ls != ASH_OK) {
       cudaFreeAsync(scratch, st);
       return ls;
     }
+  }
+  {
     ash::TraceScope tr(ash::kKRayRange, st, 2);
-    ash::vol::range_reset_kernel<<<(n_tiles + 255) / 256, 256, 0, st>>>(zmin, zmax, n_tiles);
-    ash::vol::block_range_kernel<<<grid_for(lookup->capacity, launch_of(lookup, st)), ash::vol::kThreads, 0, st>>>(
-        lookup->kb, lookup->ks, ell, live, lookup->capacity, live_count, cam, voxel_size, width, height, tiles_x,
-        tiles_y, zmin, zmax);
+    ash::launch_dependent(ash::vol::range_reset_kernel, 65, 256, st, zmin, zmax, use_range ? n_tiles : 0, occupied,
+                          counter);
+    ash::launch_dependent(ash::vol::block_range_kernel, grid_for(lookup->capacity * 32, launch_of(lookup, st)),
+                          ash::vol::kThreads, st, lookup->kb, lookup->ks, ell, lookup->ctrl, live, lookup->capacity,
+                          live_count, cam, voxel_size, width, height, tiles_x, tiles_y, use_range ? zmin : nullptr,
+                          zmax, occupied);
   }
   int dev = 0;
   cudaGetDevice(&dev);
-  const int64_t warps_needed = (n_pix + 31) / 32;
+  const int64_t warps_needed = static_cast<int64_t>(n_tiles) * 2;
   // one wave of resident blocks (all variants use about the same registers)
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ash::vol::raycast_kernel<8, 4>, ash::vol::kThreads, 0) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ash::vol::raycast_kernel<8, 4, true>, ash::vol::kThreads, 0) !=
           cudaSuccess ||
       per_sm < 1) {
     cudaGetLastError();
@@ -791,21 +901,24 @@ ash_status ash_tsdf_raycast(ash_map* blocks, int tsdf_buffer, int weight_buffer,
   if (grid64 * (ash::vol::kThreads / 32) > warps_needed) grid64 = (warps_needed + 7) / 8;
   const unsigned grid = static_cast<unsigned>(grid64 < 1 ? 1 : grid64);
   ash::TraceScope ts(ash::kKRaycast, st);
-#define ASH_RAYCAST(E, SB)                                                                                          \
-  ash::vol::raycast_kernel<E, SB><<<grid, ash::vol::kThreads, 0, st>>>(tv, ltv, lvals, use_local, tsdf, weight, cap, \
-                                                                       cam, width, n_pix, voxel_size, depth_min,     \
-                                                                       step, inv_step,                               \
-                                                                       static_cast<int32_t>(n_steps), zmin, zmax,   \
-                                                                       tiles_x, use_range, counter, depth_out)
+#define ASH_RAYCAST_M(E, SB, M)                                                                                     \
+  ash::launch_dependent(ash::vol::raycast_kernel<E, SB, M>, static_cast<int>(grid), ash::vol::kThreads, st, tv, ltv, \
+                        lvals, use_local, tsdf, weight, occupied, cap, cam, width, height, voxel_size, inv_voxel,    \
+                        depth_min, step, inv_step, static_cast<int32_t>(n_steps), zmin, zmax, tiles_x, tiles_y,      \
+                        use_range, counter, depth_out)
+#define ASH_RAYCAST(E, SB)           \
+  if (mul) ASH_RAYCAST_M(E, SB, true); \
+  else ASH_RAYCAST_M(E, SB, false)
   if (ell == 8) {
-    if (blocks->S == 4) ASH_RAYCAST(8, 4);
-    else if (blocks->S == 8) ASH_RAYCAST(8, 8);
-    else ASH_RAYCAST(8, 16);
+    if (blocks->S == 4) { ASH_RAYCAST(8, 4); }
+    else if (blocks->S == 8) { ASH_RAYCAST(8, 8); }
+    else { ASH_RAYCAST(8, 16); }
   } else {
-    if (blocks->S == 4) ASH_RAYCAST(16, 4);
-    else if (blocks->S == 8) ASH_RAYCAST(16, 8);
-    else ASH_RAYCAST(16, 16);
+    if (blocks->S == 4) { ASH_RAYCAST(16, 4); }
+    else if (blocks->S == 8) { ASH_RAYCAST(16, 8); }
+    else { ASH_RAYCAST(16, 16); }
   }
+#undef ASH_RAYCAST_M
 #undef ASH_RAYCAST
   const ash_status s = check_launch("tsdf_raycast");
   cudaFreeAsync(scratch, st);
