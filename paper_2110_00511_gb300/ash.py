@@ -13,6 +13,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 
 import torch
 
@@ -95,6 +96,10 @@ class BatchOp(ctypes.Structure):
     _fields_ = [("map", ctypes.c_void_p), ("op", ctypes.c_int32), ("pad", ctypes.c_int32),
                 ("keys", ctypes.c_void_p), ("values", ctypes.c_void_p), ("n", ctypes.c_int64),
                 ("buf_indices", ctypes.c_void_p), ("masks", ctypes.c_void_p)]
+
+
+# A BatchOp's fields for struct.pack_into (cheaper than a ctypes object each).
+_BATCH_OP = struct.Struct("=QiiQQqQQ")
 
 # C signatures: name -> (restype, argtypes)
 _SIGS = {
@@ -195,32 +200,41 @@ def _check(status):
         raise AshError(status, lib().ash_last_error().decode())
 
 
-def _stream(device=None):
-    return ctypes.c_void_p(torch.cuda.current_stream(device).cuda_stream)
-
-
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream_of(device_index):
-    """The current CUDA stream of a device as an integer handle (the fast
-    route of the map methods; same stream as _stream)."""
+    """The current CUDA stream of a device as an integer handle."""
     if _raw_stream is not None:
         return _raw_stream(device_index)
     return torch.cuda.current_stream(device_index).cuda_stream
 
 
+def _stream(device=None):
+    """The same for a torch.device, an index or None (the current device)."""
+    index = device if isinstance(device, int) else getattr(device, "index", None)
+    return _stream_of(torch.cuda.current_device() if index is None else index)
+
+
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else ctypes.c_void_p(0)
+    """A tensor's address as the integer that ctypes passes for a pointer."""
+    return t.data_ptr() if t is not None else None
 
 
 def _need_cuda(t, name, dtype=None):
     if not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor")
-    if dtype is not None and t.dtype != dtype:
+    if dtype is not None and t.dtype is not dtype:
         raise ValueError(f"{name} must be {dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
+
+
+def _index_rows(indices):
+    """Buffer indices as contiguous int32."""
+    if indices.dtype is torch.int32 and indices.is_contiguous():
+        return indices
+    return indices.to(torch.int32).contiguous()
 
 
 class _DeviceArray:
@@ -473,7 +487,9 @@ class Batch:
             self._h = None
 
     def run(self, items, outputs=None):
-        ops, outs = [], []
+        outs = []
+        buf = bytearray(_BATCH_OP.size * max(1, len(items)))
+        at = 0
         for j, (hm, op, keys, values) in enumerate(items):
             n = keys.shape[0]
             if outputs is not None:
@@ -481,10 +497,13 @@ class Batch:
             else:
                 idx = torch.empty(n, dtype=torch.int32, device=keys.device) if op != ASH_OP_ERASE else None
                 mask = torch.empty(n, dtype=torch.bool, device=keys.device)
-            ops.append(BatchOp(hm.handle.value, op, 0, keys.data_ptr(), values.data_ptr() if values is not None else None,
-                               n, idx.data_ptr() if idx is not None else None, mask.data_ptr()))
+            _BATCH_OP.pack_into(buf, at, hm._h.value, op, 0, keys.data_ptr(),
+                                values.data_ptr() if values is not None else 0, n,
+                                idx.data_ptr() if idx is not None else 0, mask.data_ptr())
+            at += _BATCH_OP.size
             outs.append((idx, mask))
-        ash_batch_run(self._h, ops)
+        arr = (BatchOp * max(1, len(items))).from_buffer(buf)
+        _check(lib().ash_batch_run(self._h, arr, len(items), _stream()))
         return outs
 
 
@@ -619,7 +638,7 @@ class HashMap:
         self.value_dtypes = list(value_dtypes)
         numel = [int(torch.Size(s).numel()) for s in self.value_shapes]
         self._h = ash_create(self.key_dim, capacity, numel, self.value_dtypes, self.device.index, tuning,
-                             _stream(self.device))
+                             _stream_of(self.device.index))
 
     @classmethod
     def wrap(cls, handle, key_dim, value_shapes=(), value_dtypes=(), device=0):
@@ -728,18 +747,18 @@ class HashMap:
         no host synchronisation; indices[:count] are the live entries."""
         out = torch.empty(max(1, self.capacity()), dtype=torch.int32, device=self.device)
         count = torch.empty(1, dtype=torch.int64, device=self.device)
-        _check(lib().ash_get_active_indices_async(self._h, _ptr(out), out.numel(), _ptr(count), _stream(self.device)))
+        _check(lib().ash_get_active_indices_async(self._h, _ptr(out), out.numel(), _ptr(count), _stream_of(self.device.index)))
         return out, count
 
     def gather_keys_count(self, indices, count):
         """[len(indices), key_dim] key rows; only the first *count (device) rows are written."""
         out = torch.empty((indices.numel(), self.key_dim), dtype=torch.int32, device=self.device)
         _check(lib().ash_gather_keys_count(self._h, _ptr(indices), indices.numel(), _ptr(count), _ptr(out),
-                                           _stream(self.device)))
+                                           _stream_of(self.device.index)))
         return out
 
     def size(self):
-        return ash_size(self._h, _stream(self.device))
+        return ash_size(self._h, _stream_of(self.device.index))
 
     def capacity(self):
         return int(lib().ash_capacity(self._h))
@@ -748,34 +767,34 @@ class HashMap:
         """Table health (synchronises): capacity, table_slots, live, used_slots
         (live + tombstones), host_syncs, rebuilds."""
         st = MapStats()
-        _check(lib().ash_get_map_stats(self._h, ctypes.byref(st), _stream(self.device)))
+        _check(lib().ash_get_map_stats(self._h, ctypes.byref(st), _stream_of(self.device.index)))
         return st.as_dict()
 
     def rehash(self, new_capacity=0):
-        ash_rehash(self._h, new_capacity, _stream(self.device))
+        ash_rehash(self._h, new_capacity, _stream_of(self.device.index))
 
     def reserve(self, new_capacity):
-        ash_reserve(self._h, new_capacity, _stream(self.device))
+        ash_reserve(self._h, new_capacity, _stream_of(self.device.index))
 
     def reserve_async(self, new_capacity):
-        ash_reserve_async(self._h, new_capacity, _stream(self.device))
+        ash_reserve_async(self._h, new_capacity, _stream_of(self.device.index))
 
     def clear(self):
-        ash_clear(self._h, _stream(self.device))
+        ash_clear(self._h, _stream_of(self.device.index))
 
     def sync_status(self):
-        ash_sync_status(self._h, _stream(self.device))
+        ash_sync_status(self._h, _stream_of(self.device.index))
 
     def gather_keys(self, indices):
         out = torch.empty((indices.numel(), self.key_dim), dtype=torch.int32, device=self.device)
-        ash_gather_keys(self._h, indices.to(torch.int32).contiguous(), out)
+        ash_gather_keys(self._h, _index_rows(indices), out)
         return out
 
     def gather_values(self, indices, j=0):
         """[n, *shape_j] rows of value buffer j at `indices` (zeros outside [0, c))."""
-        idx = indices.to(torch.int32).contiguous()
+        idx = _index_rows(indices)
         out = torch.empty((idx.numel(), *self.value_shapes[j]), dtype=self.value_dtypes[j], device=self.device)
-        _check(lib().ash_gather_values(self._h, j, _ptr(idx), idx.numel(), _ptr(out), _stream(self.device)))
+        _check(lib().ash_gather_values(self._h, j, _ptr(idx), idx.numel(), _ptr(out), _stream_of(self.device.index)))
         return out
 
     def _points(self, points):
@@ -795,21 +814,21 @@ class HashMap:
         idx, mask = self._outputs(points.shape[0])
         arr = (ctypes.c_void_p * max(1, len(values)))(*[v.data_ptr() for v in values])
         _check(lib().ash_insert_points(self._h, _ptr(points), ctypes.c_float(cell), arr, points.shape[0], _ptr(idx),
-                                       _ptr(mask), _stream(self.device)))
+                                       _ptr(mask), _stream_of(self.device.index)))
         return idx, mask
 
     def activate_points(self, points, cell):
         points = self._points(points)
         idx, mask = self._outputs(points.shape[0])
         _check(lib().ash_activate_points(self._h, _ptr(points), ctypes.c_float(cell), points.shape[0], _ptr(idx),
-                                         _ptr(mask), _stream(self.device)))
+                                         _ptr(mask), _stream_of(self.device.index)))
         return idx, mask
 
     def find_points(self, points, cell):
         points = self._points(points)
         idx, mask = self._outputs(points.shape[0])
         _check(lib().ash_find_points(self._h, _ptr(points), ctypes.c_float(cell), points.shape[0], _ptr(idx),
-                                     _ptr(mask), _stream(self.device)))
+                                     _ptr(mask), _stream_of(self.device.index)))
         return idx, mask
 
     def find_neighbors(self, keys, radius=1):
@@ -820,7 +839,7 @@ class HashMap:
         idx = torch.empty((keys.shape[0], k), dtype=torch.int32, device=self.device)
         mask = torch.empty((keys.shape[0], k), dtype=torch.bool, device=self.device)
         _check(lib().ash_find_neighbors(self._h, _ptr(keys), keys.shape[0], int(radius), _ptr(idx), _ptr(mask),
-                                        _stream(self.device)))
+                                        _stream_of(self.device.index)))
         return idx, mask
 
     def find_offsets(self, keys, offsets):
@@ -831,7 +850,7 @@ class HashMap:
         idx = torch.empty((keys.shape[0], off.shape[0]), dtype=torch.int32, device=self.device)
         mask = torch.empty((keys.shape[0], off.shape[0]), dtype=torch.bool, device=self.device)
         _check(lib().ash_find_offsets(self._h, _ptr(keys), keys.shape[0], _ptr(off), off.shape[0], _ptr(idx),
-                                      _ptr(mask), _stream(self.device)))
+                                      _ptr(mask), _stream_of(self.device.index)))
         return idx, mask
 
     def export(self):
@@ -889,10 +908,17 @@ class HashMap:
 
 
 # ------------------------------------------------------------ geometry (Sec. 6.2)
+_F4, _F12 = ctypes.c_float * 4, ctypes.c_float * 12
+
+
 def _cam_arrays(intrinsics, extrinsic):
-    intr = (ctypes.c_float * 4)(*[float(x) for x in intrinsics])
-    e = [float(x) for x in torch.as_tensor(extrinsic, dtype=torch.float32).reshape(12).tolist()]
-    return intr, (ctypes.c_float * 12)(*e)
+    """(fx, fy, cx, cy) and the 12 floats of [R | t] on the host; a float32 CPU
+    tensor in row order is passed as it lies in memory."""
+    intr = _F4(*map(float, intrinsics))
+    if (isinstance(extrinsic, torch.Tensor) and extrinsic.dtype is torch.float32 and extrinsic.device.type == "cpu"
+            and extrinsic.numel() == 12 and extrinsic.is_contiguous()):
+        return intr, extrinsic.data_ptr()
+    return intr, _F12(*torch.as_tensor(extrinsic, dtype=torch.float32).reshape(12).tolist())
 
 
 def ash_depth_to_block_keys(depth, intrinsics, extrinsic, block_edge, depth_max, keys=None, count_dev=None,
@@ -934,7 +960,7 @@ def ash_tsdf_integrate(blocks, block_indices, depth, intrinsics, extrinsic, voxe
     """TSDF integration of one frame (Sec. 6.2, Eq. (7)-(9)) into the blocks at
     block_indices (int32 device tensor of buffer indices)."""
     _need_cuda(depth, "depth", torch.float32)
-    bi = block_indices.to(torch.int32).contiguous()
+    bi = _index_rows(block_indices)
     intr, extr = _cam_arrays(intrinsics, extrinsic)
     h, w = depth.shape
     _check(lib().ash_tsdf_integrate(blocks.handle, tsdf_buffer, weight_buffer, _ptr(bi), bi.numel(), _ptr(depth), w,
