@@ -1253,7 +1253,7 @@ def sweep_figures(args, device, hbm_peak):
     rate for the random sectors, the copy peak the rate for the streamed bytes (see
     random_access_fraction).
 
-    Points whose table is larger than twice L2 (2^20 keys or more) run, by
+    Points whose table is larger than 1.5 times L2 (2^20 keys or more) run, by
     default, with the keys in home-bucket range order (tuning
     partition_keys): their random accesses are then local to one range at a
     time, so the random-access roofline no longer bounds them.  Those points
@@ -1310,7 +1310,7 @@ def sweep_figures(args, device, hbm_peak):
         small = small_call_figures(keys, queries, n, device, flush) if n <= 100_000 else None
         t = hm.tuning()
         slots = int(n * t.slots_per_capacity)
-        ranged = slots * 8 > 2 * l2 and n >= (1 << 20)
+        ranged = 2 * slots * 8 > 3 * l2 and n >= (1 << 20)
         input_order = None
         if ranged:
             t1 = ash.default_tuning()

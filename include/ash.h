@@ -112,13 +112,12 @@ typedef struct ash_tuning {
                                  1 = use the keys in input order; 2 = first put them in the order
                                  of their home buckets' ranges (a stable partition into ranges of
                                  about L2/2 bytes of table each, 8 ranges at least) and work range
-                                 by range, each range's table buckets prefetched into L2 before its
-                                 keys, so that the kernels find the table (and kB) in L2 instead of
-                                 missing at random; the outputs come back in input order, and equal
+                                 by range, so that the kernels find most of the table (and kB) in L2
+                                 instead of missing at random; the outputs come back in input order, and equal
                                  keys keep their input order (the first occurrence still wins);
-                                 0 = 2 for calls of at least 2^20 keys on a table larger than twice
-                                 L2, else 1 (a ranged find reads kB in range order only when the
-                                 inserts were ranged too, so both switch together).  Takes about
+                                 0 = 2 for calls of at least 2^20 keys on a table larger than 1.5
+                                 times L2, else 1 (a ranged find gains most when the inserts were
+                                 ranged too: it then reads kB in range order).  Takes about
                                  9 + 4d bytes of stream-ordered scratch per key during the call;
                                  if that cannot be had the call uses input order */
 } ash_tuning;

@@ -52,9 +52,6 @@ struct InitPlan {
   void word(void* dst, uint64_t v) { add(kWord, dst, nullptr, v, 8); }
 };
 void launch_init(const InitPlan& plan, const Launch& L);
-// L2 prefetch of a byte range (a hint; plain stream order, no programmatic
-// overlap, so it never runs beside the kernel before it).
-void launch_prefetch_l2(const void* base, int64_t bytes, const Launch& L);
 // Publishes the control block to a host-visible snapshot (publish_snapshot).
 void launch_snapshot(Ctrl* ctrl, Snap* snap, uint32_t seq, const Launch& L);
 // Value rows of an insert's winners (idx[p] >= 0): dst_j row idx[p] <- src_j row p.

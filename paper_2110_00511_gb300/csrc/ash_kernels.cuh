@@ -1047,29 +1047,39 @@ __global__ void __launch_bounds__(256) commit_kernel(TableView t, const In keys,
 // keys.  A count pass histograms each block's span per range (counts[P][G]);
 // a scan turns each range's row into the blocks' offsets within the range
 // (and the range totals); the scatter pass sorts each tile by range in
-// shared memory (stable: warp w holds tile positions [256 w, 256 w + 256) in
+// shared memory (stable: each warp holds consecutive tile positions in
 // steps of 32, ranked by __match_any_sync) and writes each range's part of
 // the tile as one run after the block's previous tiles' runs.  dest[pos]
 // records where input row pos went, for the outputs' way back.
-constexpr int kPartTile = 2048;     // keys per tile: 256 threads x 8
-constexpr int kPartSteps = kPartTile / 256;
+//
+// The scatter is bound by instruction issue and by its tiles' barriers, not by
+// HBM (10^8 rows of 12 bytes: 894 -> 683 us, 4.1 TB/s).  What brought it
+// there: the count pass hands over each key's range in a byte (752 -> 683,
+// count 215 -> 229), up to 32 ranges are scanned by one warp (806 -> 765),
+// dest is written by the thread that holds the row, in input order, and the
+// counts take shared memory for P ranges only (894 -> 806 together).  Sorted
+// rows leave row by row (word by word, so that stores coalesce, 765 against
+// 752).  512 or 1024 threads per tile: 974 and 1420 us; tiles of 1024 or 4096
+// keys: 798 and 777; 3, 5 or 6 blocks per SM: 714, 785, 920.
+constexpr int kPartTile = 2048;     // keys per tile
+constexpr int kCountThreads = 256;
+constexpr int kScatterThreads = 256;
+constexpr int kPartBlocksPerSm = 4;
 constexpr int kPartMaxLog = 8;      // at most 256 ranges
 constexpr uint32_t kNoRange = 0xFFFFFFFFu;
 
 __device__ __forceinline__ uint32_t key_range(uint64_t h, int log_p) { return hi32(h) >> (32 - log_p); }
 
-// The kPartSteps key rows of one lane in warp w's part of a tile (local
-// positions 256 w + 32 j + lane); zeros past the tile.
-template <int D>
+// The STEPS key rows of one lane in warp w's part of a tile (local positions
+// 32 (STEPS w + j) + lane); zeros past the tile.
+template <int D, int STEPS>
 __device__ __forceinline__ void load_tile_rows(const int32_t* __restrict__ keys, int64_t base, int tn,
-                                               int32_t (&k)[kPartSteps][D]) {
-  const int w = threadIdx.x >> 5;
-  const int lane = threadIdx.x & 31;
+                                               int32_t (&k)[STEPS][D]) {
+  const int first = (threadIdx.x >> 5) * 32 * STEPS + (threadIdx.x & 31);
 #pragma unroll
-  for (int j = 0; j < kPartSteps; ++j) {
-    const int local = w * 256 + j * 32 + lane;
-    if (local < tn) {
-      load_input_key<D>(keys, base + local, k[j]);
+  for (int j = 0; j < STEPS; ++j) {
+    if (first + j * 32 < tn) {
+      load_input_key<D>(keys, base + first + j * 32, k[j]);
     } else {
 #pragma unroll
       for (int c = 0; c < D; ++c) k[j][c] = 0;
@@ -1078,14 +1088,12 @@ __device__ __forceinline__ void load_tile_rows(const int32_t* __restrict__ keys,
 }
 
 // Their ranges (kNoRange past the tile).
-template <int D>
-__device__ __forceinline__ void tile_ranges(const int32_t (&k)[kPartSteps][D], int tn, int log_p,
-                                            uint32_t (&r)[kPartSteps]) {
-  const int w = threadIdx.x >> 5;
-  const int lane = threadIdx.x & 31;
+template <int D, int STEPS>
+__device__ __forceinline__ void tile_ranges(const int32_t (&k)[STEPS][D], int tn, int log_p, uint32_t (&r)[STEPS]) {
+  const int first = (threadIdx.x >> 5) * 32 * STEPS + (threadIdx.x & 31);
 #pragma unroll
-  for (int j = 0; j < kPartSteps; ++j)
-    r[j] = w * 256 + j * 32 + lane < tn ? key_range(hash_key<D>(k[j]), log_p) : kNoRange;
+  for (int j = 0; j < STEPS; ++j)
+    r[j] = first + j * 32 < tn ? key_range(hash_key<D>(k[j]), log_p) : kNoRange;
 }
 
 // Keys in tile at `base` of a span ending at t1.
@@ -1093,10 +1101,12 @@ __device__ __forceinline__ int tile_keys(int64_t base, int64_t t1) {
   return t1 - base < kPartTile ? static_cast<int>(t1 - base) : kPartTile;
 }
 
-// counts[p * G + b]: keys of range p in block b's span.
+// counts[p * G + b]: keys of range p in block b's span; ranges[pos]: the range
+// of each key, so that the scatter need not hash again.
 template <int D>
-__global__ void __launch_bounds__(256) partition_count_kernel(const int32_t* __restrict__ keys, int64_t n, int log_p,
-                                                              int tiles_per_block, uint32_t* __restrict__ counts) {
+__global__ void __launch_bounds__(kCountThreads) partition_count_kernel(const int32_t* __restrict__ keys, int64_t n, int log_p,
+                                                              int tiles_per_block, uint32_t* __restrict__ counts,
+                                                              uint8_t* __restrict__ ranges) {
   __shared__ uint32_t s_hist[1 << kPartMaxLog];
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int P = 1 << log_p;
@@ -1107,43 +1117,47 @@ __global__ void __launch_bounds__(256) partition_count_kernel(const int32_t* __r
                          ? t0 + static_cast<int64_t>(tiles_per_block) * kPartTile
                          : n;
   // each tile's rows are loaded while the tile before is being counted
-  int32_t k[kPartSteps][D];
-  if (t0 < t1) load_tile_rows<D>(keys, t0, tile_keys(t0, t1), k);
+  constexpr int kSteps = kPartTile / kCountThreads;
+  int32_t k[kSteps][D];
+  if (t0 < t1) load_tile_rows<D, kSteps>(keys, t0, tile_keys(t0, t1), k);
   for (int64_t base = t0; base < t1; base += kPartTile) {
     const int tn = tile_keys(base, t1);
-    uint32_t r[kPartSteps];
-    tile_ranges<D>(k, tn, log_p, r);
-    if (base + kPartTile < t1) load_tile_rows<D>(keys, base + kPartTile, tile_keys(base + kPartTile, t1), k);
+    uint32_t r[kSteps];
+    tile_ranges<D, kSteps>(k, tn, log_p, r);
+    if (base + kPartTile < t1) load_tile_rows<D, kSteps>(keys, base + kPartTile, tile_keys(base + kPartTile, t1), k);
 #pragma unroll
-    for (int j = 0; j < kPartSteps; ++j)
-      if (r[j] != kNoRange) atomicAdd(&s_hist[r[j]], 1u);
+    for (int j = 0; j < kSteps; ++j) {
+      if (r[j] != kNoRange) {
+        atomicAdd(&s_hist[r[j]], 1u);
+        ranges[base + ((threadIdx.x >> 5) * kSteps + j) * 32 + (threadIdx.x & 31)] = static_cast<uint8_t>(r[j]);
+      }
+    }
   }
   __syncthreads();
   for (int p = threadIdx.x; p < P; p += blockDim.x) counts[static_cast<int64_t>(p) * gridDim.x + blockIdx.x] = s_hist[p];
 }
 
-// Dynamic shared memory of the scatter kernel: the tile's key rows.
+// Dynamic shared memory of the scatter kernel: the tile's key rows, their
+// places, and each warp's counts per range.
 template <int D>
-constexpr size_t partition_scatter_smem() {
-  return sizeof(int32_t) * kPartTile * D;
+constexpr size_t partition_scatter_smem(int P) {
+  return sizeof(int32_t) * (kPartTile * (D + 1) + kScatterThreads / 32 * P);
 }
 
 // row_offsets: counts after the scan (block b's first place within range p);
 // range_totals: keys per range.
 template <int D>
-__global__ void __launch_bounds__(256) partition_scatter_kernel(const int32_t* __restrict__ keys, int64_t n, int log_p,
-                                                                int tiles_per_block,
-                                                                const uint32_t* __restrict__ row_offsets,
-                                                                const uint32_t* __restrict__ range_totals,
-                                                                int32_t* __restrict__ keys_out,
-                                                                int32_t* __restrict__ dest) {
-  extern __shared__ int32_t s_keys[];  // [kPartTile][D], the tile in range order
+__global__ void __launch_bounds__(kScatterThreads) partition_scatter_kernel(
+    const int32_t* __restrict__ keys, const uint8_t* __restrict__ ranges, int64_t n, int log_p, int tiles_per_block,
+    const uint32_t* __restrict__ row_offsets, const uint32_t* __restrict__ range_totals,
+    int32_t* __restrict__ keys_out, int32_t* __restrict__ dest) {
+  constexpr int kWarps = kScatterThreads / 32;
+  constexpr int kSteps = kPartTile / kScatterThreads;
+  extern __shared__ int32_t s_keys[];             // [kPartTile][D], the tile in range order
+  uint32_t* s_to = reinterpret_cast<uint32_t*>(s_keys) + kPartTile * D;  // place in keys_out of each of its rows
+  uint32_t* s_cnt = s_to + kPartTile;             // [kWarps][P]: keys of each range, then the warp's offset in it
   __shared__ uint32_t s_run[1 << kPartMaxLog];    // next place of each range for this block
   __shared__ uint32_t s_start[1 << kPartMaxLog];  // first tile slot of each range
-  __shared__ uint32_t s_tcnt[1 << kPartMaxLog];   // the tile's keys of each range
-  __shared__ uint32_t s_cnt[8][1 << kPartMaxLog]; // per warp: keys of each range, then its offset in the range
-  __shared__ uint16_t s_pos[kPartTile];           // tile position of each slot
-  __shared__ uint8_t s_r[kPartTile];              // range of each slot
   __shared__ int s_warp[33];
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int P = 1 << log_p;
@@ -1151,6 +1165,7 @@ __global__ void __launch_bounds__(256) partition_scatter_kernel(const int32_t* _
   const int w = tid >> 5;
   const int lane = tid & 31;
   const unsigned lt = (1u << lane) - 1u;
+  uint32_t* mine = s_cnt + w * P;
   {
     int unused;
     const uint32_t tot = tid < P ? range_totals[tid] : 0u;
@@ -1164,60 +1179,75 @@ __global__ void __launch_bounds__(256) partition_scatter_kernel(const int32_t* _
                          : n;
   for (int64_t base = t0; base < t1; base += kPartTile) {
     const int tn = tile_keys(base, t1);
-    for (int p = lane; p < P; p += 32) s_cnt[w][p] = 0u;
+    for (int p = lane; p < P; p += 32) mine[p] = 0u;
     __syncwarp();
-    int32_t k[kPartSteps][D];
-    uint32_t r[kPartSteps];
-    load_tile_rows<D>(keys, base, tn, k);
-    tile_ranges<D>(k, tn, log_p, r);
-    uint32_t rank[kPartSteps];
+    int32_t k[kSteps][D];
+    uint32_t r[kSteps];
 #pragma unroll
-    for (int j = 0; j < kPartSteps; ++j) {
+    for (int j = 0; j < kSteps; ++j) {
+      const int local = (w * kSteps + j) * 32 + lane;
+      r[j] = local < tn ? __ldg(ranges + base + local) : kNoRange;
+    }
+    load_tile_rows<D, kSteps>(keys, base, tn, k);
+    uint32_t rank[kSteps];
+#pragma unroll
+    for (int j = 0; j < kSteps; ++j) {
       const bool valid = r[j] != kNoRange;
       const unsigned peers = __match_any_sync(0xFFFFFFFFu, r[j]);
-      const uint32_t c = valid ? s_cnt[w][r[j]] : 0u;
+      const uint32_t c = valid ? mine[r[j]] : 0u;
       rank[j] = c + __popc(peers & lt);
       __syncwarp();
-      if (valid && lane == __ffs(peers) - 1) s_cnt[w][r[j]] = c + __popc(peers);
+      if (valid && lane == __ffs(peers) - 1) mine[r[j]] = c + __popc(peers);
       __syncwarp();
     }
     __syncthreads();
-    uint32_t tc = 0;
+    // per range: the warps' counts to their offsets within it, then the
+    // ranges' first slots; up to 32 ranges are one warp's work, with no
+    // barrier in it
+    uint32_t tc = 0;  // the tile's keys of range tid
     if (tid < P) {
-      for (int ww = 0; ww < 8; ++ww) {
-        const uint32_t c = s_cnt[ww][tid];
-        s_cnt[ww][tid] = tc;
+#pragma unroll
+      for (int ww = 0; ww < kWarps; ++ww) {
+        const uint32_t c = s_cnt[ww * P + tid];
+        s_cnt[ww * P + tid] = tc;
         tc += c;
       }
     }
-    int tile_total;
-    const uint32_t st = static_cast<uint32_t>(block_exclusive_scan(static_cast<int>(tc), tile_total, s_warp));
-    if (tid < P) {
-      s_start[tid] = st;
-      s_tcnt[tid] = tc;
+    if (P <= 32) {
+      if (w == 0) {
+        uint32_t x = tc;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+          if (lane >= o) x += y;
+        }
+        s_start[lane] = x - tc;
+      }
+    } else {
+      int tile_total;
+      const uint32_t st = static_cast<uint32_t>(block_exclusive_scan(static_cast<int>(tc), tile_total, s_warp));
+      if (tid < P) s_start[tid] = st;
     }
     __syncthreads();
 #pragma unroll
-    for (int j = 0; j < kPartSteps; ++j) {
+    for (int j = 0; j < kSteps; ++j) {
       if (r[j] != kNoRange) {
-        const uint32_t slot = s_start[r[j]] + s_cnt[w][r[j]] + rank[j];
+        const uint32_t off = mine[r[j]] + rank[j];
+        const uint32_t slot = s_start[r[j]] + off;
+        const uint32_t to = s_run[r[j]] + off;
 #pragma unroll
         for (int c = 0; c < D; ++c) s_keys[slot * D + c] = k[j][c];
-        s_pos[slot] = static_cast<uint16_t>(w * 256 + j * 32 + lane);
-        s_r[slot] = static_cast<uint8_t>(r[j]);
+        s_to[slot] = to;
+        dest[base + (w * kSteps + j) * 32 + lane] = static_cast<int32_t>(to);
       }
     }
     __syncthreads();
-    for (int slot = tid; slot < tn; slot += blockDim.x) {
-      const uint32_t rr = s_r[slot];
-      const uint32_t d = s_run[rr] + (slot - s_start[rr]);
-      int32_t* row = keys_out + static_cast<int64_t>(d) * D;
+    for (int slot = tid; slot < tn; slot += kScatterThreads) {
+      int32_t* row = keys_out + static_cast<int64_t>(s_to[slot]) * D;
 #pragma unroll
       for (int c = 0; c < D; ++c) row[c] = s_keys[slot * D + c];
-      dest[base + s_pos[slot]] = static_cast<int32_t>(d);
     }
-    __syncthreads();
-    if (tid < P) s_run[tid] += s_tcnt[tid];
+    if (tid < P) s_run[tid] += tc;
     __syncthreads();
   }
 }
@@ -1505,15 +1535,15 @@ inline int grid_for(int64_t n, const Launch& L) {
 // counts counts[p][0..G) becomes its exclusive scan, the row's total goes to
 // range_totals[p].
 void launch_partition_scan(uint32_t* counts, int G, int P, uint32_t* range_totals, const Launch& L);
-// idx[pos] = idx_p[dest[pos]], mask[pos] = mask_p[dest[pos]]: a partitioned
-// call's outputs back in input order.
-void launch_unpermute(const int32_t* dest, int64_t n, const int32_t* idx_p, const uint8_t* mask_p, int32_t* idx,
-                      uint8_t* mask, const Launch& L);
+// idx[pos] = idx_p[dest[pos]], mask[pos] = idx[pos] >= 0: a partitioned call's
+// outputs back in input order.
+void launch_unpermute(const int32_t* dest, int64_t n, const int32_t* idx_p, int32_t* idx, uint8_t* mask,
+                      const Launch& L);
 
 // Blocks of a partition pass over n keys (G) and whole tiles per block.
 inline int partition_grid(int64_t n, const Launch& L, int* tiles_per_block) {
   const int64_t tiles = (n + kPartTile - 1) / kPartTile;
-  const int64_t cap = L.sms > 0 ? static_cast<int64_t>(L.sms) * 4 : 512;
+  const int64_t cap = L.sms > 0 ? static_cast<int64_t>(L.sms) * kPartBlocksPerSm : 512;
   const int64_t g0 = tiles < cap ? tiles : cap;
   const int64_t tpb = (tiles + g0 - 1) / g0;
   *tiles_per_block = static_cast<int>(tpb);
@@ -1543,7 +1573,7 @@ struct DimKernels {
                   const Launch&);
   void (*find_group)(int S, const TableView&, const int32_t*, int64_t, int32_t*, uint8_t*, const Launch&);
   // stable partition of n key rows by home-bucket range (scratch: see partition_bytes)
-  void (*partition)(const int32_t*, int64_t, int, uint32_t*, int32_t*, int32_t*, const Launch&);
+  void (*partition)(const int32_t*, int64_t, int, uint32_t*, uint8_t*, int32_t*, int32_t*, const Launch&);
   // the same operations on float32 points quantised in the kernels
   void (*find_pts)(int S, int kpt, const TableView&, const PointRows&, int64_t, int32_t*, uint8_t*, const Launch&);
   void (*claim_pts)(int S, int kpt, int pref, const TableView&, const PointRows&, int64_t, int32_t*, const Launch&);
@@ -1714,24 +1744,25 @@ struct DimLaunchers {
     else if (S == 8) find_group_s<8>(t, keys, n, idx, mask, L);
     else find_group_s<16>(t, keys, n, idx, mask, L);
   }
-  // counts: partition_count_words(n, log_p, L) words; keys_out: n rows; dest: n.
-  static void partition(const int32_t* keys, int64_t n, int log_p, uint32_t* counts, int32_t* keys_out, int32_t* dest,
-                        const Launch& L) {
+  // counts: partition_count_words(n, log_p, L) words; ranges: n bytes;
+  // keys_out: n rows; dest: n.
+  static void partition(const int32_t* keys, int64_t n, int log_p, uint32_t* counts, uint8_t* ranges,
+                        int32_t* keys_out, int32_t* dest, const Launch& L) {
     TraceScope ts(kKPartition, L.stream, 3);
     int tpb = 0;
     const int G = partition_grid(n, L, &tpb);
     const int P = 1 << log_p;
     uint32_t* range_totals = counts + static_cast<int64_t>(P) * G;
-    launch_dependent(partition_count_kernel<D>, G, 256, L.stream, keys, n, log_p, tpb, counts);
+    launch_dependent(partition_count_kernel<D>, G, kCountThreads, L.stream, keys, n, log_p, tpb, counts, ranges);
     launch_partition_scan(counts, G, P, range_totals, L);
-    constexpr size_t smem = partition_scatter_smem<D>();
     static bool attr_set = false;  // per key dimension; above 48 KB the kernel must opt in
     if (!attr_set) {
       cudaFuncSetAttribute(partition_scatter_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(smem));
+                           static_cast<int>(partition_scatter_smem<D>(1 << kPartMaxLog)));
       attr_set = true;
     }
-    launch_dependent_smem(partition_scatter_kernel<D>, G, 256, smem, L.stream, keys, n, log_p, tpb,
+    launch_dependent_smem(partition_scatter_kernel<D>, G, kScatterThreads, partition_scatter_smem<D>(P), L.stream, keys,
+                          static_cast<const uint8_t*>(ranges), n, log_p, tpb,
                           static_cast<const uint32_t*>(counts), static_cast<const uint32_t*>(range_totals), keys_out,
                           dest);
   }

@@ -246,21 +246,26 @@ int claim_prefers_slot(const ash_map* m) {
 // log2 of the number of home-bucket ranges a call on n keys is partitioned
 // into, 0 for input order (tuning.partition_keys): 2 to 256 ranges of at
 // most L2/2 bytes of table (8 at least when forced).  By default, calls of
-// 2^20 keys or more on a table larger than twice L2.  The pay-off needs
-// both sides: a ranged find reads kB in range order only if the inserts
-// handed out indices in the same ranges.  Measured on GB300 (uniform keys,
-// uniqueness 0.5, capacity n, queries in a fresh random order), ranged
-// against input order: at 10^8 keys activate 5.6 / 7.9 ms and find 3.1 /
-// 5.1 ms; at 2x10^7 activate 1.12 / 1.23 ms and find 0.58 / 0.80 ms.  Before
-// the calls worked range by range (one launch over all ranged keys), a
-// ranged activate of 10^7 keys (table 1.2x L2) took 0.59 against 0.53 ms,
-// and ranges of L2/4 ran level with L2/2 at 10^8.
+// 2^20 keys or more on a table larger than one and a half times L2.  Measured
+// on GB300 (uniform keys, uniqueness 0.5, capacity n, half of the queries
+// absent), ranged against input order, us:
+//   table / L2    activate       find           find, inserts in input order
+//   0.71          378 / 268      156 / 113
+//   1.18          557 / 533      240 / 242      259 / 220
+//   1.65          713 / 812      311 / 393      345 / 359
+//   2.36          963 / 1245     433 / 633      511 / 576
+//   11.8          4960 / 7898    2302 / 3969    1775 / 2107 (at 7.1)
+// (inserts into maps with value buffers go in input order, so kB is not in
+// range order there).  Ranges of L2/4 or L2 took 8.3 and 8.7 ms where L2/2
+// took 7.5 (both calls at 11.8).  The kernels bring a range's buckets into L2
+// themselves: a prefetch of each range before them cost 0.1 ms, and one that
+// ran beside the kernel before it 0.3 ms.
 int partition_log(const ash_map* m, int64_t n) {
   const int mode = m->tuning.partition_keys;
   if (mode == 1 || n <= 0) return 0;
   const int64_t table = m->n_slots * 8;
   const int64_t l2 = l2_bytes(m->device);
-  if (mode == 0 && (table <= 2 * l2 || n < (int64_t{1} << 20))) return 0;
+  if (mode == 0 && (2 * table <= 3 * l2 || n < (int64_t{1} << 20))) return 0;
   int lg = 1;
   while (lg < ash::kPartMaxLog && (table >> lg) > l2 / 2) ++lg;
   return mode == 2 ? std::max(lg, 3) : lg;
@@ -293,22 +298,14 @@ bool partition_call(ash_map* m, const int32_t* keys, int64_t n, int log_p, cudaS
   pb->dest = reinterpret_cast<int32_t*>(base + words + rows);
   pb->idx = reinterpret_cast<int32_t*>(base + words + rows + ints);
   pb->mask = reinterpret_cast<uint8_t*>(base + words + rows + 2 * ints);
-  m->K.partition(keys, n, log_p, reinterpret_cast<uint32_t*>(base), pb->keys, pb->dest, launch_of(m, st));
+  // the masks' bytes hold the keys' ranges until the scatter has read them
+  m->K.partition(keys, n, log_p, reinterpret_cast<uint32_t*>(base), pb->mask, pb->keys, pb->dest, launch_of(m, st));
   return true;
-}
-
-// The table buckets of range p of P (and a bucket past it, for probes
-// that run on), asked into L2 before the range's keys are worked on.
-void prefetch_table_range(const ash_map* m, int p, int P, const ash::Launch& L) {
-  const int64_t b0 = static_cast<int64_t>(m->n_buckets) * p / P;
-  int64_t b1 = static_cast<int64_t>(m->n_buckets) * (p + 1) / P + 1;
-  if (b1 > m->n_buckets) b1 = m->n_buckets;
-  ash::launch_prefetch_l2(m->slots + b0 * m->S, (b1 - b0) * m->S * 8, L);
 }
 
 // The partitioned call's outputs back in input order; its scratch freed.
 void partition_finish(ash_map* m, const PartBufs& pb, int64_t n, int32_t* idx, uint8_t* mask, cudaStream_t st) {
-  ash::launch_unpermute(pb.dest, n, pb.idx, pb.mask, idx, mask, launch_of(m, st));
+  ash::launch_unpermute(pb.dest, n, pb.idx, idx, mask, launch_of(m, st));
   dev_free(m, pb.mem, st);
 }
 
@@ -881,8 +878,8 @@ ash_status insert_impl(ash_map* m, const int32_t* keys, const void* const* value
     m->K.claim_pts(m->S, kpt, pref, tv, *pts, n, idx, L);
     m->K.commit_pts(ckpt, tv, *pts, n, idx, mask, inline_value ? &vr : nullptr, L);
   } else if (log_p > 0) {
-    // One range after the other: its table buckets are asked into L2, then
-    // its keys claimed and committed.  The slices are the ranged order cut
+    // One range after the other: its keys are claimed, which brings its
+    // table buckets into L2, then committed.  The slices are the ranged order cut
     // at n p / P (about the ranges' bounds, which only the device knows).
     // Cutting claims and commits by position keeps the results: a slice's
     // keys equal to a key committed by an earlier slice report it present,
@@ -892,7 +889,6 @@ ash_status insert_impl(ash_map* m, const int32_t* keys, const void* const* value
       const int64_t a = n * p / P;
       const int64_t b = n * (p + 1) / P;  // the last slice is never empty
       if (b == a) continue;
-      prefetch_table_range(m, p, P, L);
       ash::TableView tvp = tv;
       if (p != P - 1) tvp.snap = nullptr;  // the last commit publishes the control block
       const int32_t* sk = ckeys + a * m->key_dim;
@@ -1060,18 +1056,17 @@ ash_status ash_find(ash_map* m, const int32_t* keys, int64_t n, int32_t* buf_ind
   const ash::Launch L = launch_of(m, st);
   const int fkpt = m->tuning.find_keys_per_thread ? m->tuning.find_keys_per_thread : m->tuning.keys_per_thread;
   const int P = log_p > 0 ? 1 << log_p : 1;
+  const ash::TableView tv = view_of(m);
   for (int p = 0; p < P; ++p) {
-    // ranged: one range after the other, its table buckets asked into L2
-    // first (slices cut at n p / P, as for inserts)
+    // ranged: one range after the other (slices cut at n p / P, as for inserts)
     const int64_t a = n * p / P;
     const int64_t b = n * (p + 1) / P;
     if (b == a) continue;
-    if (log_p > 0) prefetch_table_range(m, p, P, L);
     const int32_t* sk = fkeys + a * m->key_dim;
     if (m->tuning.warp_probe == 1)
-      m->K.find_group(m->S, view_of(m), sk, b - a, fidx + a, fmask + a, L);
+      m->K.find_group(m->S, tv, sk, b - a, fidx + a, fmask + a, L);
     else
-      m->K.find(m->S, fkpt, view_of(m), sk, b - a, fidx + a, fmask + a, L);
+      m->K.find(m->S, fkpt, tv, sk, b - a, fidx + a, fmask + a, L);
   }
   if (log_p > 0) partition_finish(m, pb, n, buf_indices, masks, st);
   return check_launch("find");
