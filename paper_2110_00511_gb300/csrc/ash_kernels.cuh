@@ -180,6 +180,117 @@ __device__ __forceinline__ void find_keys(const TableView& t, const int32_t (&k)
   }
 }
 
+// A warp's keys that their home bucket did not settle, in shared memory: they
+// probe on 32 at a time, so that the rounds past the home bucket run on full
+// warps.  Entry: key, fingerprint, the bucket looked at last, how many buckets
+// that makes, and the output row.  Every lane of the warp calls push and
+// round.
+template <int D>
+struct ProbeList {
+  static constexpr int kCap = 64;  // fewer than 32 before a push of up to 32
+  struct Store {
+    int64_t row[kCap];
+    int32_t key[D][kCap];
+    uint32_t fp[kCap], bucket[kCap], probes[kCap];
+  };
+  Store& s;
+  int n = 0;  // warp-uniform
+  __device__ explicit ProbeList(Store& store) : s(store) {}
+
+  __device__ __forceinline__ void push(bool mine, const int32_t (&k)[D], uint32_t fp, uint32_t b, uint32_t probes,
+                                       int64_t row) {
+    const unsigned bal = __ballot_sync(0xFFFFFFFFu, mine);
+    if (mine) {
+      const int at = n + __popc(bal & ((1u << (threadIdx.x & 31)) - 1u));
+      s.row[at] = row;
+#pragma unroll
+      for (int j = 0; j < D; ++j) s.key[j][at] = k[j];
+      s.fp[at] = fp;
+      s.bucket[at] = b;
+      s.probes[at] = probes;
+    }
+    n += __popc(bal);
+    __syncwarp();
+  }
+
+  // The next bucket of up to 32 entries; those that it does not settle are
+  // pushed again.
+  template <int S>
+  __device__ __forceinline__ void round(const TableView& t, int32_t* __restrict__ idx, uint8_t* __restrict__ mask) {
+    const int lane = threadIdx.x & 31;
+    const int from = n > 32 ? n - 32 : 0;
+    const bool v = from + lane < n;
+    const int at = v ? from + lane : 0;
+    int32_t k[1][D];
+#pragma unroll
+    for (int j = 0; j < D; ++j) k[0][j] = s.key[j][at];
+    const uint32_t fp[1] = {s.fp[at]};
+    const uint32_t b[1] = {next_bucket(s.bucket[at], t.n_buckets)};
+    const uint32_t probes = s.probes[at] + 1;
+    const int64_t row = s.row[at];
+    __syncwarp();
+    n = from;
+    bool go[1] = {v && probes <= t.max_probes};
+    int32_t out[1] = {-1};
+    bool rare = false;
+    probe_round<D, S, 1, false>(t, k, fp, b, go, out, rare);
+    if (rare && out[0] < 0) {
+      KeyOf<D> key;
+#pragma unroll
+      for (int j = 0; j < D; ++j) key.v[j] = k[0][j];
+      out[0] = find_slow<D, S>(t, key);
+      go[0] = false;
+    }
+    if (v && !go[0]) {
+      idx[row] = out[0];
+      mask[row] = out[0] >= 0 ? 1 : 0;
+    }
+    push(go[0], k[0], fp[0], b[0], probes, row);
+  }
+};
+
+// Looks up KPT keys of each lane (ok[q]: wanted; row[q]: their output rows),
+// writing what their home buckets settle and listing the rest.
+template <int D, int S, int KPT>
+__device__ __forceinline__ void find_or_list(const TableView& t, const int32_t (&k)[KPT][D], const bool (&ok)[KPT],
+                                             const int64_t (&row)[KPT], ProbeList<D>& list, int32_t* __restrict__ idx,
+                                             uint8_t* __restrict__ mask) {
+  uint32_t fp[KPT], b[KPT];
+  int32_t out[KPT];
+  bool go[KPT];
+  bool rare = false;
+#pragma unroll
+  for (int q = 0; q < KPT; ++q) {
+    const uint64_t h = hash_key<D>(k[q]);
+    fp[q] = fingerprint(h);
+    b[q] = home_bucket(h, t.n_buckets);
+    go[q] = ok[q];
+    out[q] = -1;
+  }
+  probe_round<D, S, KPT, true>(t, k, fp, b, go, out, rare);
+  if (rare) {
+#pragma unroll
+    for (int q = 0; q < KPT; ++q) {
+      if (ok[q] && out[q] < 0) {
+        KeyOf<D> key;
+#pragma unroll
+        for (int j = 0; j < D; ++j) key.v[j] = k[q][j];
+        out[q] = find_slow<D, S>(t, key);
+        go[q] = false;
+      }
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < KPT; ++q) {
+    if (ok[q] && !go[q]) {
+      idx[row[q]] = out[q];
+      mask[row[q]] = out[q] >= 0 ? 1 : 0;
+    }
+    list.push(go[q], k[q], fp[q], b[q], 1u, row[q]);
+    while (list.n >= 32) list.template round<S>(t, idx, mask);
+  }
+}
+
 // Offsets of a neighbour query.  RadiusOffsets: [-radius, radius]^D row-major
 // (the last coordinate fastest), digit by digit of the offset's number in
 // base width = 2 radius + 1; the division by width is a multiplication by
@@ -232,12 +343,17 @@ __global__ void __launch_bounds__(256) neighbors_kernel(TableView t, const int32
   const uint32_t jump_o = static_cast<uint32_t>(jump - jump_r * n_off);
   int64_t r = first / n_off;
   uint32_t o = static_cast<uint32_t>(first - r * n_off);
-  for (int64_t e = first; e < total; e += gridDim.x * tile) {
+  __shared__ typename ProbeList<D>::Store s_list[8];
+  ProbeList<D> list(s_list[threadIdx.x >> 5]);
+  const int lane = threadIdx.x & 31;
+  for (int64_t e = first; e - lane < total; e += gridDim.x * tile) {
     int32_t k[U][D];
     bool ok[U];
+    int64_t row[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      ok[u] = e + u * blockDim.x < total;
+      row[u] = e + u * blockDim.x;
+      ok[u] = row[u] < total;
       if (ok[u]) {
         load_input_key<D>(keys, r, k[u]);
         off.add(o, k[u]);
@@ -252,15 +368,7 @@ __global__ void __launch_bounds__(256) neighbors_kernel(TableView t, const int32
         ++r;
       }
     }
-    int32_t out[U];
-    find_keys<D, S, U>(t, k, ok, out);
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (ok[u]) {
-        idx[e + u * blockDim.x] = out[u];
-        mask[e + u * blockDim.x] = out[u] >= 0 ? 1 : 0;
-      }
-    }
+    find_or_list<D, S, U>(t, k, ok, row, list, idx, mask);
     r += jump_r;
     o += jump_o;
     if (o >= n_off) {
@@ -268,6 +376,7 @@ __global__ void __launch_bounds__(256) neighbors_kernel(TableView t, const int32
       ++r;
     }
   }
+  while (list.n > 0) list.template round<S>(t, idx, mask);
 }
 
 // KPT keys per thread: positions base, base + blockDim.x, ... so every load
@@ -1581,6 +1690,7 @@ struct DimKernels {
                      const Launch&);
 };
 
+#define NGRID resident_grid
 template <int D>
 struct DimLaunchers {
   template <int S, int KPT, class In>
@@ -1709,8 +1819,9 @@ struct DimLaunchers {
                           int32_t* idx, uint8_t* mask, const Launch& L) {
     TraceScope ts(kKNeighbors, L.stream);
     constexpr int U = kNeighborUnroll;
-    launch_dependent(neighbors_kernel<D, S, U, Off>, grid_for((n * n_off + U - 1) / U, L), L.block, L.stream, t, keys,
-                     n, off, static_cast<uint32_t>(n_off), idx, mask);
+    auto* k = neighbors_kernel<D, S, U, Off>;
+    launch_dependent(k, NGRID(k, grid_for((n * n_off + U - 1) / U, L), L), L.block, L.stream, t, keys, n, off,
+                     static_cast<uint32_t>(n_off), idx, mask);
   }
   template <class Off>
   static void neighbors_off(int S, const TableView& t, const int32_t* keys, int64_t n, const Off& off, int64_t n_off,
