@@ -250,7 +250,10 @@ struct ProbeList {
 };
 
 // Looks up KPT keys of each lane (ok[q]: wanted; row[q]: their output rows),
-// writing what their home buckets settle and listing the rest.
+// writing what their home buckets settle and listing the rest.  For kernels
+// bound by issue; the plain find, bound by random sectors, is the faster the
+// more warps it has and keeps find_keys (with the list, at 48 registers, 4M
+// finds took 78 us against 61, 6M on 80 MB of table 150 against 127).
 template <int D, int S, int KPT>
 __device__ __forceinline__ void find_or_list(const TableView& t, const int32_t (&k)[KPT][D], const bool (&ok)[KPT],
                                              const int64_t (&row)[KPT], ProbeList<D>& list, int32_t* __restrict__ idx,
@@ -320,6 +323,13 @@ struct TableOffsets {
   }
 };
 
+// GB300, 200k keys x 27 offsets over a table in L2 (5.4M queries), bound by
+// instruction issue: 110 -> 70 us with the keys that their home bucket does
+// not settle probing on in place, -> 51 us with those in a list per warp
+// (ProbeList) on a grid of the blocks that fit at once (54 on 8 per SM).  One
+// pair per thread: two 4 us slower, four 32 us (before the list); held to 48
+// or fewer registers for more warps, 64-80 us.  L1 allocation of the buckets
+// that neighbouring queries share gained 1 %, so they bypass it.
 constexpr int kNeighborUnroll = 1;
 
 // Neighbour query (the radius search and the neighbour tables of Sec.
@@ -1690,7 +1700,6 @@ struct DimKernels {
                      const Launch&);
 };
 
-#define NGRID resident_grid
 template <int D>
 struct DimLaunchers {
   template <int S, int KPT, class In>
@@ -1820,7 +1829,7 @@ struct DimLaunchers {
     TraceScope ts(kKNeighbors, L.stream);
     constexpr int U = kNeighborUnroll;
     auto* k = neighbors_kernel<D, S, U, Off>;
-    launch_dependent(k, NGRID(k, grid_for((n * n_off + U - 1) / U, L), L), L.block, L.stream, t, keys, n, off,
+    launch_dependent(k, resident_grid(k, grid_for((n * n_off + U - 1) / U, L), L), L.block, L.stream, t, keys, n, off,
                      static_cast<uint32_t>(n_off), idx, mask);
   }
   template <class Off>
