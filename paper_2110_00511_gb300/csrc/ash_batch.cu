@@ -160,24 +160,23 @@ __global__ void __launch_bounds__(kBatchThreads) batch_claim_kernel(const BatchT
 
 __global__ void __launch_bounds__(kBatchThreads) batch_commit_kernel(const BatchTable* __restrict__ tb) {
   __shared__ int64_t s_tile0[kBatchMaxOps];
-  __shared__ int s_warp[33];
-  __shared__ int s_base;
-  __shared__ int s_got;
+  __shared__ TileShared sh;
   load_tile_starts(tb, kPhaseInsert, s_tile0);
   const BatchPhase ph = tb->ph[kPhaseInsert];
-  for (int64_t tile = blockIdx.x; tile < ph.tiles; tile += gridDim.x) {
+  int turn = 0;
+  for (int64_t tile = blockIdx.x; tile < ph.tiles; tile += gridDim.x, turn ^= 1) {
     const BatchOp& op = tb->ops[ph.first + op_of_tile(s_tile0, ph.count, tile)];
     const int64_t base0 = (tile - op.tile0) * blockDim.x;
     const bool val = op.v.row_bytes > 0;  // uniform over the block
     switch (op.key_dim * 2 + (val ? 1 : 0)) {
-      case 2: commit_tile<1, 1, false>(op.t, op.keys, op.n, base0, op.idx, op.mask, op.v, s_warp, &s_base, &s_got); break;
-      case 3: commit_tile<1, 1, true>(op.t, op.keys, op.n, base0, op.idx, op.mask, op.v, s_warp, &s_base, &s_got); break;
-      case 4: commit_tile<2, 1, false>(op.t, op.keys, op.n, base0, op.idx, op.mask, op.v, s_warp, &s_base, &s_got); break;
-      case 5: commit_tile<2, 1, true>(op.t, op.keys, op.n, base0, op.idx, op.mask, op.v, s_warp, &s_base, &s_got); break;
-      case 6: commit_tile<3, 1, false>(op.t, op.keys, op.n, base0, op.idx, op.mask, op.v, s_warp, &s_base, &s_got); break;
-      case 7: commit_tile<3, 1, true>(op.t, op.keys, op.n, base0, op.idx, op.mask, op.v, s_warp, &s_base, &s_got); break;
-      case 8: commit_tile<4, 1, false>(op.t, op.keys, op.n, base0, op.idx, op.mask, op.v, s_warp, &s_base, &s_got); break;
-      default: commit_tile<4, 1, true>(op.t, op.keys, op.n, base0, op.idx, op.mask, op.v, s_warp, &s_base, &s_got); break;
+      case 2: commit_tile<1, 1, false>(op.t, op.keys, op.n, base0, op.idx, op.mask, op.v, sh, turn); break;
+      case 3: commit_tile<1, 1, true>(op.t, op.keys, op.n, base0, op.idx, op.mask, op.v, sh, turn); break;
+      case 4: commit_tile<2, 1, false>(op.t, op.keys, op.n, base0, op.idx, op.mask, op.v, sh, turn); break;
+      case 5: commit_tile<2, 1, true>(op.t, op.keys, op.n, base0, op.idx, op.mask, op.v, sh, turn); break;
+      case 6: commit_tile<3, 1, false>(op.t, op.keys, op.n, base0, op.idx, op.mask, op.v, sh, turn); break;
+      case 7: commit_tile<3, 1, true>(op.t, op.keys, op.n, base0, op.idx, op.mask, op.v, sh, turn); break;
+      case 8: commit_tile<4, 1, false>(op.t, op.keys, op.n, base0, op.idx, op.mask, op.v, sh, turn); break;
+      default: commit_tile<4, 1, true>(op.t, op.keys, op.n, base0, op.idx, op.mask, op.v, sh, turn); break;
     }
   }
 }
@@ -209,17 +208,16 @@ __global__ void __launch_bounds__(kBatchThreads) batch_erase_mark_kernel(const B
 template <bool WIDE>
 __global__ void __launch_bounds__(kBatchThreads) batch_erase_resolve_kernel(const BatchTable* __restrict__ tb) {
   __shared__ int64_t s_tile0[kBatchMaxOps];
-  __shared__ int s_warp[33];
-  __shared__ int s_cnt;
-  __shared__ int s_base;
+  __shared__ TileShared sh;
   load_tile_starts(tb, kPhaseErase, s_tile0);
   const BatchPhase ph = tb->ph[kPhaseErase];
-  for (int64_t tile = blockIdx.x; tile < ph.tiles; tile += gridDim.x) {
+  int turn = 0;
+  for (int64_t tile = blockIdx.x; tile < ph.tiles; tile += gridDim.x, turn ^= 1) {
     const BatchOp& op = tb->ops[ph.first + op_of_tile(s_tile0, ph.count, tile)];
     const int64_t base0 = (tile - op.tile0) * blockDim.x;
-    if (!WIDE || op.S == 4) erase_resolve_tile<4>(op.t, op.n, base0, op.idx, op.mask, s_warp, &s_cnt, &s_base);
-    else if (op.S == 8) erase_resolve_tile<8>(op.t, op.n, base0, op.idx, op.mask, s_warp, &s_cnt, &s_base);
-    else erase_resolve_tile<16>(op.t, op.n, base0, op.idx, op.mask, s_warp, &s_cnt, &s_base);
+    if (!WIDE || op.S == 4) erase_resolve_tile<4>(op.t, op.n, base0, op.idx, op.mask, sh, turn);
+    else if (op.S == 8) erase_resolve_tile<8>(op.t, op.n, base0, op.idx, op.mask, sh, turn);
+    else erase_resolve_tile<16>(op.t, op.n, base0, op.idx, op.mask, sh, turn);
   }
 }
 

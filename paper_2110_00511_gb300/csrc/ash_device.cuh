@@ -52,7 +52,7 @@ struct Ctrl {
   // (committed + tombstones).  One 64-bit atomic updates both.
   unsigned long long top_used;
   int status;
-  unsigned int commit_done;   // blocks of a snapshotting commit that have finished
+  unsigned int commit_done;   // blocks of a snapshotting kernel that have finished
   unsigned long long count;   // listing counter
   unsigned long long list_done;  // blocks of a counting compaction that have finished
 };
@@ -153,6 +153,17 @@ __device__ __forceinline__ void publish_snapshot(Ctrl* ctrl, Snap* snap, uint32_
   *reinterpret_cast<ulonglong2*>(snap) = make_ulonglong2(tu, tu ^ snap_tag(seq));
 }
 
+// Called by thread 0 of every block after the block's heap atomics (its own):
+// the last block publishes the control block for the host's growth checks.
+__device__ __forceinline__ void publish_when_last(const TableView& t) {
+  __threadfence();
+  if (atomicAdd(&t.ctrl->commit_done, 1u) == gridDim.x - 1) {
+    __threadfence();
+    t.ctrl->commit_done = 0u;
+    publish_snapshot(t.ctrl, t.snap, t.snap_seq);
+  }
+}
+
 __device__ __forceinline__ uint64_t coord_mult(int j) {
   // distinct odd constants (fractional parts of golden ratio / sqrt primes)
   switch (j) {
@@ -232,13 +243,26 @@ __device__ __forceinline__ bool input_key_equal(const In& keys, int64_t pos, con
 }
 
 // Home bucket of kB row i, for the kernels that are not compiled per key
-// dimension (same hash as hash_key).
+// dimension (same hash as hash_key): the row by vector loads.
 __device__ __forceinline__ uint32_t home_of_row(const int32_t* kb, int d, uint32_t n_buckets, uint32_t i) {
-  const int ks = d <= 1 ? 1 : (d <= 2 ? 2 : (d <= 4 ? 4 : 8));
-  const int32_t* row = kb + static_cast<size_t>(i) * ks;
+  int4 a = make_int4(0, 0, 0, 0), c = a;
+  if (d <= 1) {
+    a.x = __ldg(kb + i);
+  } else if (d <= 2) {
+    const int2 v = __ldg(reinterpret_cast<const int2*>(kb) + i);
+    a.x = v.x;
+    a.y = v.y;
+  } else if (d <= 4) {
+    a = __ldg(reinterpret_cast<const int4*>(kb) + i);
+  } else {
+    a = __ldg(reinterpret_cast<const int4*>(kb) + 2 * static_cast<size_t>(i));
+    c = __ldg(reinterpret_cast<const int4*>(kb) + 2 * static_cast<size_t>(i) + 1);
+  }
+  // coordinates past d are zero in kB
+  const int32_t k[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w};
   uint64_t h = static_cast<uint64_t>(d);
-#pragma unroll 1
-  for (int j = 0; j < d; ++j) h += static_cast<uint64_t>(static_cast<uint32_t>(__ldg(row + j))) * coord_mult(j);
+#pragma unroll
+  for (int j = 0; j < 8; ++j) h += static_cast<uint64_t>(static_cast<uint32_t>(k[j])) * coord_mult(j);
   return home_bucket(mix64(h), n_buckets);
 }
 
@@ -324,6 +348,28 @@ __device__ __forceinline__ uint64_t load_slot_relaxed(const uint64_t* p) {
 }
 
 // --------------------------------------------------------------- aggregation
+// Shared memory of a tile loop that ranks threads and takes one heap atomic
+// per tile.  Two copies, used in turn: what a tile wrote is not overwritten
+// before every thread has passed the next tile's first barrier, so a tile
+// needs two barriers (counts written; heap reserved) and none at its end.
+struct TileShared {
+  int cnt[2][32];
+  int base[2];
+  int got[2];
+  uint32_t ask[8][8];  // per warp: buckets that nobody_probes_past looks at together
+};
+
+// Inclusive warp scan.
+__device__ __forceinline__ int warp_scan(int x) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+    if (lane >= o) x += y;
+  }
+  return x;
+}
+
 // Block-wide exclusive rank of threads with `flag` set and the block total.
 // Every thread of the block must call it (it contains __syncthreads).
 // `s_warp` needs blockDim.x / 32 + 1 ints of shared memory.
@@ -375,15 +421,6 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int& total, int* s_wa
   __syncthreads();
   total = s_warp[n_warps];
   return s_warp[warp] + x - v;
-}
-
-__device__ __forceinline__ int block_count(bool flag, int* s_cnt) {
-  const unsigned ballot = __ballot_sync(0xFFFFFFFFu, flag);
-  if (threadIdx.x == 0) *s_cnt = 0;
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0 && ballot) atomicAdd(s_cnt, __popc(ballot));
-  __syncthreads();
-  return *s_cnt;
 }
 
 }  // namespace ash

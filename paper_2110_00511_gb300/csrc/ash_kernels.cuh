@@ -1023,15 +1023,19 @@ __device__ __forceinline__ void copy_small_row(const ValueRow& v, int32_t i, int
 // KPT keys per thread per block iteration (blockDim.x * KPT keys).  Who won
 // each key: FLAGS, a position holding a slot index whose winner-flag bit
 // (t.lost) is clear, from two streamed reads; otherwise the slot word, read
-// at random, names the winning position.  One block-wide scan ranks the
-// winners and ONE heap atomic serves the iteration (Sec. 4.3: t is raised by
-// the number of indices taken).  Winners then write kB(i), the value row, the
-// committed slot word and their outputs.
+// at random, names the winning position.  The warps' counts of winners are
+// scanned by every warp for itself and ONE heap atomic serves the iteration
+// (Sec. 4.3: t is raised by the number of indices taken).  Winners then write
+// kB(i), the value row, the committed slot word and their outputs.  `turn`
+// alternates between 0 and 1 from tile to tile (TileShared).
 template <int D, int KPT, bool VAL, class In, bool FLAGS = false>
 __device__ __forceinline__ void commit_tile(const TableView& t, const In& keys, int64_t n,
                                             int64_t base0, int32_t* __restrict__ idx, uint8_t* __restrict__ mask,
-                                            const ValueRow& v, int* s_warp, int* s_base, int* s_got) {
+                                            const ValueRow& v, TileShared& sh, int turn) {
   const int64_t base = base0 + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5;
+  const int n_warps = blockDim.x >> 5;
   int32_t s[KPT];
 #pragma unroll
   for (int q = 0; q < KPT; ++q) {
@@ -1039,21 +1043,23 @@ __device__ __forceinline__ void commit_tile(const TableView& t, const In& keys, 
     s[q] = pos < n ? idx[pos] : -1;
   }
   uint64_t w[KPT];
-  bool win[KPT];
-  int cnt = 0;
+  unsigned won[KPT];  // of this warp
   if constexpr (FLAGS) {
     uint32_t lw[KPT];
 #pragma unroll
     for (int q = 0; q < KPT; ++q) {
       const int64_t pos = base + static_cast<int64_t>(q) * blockDim.x;
+      w[q] = 0;
       lw[q] = pos < n ? t.lost[pos >> 5] : 0u;
     }
 #pragma unroll
     for (int q = 0; q < KPT; ++q) {
       const int64_t pos = base + static_cast<int64_t>(q) * blockDim.x;
-      w[q] = 0;
-      win[q] = s[q] >= 0 && !((lw[q] >> (pos & 31)) & 1u);
-      cnt += win[q] ? 1 : 0;
+      won[q] = __ballot_sync(0xFFFFFFFFu, s[q] >= 0 && !((lw[q] >> (pos & 31)) & 1u));
+      // leave the flags clear for the next insert (blockDim and the tile base
+      // are multiples of 32, so a warp's 32 positions of one slice are one
+      // word, which no other warp reads)
+      if (lane == 0 && lw[q] != 0u) t.lost[pos >> 5] = 0u;
     }
   } else {
 #pragma unroll
@@ -1061,48 +1067,45 @@ __device__ __forceinline__ void commit_tile(const TableView& t, const In& keys, 
 #pragma unroll
     for (int q = 0; q < KPT; ++q) {
       const int64_t pos = base + static_cast<int64_t>(q) * blockDim.x;
-      win[q] = s[q] >= 0 && lo32(w[q]) == (kClaimBit | static_cast<uint32_t>(pos));
-      cnt += win[q] ? 1 : 0;
+      won[q] = __ballot_sync(0xFFFFFFFFu, s[q] >= 0 && lo32(w[q]) == (kClaimBit | static_cast<uint32_t>(pos)));
     }
   }
-  int total;
-  const int off = block_exclusive_scan(cnt, total, s_warp);  // a block barrier: every flag word was read
-  if constexpr (FLAGS) {
-    // leave the flags clear for the next insert (one lane per 32 positions;
-    // blockDim and the tile base are multiples of 32, so a warp's 32
-    // positions of one slice share one word)
+  if (lane == 0) {
 #pragma unroll
-    for (int q = 0; q < KPT; ++q) {
-      const int64_t pos = base + static_cast<int64_t>(q) * blockDim.x;
-      if (pos < n && (pos & 31) == 0) t.lost[pos >> 5] = 0u;
-    }
-  }
-  if (threadIdx.x == 0) {
-    int got = 0, top = 0;
-    if (total > 0) {
-      const unsigned long long add = (static_cast<unsigned long long>(total) << 32) | static_cast<unsigned long long>(total);
-      const unsigned long long old = atomicAdd(&t.ctrl->top_used, add);
-      top = static_cast<int>(static_cast<uint32_t>(old));
-      got = t.capacity - top;
-      got = got < 0 ? 0 : (got > total ? total : got);
-      if (got < total) {
-        // give back the part of t that the heap could not serve
-        atomicAdd(&t.ctrl->top_used, 0ull - static_cast<unsigned long long>(total - got));
-        atomicOr(&t.ctrl->status, kStatusCapacity);
-      }
-    }
-    *s_base = top;
-    *s_got = got;
+    for (int q = 0; q < KPT; ++q) sh.cnt[turn][q * n_warps + warp] = __popc(won[q]);
   }
   __syncthreads();
-  const int got = *s_got;
-  const int hbase = *s_base;
-  int r = off;
+  const int c = lane < KPT * n_warps ? sh.cnt[turn][lane] : 0;
+  const int upto = warp_scan(c);
+  if (threadIdx.x < 32) {
+    const int total = __shfl_sync(0xFFFFFFFFu, upto, 31);
+    if (threadIdx.x == 0) {
+      int got = 0, top = 0;
+      if (total > 0) {
+        const unsigned long long add = (static_cast<unsigned long long>(total) << 32) | static_cast<unsigned long long>(total);
+        const unsigned long long old = atomicAdd(&t.ctrl->top_used, add);
+        top = static_cast<int>(static_cast<uint32_t>(old));
+        got = t.capacity - top;
+        got = got < 0 ? 0 : (got > total ? total : got);
+        if (got < total) {
+          // give back the part of t that the heap could not serve
+          atomicAdd(&t.ctrl->top_used, 0ull - static_cast<unsigned long long>(total - got));
+          atomicOr(&t.ctrl->status, kStatusCapacity);
+        }
+      }
+      sh.base[turn] = top;
+      sh.got[turn] = got;
+    }
+  }
+  __syncthreads();
+  const int got = sh.got[turn];
+  const int hbase = sh.base[turn];
 #pragma unroll
   for (int q = 0; q < KPT; ++q) {
     const int64_t pos = base + static_cast<int64_t>(q) * blockDim.x;
+    const int r = __shfl_sync(0xFFFFFFFFu, upto - c, q * n_warps + warp) + __popc(won[q] & ((1u << lane) - 1u));
     if (pos < n) {
-      if (win[q]) {
+      if ((won[q] >> lane) & 1u) {
         if (r < got) {
           const int32_t i = (t.flags & kViewHeapIdentity) ? hbase + r : t.heap[hbase + r];
           int32_t k[D];
@@ -1118,38 +1121,26 @@ __device__ __forceinline__ void commit_tile(const TableView& t, const In& keys, 
           idx[pos] = -1;
           mask[pos] = 0;
         }
-        ++r;
       } else {
         idx[pos] = -1;
         mask[pos] = 0;
       }
     }
   }
-  __syncthreads();
 }
 
 template <int D, int KPT, bool VAL, class In = const int32_t*, bool FLAGS = false>
 __global__ void __launch_bounds__(256) commit_kernel(TableView t, const In keys, int64_t n,
                                                      int32_t* __restrict__ idx, uint8_t* __restrict__ mask,
                                                      ValueRow v) {
-  __shared__ int s_warp[33];
-  __shared__ int s_base;
-  __shared__ int s_got;
+  __shared__ TileShared sh;
   // a programmatic dependent of the previous kernel: wait for its grid (a no-op otherwise)
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int64_t step = static_cast<int64_t>(gridDim.x) * blockDim.x * KPT;
-  for (int64_t base0 = static_cast<int64_t>(blockIdx.x) * blockDim.x * KPT; base0 < n; base0 += step)
-    commit_tile<D, KPT, VAL, In, FLAGS>(t, keys, n, base0, idx, mask, v, s_warp, &s_base, &s_got);
-  // The last block to finish publishes the control block for the host's
-  // growth checks (every block's heap atomics were made by its thread 0).
-  if (t.snap != nullptr && threadIdx.x == 0) {
-    __threadfence();
-    if (atomicAdd(&t.ctrl->commit_done, 1u) == gridDim.x - 1) {
-      __threadfence();
-      t.ctrl->commit_done = 0u;
-      publish_snapshot(t.ctrl, t.snap, t.snap_seq);
-    }
-  }
+  int turn = 0;
+  for (int64_t base0 = static_cast<int64_t>(blockIdx.x) * blockDim.x * KPT; base0 < n; base0 += step, turn ^= 1)
+    commit_tile<D, KPT, VAL, In, FLAGS>(t, keys, n, base0, idx, mask, v, sh, turn);
+  if (t.snap != nullptr && threadIdx.x == 0) publish_when_last(t);
 }
 
 // ------------------------------------------------------- key partitioning
@@ -1431,24 +1422,43 @@ __global__ void __launch_bounds__(256) erase_mark_kernel(TableView t, const int3
 }
 
 // ------------------------------------------------------------ erase: resolve
-// Whether no key that stays in the table probes on past bucket b: such a key
-// would have to sit in the next bucket (which holds an EMPTY slot, so none of
-// its chains goes further) with another home bucket.  Marked words leave the
-// table in this kernel, so they do not count; a slot of the next bucket that
-// another thread empties meanwhile only makes the answer truer.
+// For every lane with `asks`: whether no key that stays in the table probes
+// on past its bucket b.  Such a key would have to sit in the next bucket (which
+// holds an EMPTY slot, so none of its chains goes further) with another home
+// bucket.  Marked words leave the table in this kernel, so they do not count;
+// a slot of the next bucket that another thread empties meanwhile only makes
+// the answer truer.  Few lanes ask, so the warp answers 32 / S of them at a
+// time, a lane per slot of the next bucket: one slot load and one kB row deep
+// (a lane that walked its bucket alone held its warp for four of each, and the
+// resolve of 262k erases took 18.8 us instead of 14.2).
 template <int S>
-__device__ __noinline__ bool nobody_probes_past(const uint64_t* slots, const int32_t* kb, uint32_t n_buckets,
-                                                int key_dim, uint32_t b) {
-  const uint32_t nb = next_bucket(b, n_buckets);
-  if (nb == b) return false;
-  bool empty = false;
-#pragma unroll 1
-  for (int j = 0; j < S; ++j) {
-    const uint64_t w = load_slot_relaxed(slots + static_cast<size_t>(nb) * S + j);
-    empty |= (w == kEmpty);
-    if (is_committed(w) && home_of_row(kb, key_dim, n_buckets, lo32(w)) != nb) return false;
+__device__ __forceinline__ bool nobody_probes_past(const TableView& t, bool asks, uint32_t b, uint32_t* ask) {
+  constexpr int G = 32 / S;
+  const int lane = threadIdx.x & 31;
+  const unsigned asking = __ballot_sync(0xFFFFFFFFu, asks);
+  const int n = __popc(asking);
+  const int rank = __popc(asking & ((1u << lane) - 1u));
+  bool none = false;
+  for (int r = 0; r < n; r += G) {
+    const bool mine = asks && rank >= r && rank < r + G;
+    if (mine) ask[rank - r] = b;
+    __syncwarp();
+    const int g = lane / S;
+    bool empty = false, displaced = false;
+    if (r + g < n) {
+      const uint32_t nb = next_bucket(ask[g], t.n_buckets);
+      const uint64_t w = load_slot_relaxed(t.slots + static_cast<size_t>(nb) * S + lane % S);
+      empty = w == kEmpty;
+      displaced = nb == ask[g] || (is_committed(w) && home_of_row(t.kb, t.key_dim, t.n_buckets, lo32(w)) != nb);
+    }
+    const unsigned eb = __ballot_sync(0xFFFFFFFFu, empty), db = __ballot_sync(0xFFFFFFFFu, displaced);
+    if (mine) {
+      const unsigned group = ((1u << S) - 1u) << ((rank - r) * S);
+      none = (eb & group) != 0u && (db & group) == 0u;
+    }
+    __syncwarp();
   }
-  return empty;
+  return none;
 }
 
 // One tile of blockDim.x positions starting at base0.  Every thread of the
@@ -1456,73 +1466,88 @@ __device__ __noinline__ bool nobody_probes_past(const uint64_t* slots, const int
 template <int S>
 __device__ __forceinline__ void erase_resolve_tile(const TableView& t, int64_t n, int64_t base0,
                                                    const int32_t* __restrict__ slot_in, uint8_t* __restrict__ mask,
-                                                   int* s_warp, int* s_cnt, int* s_base) {
+                                                   TileShared& sh, int turn) {
+  const int lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5;
   const int64_t pos = base0 + threadIdx.x;
   const bool active = pos < n;
   const int32_t s = active ? slot_in[pos] : -1;
   uint64_t w = 0;
   bool win = false, to_empty = false;
+  bool past_home = false;  // its bucket has no EMPTY slot: chains may pass
+  bool held = false;       // another live key prefers the slot
   if (s >= 0) {
-    w = load_slot_relaxed(t.slots + s);
-    win = hi32(w) == static_cast<uint32_t>(pos);
-    if (win) {
-      // EMPTY only when no probe chain passes through the bucket (it already
-      // has an EMPTY slot, or nobody_probes_past it) and, while the map keeps
-      // the preferred-slot invariant, no other live key of the bucket prefers
-      // the freed slot; a TOMBSTONE otherwise (the freed slot itself holds a
-      // marked word, which never counts).  The bucket is read 32 bytes at a
-      // time to keep few words live.
-      const uint64_t* bp = t.slots + static_cast<size_t>(s / S) * S;
-      const uint32_t own = static_cast<uint32_t>(s) & (S - 1);
-      bool preferred = false;
+    // EMPTY only when no probe chain passes through the bucket (it already has
+    // an EMPTY slot, or nobody_probes_past it) and, while the map keeps the
+    // preferred-slot invariant, no other live key of the bucket prefers the
+    // freed slot; a TOMBSTONE otherwise (the freed slot itself holds a marked
+    // word, which never counts).  The bucket is read 32 bytes at a time, the
+    // slot's own 32 bytes first: they tell the winner.
+    const uint64_t* bp = t.slots + static_cast<size_t>(s / S) * S;
+    const uint32_t own = static_cast<uint32_t>(s) & (S - 1);
+    bool preferred = false;
 #pragma unroll 1
-      for (int c = 0; c < S / 4; ++c) {
-        uint64_t cw[4];
-        load32<false>(bp + 4 * c, cw[0], cw[1], cw[2], cw[3]);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          to_empty |= (cw[j] == kEmpty);
-          preferred |= is_committed(cw[j]) && pref_slot<S>(hi32(cw[j])) == own;
-        }
+    for (int c = 0; c < S / 4; ++c) {
+      const uint32_t part = (own / 4 + c) % (S / 4);
+      uint64_t cw[4];
+      load32<false>(bp + 4 * part, cw[0], cw[1], cw[2], cw[3]);
+      if (c == 0) {
+        w = (own & 2) ? ((own & 1) ? cw[3] : cw[2]) : ((own & 1) ? cw[1] : cw[0]);
+        win = hi32(w) == static_cast<uint32_t>(pos);
+        if (!win) break;
       }
-      preferred &= (t.flags & kViewPrefPlaced) != 0;
-      if (!to_empty && !preferred) to_empty = nobody_probes_past<S>(t.slots, t.kb, t.n_buckets, t.key_dim, static_cast<uint32_t>(s) / S);
-      to_empty &= !preferred;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        to_empty |= (cw[j] == kEmpty);
+        preferred |= is_committed(cw[j]) && pref_slot<S>(hi32(cw[j])) == own;
+      }
     }
+    past_home = win && !to_empty;
+    held = preferred && (t.flags & kViewPrefPlaced);
   }
-  int rank, total;
-  block_rank(win, rank, total, s_warp);
-  const int n_empty = block_count(to_empty, s_cnt);
-  if (threadIdx.x == 0) {
-    int top = 0;
-    if (total > 0) {
-      const unsigned long long sub = (static_cast<unsigned long long>(n_empty) << 32) + static_cast<unsigned long long>(total);
-      const unsigned long long old = atomicAdd(&t.ctrl->top_used, 0ull - sub);
-      top = static_cast<int>(static_cast<uint32_t>(old));
+  if (nobody_probes_past<S>(t, past_home && !held, static_cast<uint32_t>(s) / S, sh.ask[warp])) to_empty = true;
+  to_empty &= !held;
+  // winners in the low half, slots that become EMPTY in the high half
+  const unsigned won = __ballot_sync(0xFFFFFFFFu, win);
+  const unsigned emptied = __ballot_sync(0xFFFFFFFFu, to_empty);
+  if (lane == 0) sh.cnt[turn][warp] = __popc(won) | __popc(emptied) << 16;
+  __syncthreads();
+  const int c = lane < static_cast<int>(blockDim.x >> 5) ? sh.cnt[turn][lane] : 0;
+  const int upto = warp_scan(c);
+  if (threadIdx.x < 32) {
+    const int both = __shfl_sync(0xFFFFFFFFu, upto, 31);
+    if (threadIdx.x == 0) {
+      const int total = both & 0xFFFF;
+      int top = 0;
+      if (total > 0) {
+        const unsigned long long sub = (static_cast<unsigned long long>(both >> 16) << 32) + static_cast<unsigned long long>(total);
+        const unsigned long long old = atomicAdd(&t.ctrl->top_used, 0ull - sub);
+        top = static_cast<int>(static_cast<uint32_t>(old));
+      }
+      sh.base[turn] = top - total;
     }
-    *s_base = top - total;
   }
   __syncthreads();
+  const int before = __shfl_sync(0xFFFFFFFFu, upto - c, warp) & 0xFFFF;
   if (win) {
-    t.heap[*s_base + rank] = static_cast<int32_t>(lo32(w));
+    t.heap[sh.base[turn] + before + __popc(won & ((1u << lane) - 1u))] = static_cast<int32_t>(lo32(w));
     t.slots[s] = to_empty ? kEmpty : kTombstone;
     mask[pos] = 1;
   } else if (active) {
     mask[pos] = 0;
   }
-  __syncthreads();
 }
 
 template <int S>
 __global__ void __launch_bounds__(256) erase_resolve_kernel(TableView t, int64_t n, const int32_t* __restrict__ slot_in,
                                                             uint8_t* __restrict__ mask) {
-  __shared__ int s_warp[33];
-  __shared__ int s_cnt;
-  __shared__ int s_base;
+  __shared__ TileShared sh;
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t base = static_cast<int64_t>(blockIdx.x) * blockDim.x; base < n; base += stride)
-    erase_resolve_tile<S>(t, n, base, slot_in, mask, s_warp, &s_cnt, &s_base);
+  int turn = 0;
+  for (int64_t base = static_cast<int64_t>(blockIdx.x) * blockDim.x; base < n; base += stride, turn ^= 1)
+    erase_resolve_tile<S>(t, n, base, slot_in, mask, sh, turn);
+  if (t.snap != nullptr && threadIdx.x == 0) publish_when_last(t);
 }
 
 // ------------------------------------------------------------------ rebuild

@@ -1115,12 +1115,17 @@ ash_status ash_erase(ash_map* m, const int32_t* keys, int64_t n, uint8_t* masks,
   s = ensure_scratch(m, n * 4, st);
   if (s != ASH_OK) return s;
   const ash::Launch L = launch_of(m, st);
-  const ash::TableView tv = view_of(m);
+  ash::TableView tv = view_of(m);
+  m->erased_since_snap += n;
+  const bool snap = snapshot_wanted(m, st, 0);
+  if (snap) {  // published by the resolve kernel's last block
+    tv.snap = m->snap_dev;
+    tv.snap_seq = m->snap_seq;
+  }
   m->K.erase_mark(m->S, tv, keys, n, m->scratch, L);
   ash::launch_erase_resolve(m->S, tv, n, m->scratch, masks, L);
   m->heap_identity = false;
-  m->erased_since_snap += n;
-  maybe_snapshot(m, st);
+  if (snap) snapshot_issued(m);
   return check_launch("erase");
 }
 
