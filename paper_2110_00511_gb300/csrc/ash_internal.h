@@ -114,6 +114,8 @@ void* dev_alloc(ash_map* m, size_t bytes, cudaStream_t st);
 void dev_free(ash_map* m, void* p, cudaStream_t st);
 Launch launch_of(const ash_map* m, cudaStream_t st);
 TableView view_of(const ash_map* m);
+// log2 of the home-bucket ranges that a call on n keys is partitioned into (0: input order).
+int partition_log(const ash_map* m, int64_t n);
 ash_status check_keys(const ash_map* m, const void* keys, int64_t n);
 // x2 growth / table rebuild so that a batch of n insert keys fits (may synchronise st).
 ash_status ensure_room(ash_map* m, int64_t n, cudaStream_t st);

@@ -423,6 +423,24 @@ __global__ void __launch_bounds__(256) find_kernel(TableView t, const In keys, i
   }
 }
 
+// find, and the index found for row r goes to link[link_at[r]] as well.
+template <int D, int S>
+__global__ void __launch_bounds__(256) find_link_kernel(TableView t, const int32_t* __restrict__ keys, int64_t n,
+                                                        int32_t* __restrict__ idx, int32_t* __restrict__ link,
+                                                        const int32_t* __restrict__ link_at) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int64_t step = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  for (int64_t r = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; r < n; r += step) {
+    int32_t k[1][D], out[1];
+    const bool ok[1] = {true};
+    load_input_key<D>(keys, r, k[0]);
+    const int32_t at = __ldg(link_at + r);
+    find_keys<D, S, 1>(t, k, ok, out);
+    idx[r] = out[0];
+    link[at] = out[0];
+  }
+}
+
 // Warp-cooperative find: a group of G = S / 2 lanes takes one key, each lane
 // loading two slots (one 16-byte load; the group reads the whole bucket in one
 // coalesced request), so a warp has 32 / G keys in flight.  Fingerprint
@@ -1715,6 +1733,8 @@ struct DimKernels {
   void (*neighbors)(int S, const TableView&, const int32_t*, int64_t, int, int64_t, int32_t*, uint8_t*, const Launch&);
   void (*offsets)(int S, const TableView&, const int32_t*, int64_t, const int32_t*, int64_t, int32_t*, uint8_t*,
                   const Launch&);
+  void (*find_link)(int S, const TableView&, const int32_t*, int64_t, int32_t*, int32_t*, const int32_t*,
+                    const Launch&);
   void (*find_group)(int S, const TableView&, const int32_t*, int64_t, int32_t*, uint8_t*, const Launch&);
   // stable partition of n key rows by home-bucket range (scratch: see partition_bytes)
   void (*partition)(const int32_t*, int64_t, int, uint32_t*, uint8_t*, int32_t*, int32_t*, const Launch&);
@@ -1875,6 +1895,18 @@ struct DimLaunchers {
     neighbors_off(S, t, keys, n, TableOffsets{off}, n_off, idx, mask, L);
   }
   template <int S>
+  static void find_link_s(const TableView& t, const int32_t* keys, int64_t n, int32_t* idx, int32_t* link,
+                          const int32_t* link_at, const Launch& L) {
+    TraceScope ts(kKFind, L.stream);
+    launch_dependent(find_link_kernel<D, S>, grid_for(n, L), L.block, L.stream, t, keys, n, idx, link, link_at);
+  }
+  static void find_link(int S, const TableView& t, const int32_t* keys, int64_t n, int32_t* idx, int32_t* link,
+                        const int32_t* link_at, const Launch& L) {
+    if (S == 4) find_link_s<4>(t, keys, n, idx, link, link_at, L);
+    else if (S == 8) find_link_s<8>(t, keys, n, idx, link, link_at, L);
+    else find_link_s<16>(t, keys, n, idx, link, link_at, L);
+  }
+  template <int S>
   static void find_group_s(const TableView& t, const int32_t* keys, int64_t n, int32_t* idx, uint8_t* mask,
                            const Launch& L) {
     TraceScope ts(kKFind, L.stream);
@@ -1917,6 +1949,7 @@ struct DimLaunchers {
     k.neighbors = &neighbors;
     k.offsets = &offsets;
     k.find_group = &find_group;
+    k.find_link = &find_link;
     k.find_pts = &find_pts;
     k.claim_pts = &claim_pts;
     k.commit_pts = &commit_pts;

@@ -58,14 +58,21 @@ __device__ __forceinline__ float transform_row(const Cam& k, int a, float x, flo
 __device__ __forceinline__ bool depth_valid(float d, float depth_max) { return d > 0.0f && d <= depth_max; }
 
 // ------------------------------------------------------ ordered compaction
-// Three launches: per-tile counts, one-block scan of the tile counts, and a
-// write pass in which every tile places its flagged items at its offset in
-// input order.  Tiles are kTile consecutive items; item q * kThreads + tid of
-// a tile belongs to thread tid, so loads stay coalesced and the rank order
-// (q, then tid) is input order.
+// Per-tile counts, then a write pass in which every tile places its flagged
+// items at its offset in input order.  Tiles are kTile consecutive items; item
+// q * kThreads + tid of a tile belongs to thread tid, so loads stay coalesced
+// and the rank order (q, then tid) is input order.  Up to kSummedTiles tiles,
+// each block of the write pass adds up the counts before its own (16 KB from
+// L2 at most) and the last one writes the total, to the host too when it
+// waits for it; above, a one-block scan of the counts comes between.  Launches
+// and the copy of the count to the host are most of a call on an image: 640 x
+// 480 pixels 33 us with the wait for the count, 50 with three launches and a
+// copy.
+constexpr int64_t kSummedTiles = 4096;
 
 template <class Pred>
 __global__ void __launch_bounds__(kThreads) tile_count_kernel(Pred pred, int64_t n, int32_t* __restrict__ tile_count) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   __shared__ int s_warp[kThreads / 32 + 1];
   const int64_t base = static_cast<int64_t>(blockIdx.x) * kTile;
   int c = 0;
@@ -79,9 +86,11 @@ __global__ void __launch_bounds__(kThreads) tile_count_kernel(Pred pred, int64_t
   if (threadIdx.x == 0) tile_count[blockIdx.x] = total;
 }
 
-// Exclusive scan of n_tiles counts in place; the grand total goes to *total.
+// Exclusive scan of n_tiles counts in place; the grand total goes to *total
+// (and *host).
 __global__ void __launch_bounds__(kScanThreads) tile_scan_kernel(int32_t* __restrict__ tile, int64_t n_tiles,
-                                                                 int64_t* __restrict__ total) {
+                                                                 int64_t* __restrict__ total, int64_t* host) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   __shared__ int s_warp[kScanThreads / 32 + 1];
   int64_t carry = 0;
   for (int64_t base = 0; base < n_tiles; base += kScanThreads) {
@@ -93,23 +102,44 @@ __global__ void __launch_bounds__(kScanThreads) tile_scan_kernel(int32_t* __rest
     carry += chunk;
     __syncthreads();  // s_warp is reused by the next chunk
   }
-  if (threadIdx.x == 0) *total = carry;
+  if (threadIdx.x == 0) {
+    *total = carry;
+    if (host) *host = carry;
+  }
 }
 
-template <class Pred, class Write>
+// SUMMED: tile holds the counts, else their exclusive scan (total and host
+// unused then).
+template <class Pred, class Write, bool SUMMED>
 __global__ void __launch_bounds__(kThreads) tile_write_kernel(Pred pred, Write write, int64_t n,
-                                                              const int32_t* __restrict__ tile_off) {
+                                                              const int32_t* __restrict__ tile,
+                                                              int64_t* __restrict__ total, int64_t* host) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   __shared__ int s_warp[kThreads / 32 + 1];
   const int64_t base = static_cast<int64_t>(blockIdx.x) * kTile;
-  int64_t out = tile_off[blockIdx.x];
+  int64_t out = 0;
+  if constexpr (SUMMED) {
+    int sum = 0;
+    for (int i = threadIdx.x; i < static_cast<int>(blockIdx.x); i += kThreads) sum += __ldg(tile + i);
+    int before = 0;
+    block_exclusive_scan(sum, before, s_warp);
+    out = before;
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+      *total = out + tile[blockIdx.x];
+      if (host) *host = out + tile[blockIdx.x];
+    }
+    __syncthreads();  // s_warp is reused below
+  } else {
+    out = tile[blockIdx.x];
+  }
 #pragma unroll 1
   for (int q = 0; q < kItems; ++q) {
     const int64_t i = base + q * kThreads + threadIdx.x;
     const bool f = i < n && pred(i);
-    int rank = 0, total = 0;
-    block_rank(f, rank, total, s_warp);
+    int rank = 0, total_q = 0;
+    block_rank(f, rank, total_q, s_warp);
     if (f) write(i, out + rank);
-    out += total;
+    out += total_q;
     __syncthreads();  // s_warp is reused by the next round
   }
 }
@@ -168,6 +198,7 @@ struct UniqueWrite {
 __global__ void __launch_bounds__(kThreads) scatter_index_kernel(int32_t* __restrict__ local_values,
                                                                  const int32_t* __restrict__ li,
                                                                  const int32_t* __restrict__ gi, int64_t u) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   for (int64_t r = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; r < u;
        r += static_cast<int64_t>(gridDim.x) * blockDim.x)
     local_values[__ldg(li + r)] = __ldg(gi + r);
@@ -192,6 +223,7 @@ __global__ void __launch_bounds__(kThreads) integrate_kernel(const int32_t* __re
                                                              float depth_max) {
   constexpr int kVox = ELL * ELL * ELL;
   constexpr int kPer = kVox / kThreads;  // voxels per thread (2 for 8^3, 16 for 16^3)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int32_t bi = __ldg(block_idx + blockIdx.x);
   if (bi < 0 || bi >= capacity) return;
   float* trow = tsdf + static_cast<int64_t>(bi) * kVox;
@@ -640,18 +672,28 @@ void* scratch_alloc(size_t bytes, cudaStream_t st) {
 }
 
 // Ordered compaction with a caller-provided predicate and writer; the count
-// lands in *count_dev.  tile scratch: n_tiles int32.
+// lands in *count_dev, and in *count_host (mapped) unless null.  tile
+// scratch: n_tiles int32.
 template <class Pred, class Write>
-void compact(Pred pred, Write write, int64_t n, int32_t* tile, int64_t* count_dev, cudaStream_t st, int kind) {
+void compact(Pred pred, Write write, int64_t n, int32_t* tile, int64_t* count_dev, int64_t* count_host,
+             cudaStream_t st, int kind) {
   const int64_t n_tiles = (n + kTile - 1) / kTile;
   if (n_tiles == 0) {
     cudaMemsetAsync(count_dev, 0, sizeof(int64_t), st);
+    if (count_host) *count_host = 0;
     return;
   }
-  TraceScope ts(kind, st, 3);
-  tile_count_kernel<<<static_cast<unsigned>(n_tiles), kThreads, 0, st>>>(pred, n, tile);
-  tile_scan_kernel<<<1, kScanThreads, 0, st>>>(tile, n_tiles, count_dev);
-  tile_write_kernel<<<static_cast<unsigned>(n_tiles), kThreads, 0, st>>>(pred, write, n, tile);
+  const int grid = static_cast<int>(n_tiles);
+  TraceScope ts(kind, st, n_tiles <= kSummedTiles ? 2 : 3);
+  launch_dependent(tile_count_kernel<Pred>, grid, kThreads, st, pred, n, tile);
+  if (n_tiles <= kSummedTiles) {
+    launch_dependent(tile_write_kernel<Pred, Write, true>, grid, kThreads, st, pred, write, n, tile, count_dev,
+                     count_host);
+  } else {
+    launch_dependent(tile_scan_kernel, 1, kScanThreads, st, tile, n_tiles, count_dev, count_host);
+    launch_dependent(tile_write_kernel<Pred, Write, false>, grid, kThreads, st, pred, write, n, tile, count_dev,
+                     count_host);
+  }
 }
 
 int ell_of(const ash_map* m, int j) {
@@ -698,19 +740,18 @@ ash_status ash_depth_to_block_keys(const float* depth, int32_t width, int32_t he
   int64_t* cnt = count_dev ? count_dev : reinterpret_cast<int64_t*>(scratch);
   int32_t* tile = reinterpret_cast<int32_t*>(scratch + 16);
   const Cam cam = ash::vol::cam_of(intrinsics_host, extrinsic_host);
-  ash::vol::compact(ash::vol::DepthValid{depth, depth_max},
-                    ash::vol::DepthKeyWrite{depth, cam, width, block_edge, keys}, n, tile, cnt, st,
-                    ash::kKDepthKeys);
-  ash_status s = check_launch("depth_to_block_keys");
+  int64_t* pin = count_host ? ash::vol::pinned_count() : nullptr;
+  ash_status s = count_host && !pin ? fail(ASH_ERR_OOM, "pinned allocation failed") : ASH_OK;
+  if (s == ASH_OK) {
+    ash::vol::compact(ash::vol::DepthValid{depth, depth_max},
+                      ash::vol::DepthKeyWrite{depth, cam, width, block_edge, keys}, n, tile, cnt, pin, st,
+                      ash::kKDepthKeys);
+    s = check_launch("depth_to_block_keys");
+  }
   if (s == ASH_OK && count_host) {
-    int64_t* pin = ash::vol::pinned_count();
-    if (!pin) s = fail(ASH_ERR_OOM, "pinned allocation failed");
-    if (s == ASH_OK) {
-      cudaMemcpyAsync(pin, cnt, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
-      const cudaError_t e = cudaStreamSynchronize(st);
-      if (e != cudaSuccess) s = cuda_fail(e, "depth_to_block_keys");
-      else *count_host = *pin;
-    }
+    const cudaError_t e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) s = cuda_fail(e, "depth_to_block_keys");
+    else *count_host = *pin;
   }
   cudaFreeAsync(scratch, st);
   return s;
@@ -745,31 +786,36 @@ ash_status ash_double_map_activate(ash_map* local, ash_map* global, const int32_
   // 1. local activate
   s = ash_activate(local, keys, n, idx_all, mask_all, stream);
   // 2. the frame's distinct new keys, in input order
+  int64_t* pin = ash::vol::pinned_count();
+  if (s == ASH_OK && !pin) s = fail(ASH_ERR_OOM, "pinned allocation failed");
   if (s == ASH_OK) {
     ash::vol::compact(ash::vol::MaskSet{mask_all},
                       ash::vol::UniqueWrite{keys, idx_all, local->key_dim, unique_keys, local_indices}, n, tile, cnt,
-                      st, ash::kKCompact);
+                      pin, st, ash::kKCompact);
     s = check_launch("double_map_activate");
   }
   if (s == ASH_OK) {
-    int64_t* pin = ash::vol::pinned_count();
-    if (!pin) s = fail(ASH_ERR_OOM, "pinned allocation failed");
-    if (s == ASH_OK) {
-      cudaMemcpyAsync(pin, cnt, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
-      const cudaError_t e = cudaStreamSynchronize(st);
-      if (e != cudaSuccess) s = cuda_fail(e, "double_map_activate");
-      else u = *pin;
-    }
+    const cudaError_t e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) s = cuda_fail(e, "double_map_activate");
+    else u = *pin;
   }
   // 3. global activate + find; 4. local values := global indices
   if (s == ASH_OK && u > 0) {
     s = ash_activate(global, unique_keys, u, global_indices, mask_all, stream);
-    if (s == ASH_OK) s = ash_find(global, unique_keys, u, global_indices, mask_all, stream);
-    if (s == ASH_OK) {
-      ash::TraceScope ts(ash::kKScatterRows, st);
-      ash::vol::scatter_index_kernel<<<grid_for(u, launch_of(local, st)), ash::vol::kThreads, 0, st>>>(
-          static_cast<int32_t*>(local->vb[0]), local_indices, global_indices, u);
+    if (s == ASH_OK && global->tuning.warp_probe == 0 && partition_log(global, u) == 0) {
+      // in one kernel: the lookup's thread links the local entry
+      global->last_stream = st;
+      global->K.find_link(global->S, view_of(global), unique_keys, u, global_indices,
+                          static_cast<int32_t*>(local->vb[0]), local_indices, launch_of(global, st));
       s = check_launch("double_map_activate");
+    } else if (s == ASH_OK) {
+      s = ash_find(global, unique_keys, u, global_indices, mask_all, stream);
+      if (s == ASH_OK) {
+        ash::TraceScope ts(ash::kKScatterRows, st);
+        ash::launch_dependent(ash::vol::scatter_index_kernel, grid_for(u, launch_of(local, st)), ash::vol::kThreads, st,
+                              static_cast<int32_t*>(local->vb[0]), local_indices, global_indices, u);
+        s = check_launch("double_map_activate");
+      }
     }
   }
   cudaFreeAsync(scratch, st);
@@ -802,13 +848,13 @@ ash_status ash_tsdf_integrate(ash_map* blocks, int tsdf_buffer, int weight_buffe
   const int32_t cap = static_cast<int32_t>(blocks->capacity);
   ash::TraceScope ts(ash::kKIntegrate, st);
   if (ell == 8)
-    ash::vol::integrate_kernel<8><<<static_cast<unsigned>(n_blocks), ash::vol::kThreads, 0, st>>>(
-        blocks->kb, blocks->ks, cap, block_indices, tsdf, weight, depth, width, height, cam, voxel_size, trunc,
-        depth_max);
+    ash::launch_dependent(ash::vol::integrate_kernel<8>, static_cast<int>(n_blocks), ash::vol::kThreads, st,
+                          blocks->kb, blocks->ks, cap, block_indices, tsdf, weight, depth, width, height, cam,
+                          voxel_size, trunc, depth_max);
   else
-    ash::vol::integrate_kernel<16><<<static_cast<unsigned>(n_blocks), ash::vol::kThreads, 0, st>>>(
-        blocks->kb, blocks->ks, cap, block_indices, tsdf, weight, depth, width, height, cam, voxel_size, trunc,
-        depth_max);
+    ash::launch_dependent(ash::vol::integrate_kernel<16>, static_cast<int>(n_blocks), ash::vol::kThreads, st,
+                          blocks->kb, blocks->ks, cap, block_indices, tsdf, weight, depth, width, height, cam,
+                          voxel_size, trunc, depth_max);
   return check_launch("tsdf_integrate");
 }
 
