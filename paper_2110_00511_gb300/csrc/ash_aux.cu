@@ -287,6 +287,20 @@ __global__ void snapshot_kernel(Ctrl* ctrl, Snap* snap, uint32_t seq) {
   if (threadIdx.x == 0) publish_snapshot(ctrl, snap, seq);
 }
 
+// The control block to its pinned mirror, by stores of the SM: a synchronising
+// read waits for this launch instead of a copy engine's 32 bytes.
+__global__ void read_ctrl_kernel(const unsigned long long* __restrict__ ctrl, unsigned long long* host) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (threadIdx.x < sizeof(Ctrl) / 8) host[threadIdx.x] = ctrl[threadIdx.x];
+}
+
+void launch_read_ctrl(const Ctrl* ctrl, Ctrl* host, const Launch& L) {
+  static_assert(sizeof(Ctrl) % 8 == 0, "copied by 8-byte words");
+  TraceScope ts(kKSetCtrl, L.stream);
+  launch_dependent(read_ctrl_kernel, 1, 32, L.stream, reinterpret_cast<const unsigned long long*>(ctrl),
+                   reinterpret_cast<unsigned long long*>(host));
+}
+
 void launch_snapshot(Ctrl* ctrl, Snap* snap, uint32_t seq, const Launch& L) {
   TraceScope ts(kKSetCtrl, L.stream);
   launch_dependent(snapshot_kernel, 1, 32, L.stream, ctrl, snap, seq);

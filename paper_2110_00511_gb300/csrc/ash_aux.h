@@ -52,6 +52,8 @@ struct InitPlan {
   void word(void* dst, uint64_t v) { add(kWord, dst, nullptr, v, 8); }
 };
 void launch_init(const InitPlan& plan, const Launch& L);
+// Copies the control block to its pinned mirror.
+void launch_read_ctrl(const Ctrl* ctrl, Ctrl* host, const Launch& L);
 // Publishes the control block to a host-visible snapshot (publish_snapshot).
 void launch_snapshot(Ctrl* ctrl, Snap* snap, uint32_t seq, const Launch& L);
 // Value rows of an insert's winners (idx[p] >= 0): dst_j row idx[p] <- src_j row p.

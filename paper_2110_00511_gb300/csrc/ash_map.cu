@@ -374,7 +374,9 @@ int64_t slots_for(int64_t capacity, const ash_tuning& t) {
 // Reads the control block (synchronises `st`).
 ash_status refresh(ash_map* m, cudaStream_t st, int64_t* top, int64_t* used, int* status) {
   __atomic_fetch_add(&m->host_syncs, 1, __ATOMIC_RELAXED);  // read by other threads as a statistic
-  ASH_CUDA(cudaMemcpyAsync(m->ctrl_host, m->ctrl, sizeof(ash::Ctrl), cudaMemcpyDeviceToHost, st));
+  ash::launch_read_ctrl(m->ctrl, m->ctrl_host, launch_of(m, st));
+  ash_status s = check_launch("control block read");
+  if (s != ASH_OK) return s;
   ASH_CUDA(cudaStreamSynchronize(st));
   const unsigned long long tu = m->ctrl_host->top_used;
   *top = static_cast<int64_t>(tu & 0xFFFFFFFFull);
