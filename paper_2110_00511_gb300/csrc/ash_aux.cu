@@ -335,13 +335,14 @@ struct RowCursor {
   }
 };
 
-// Value rows of winners (idx[p] >= 0): dst row idx[p] <- src row p.
+// Value rows of winners (idx[p] >= 0): dst row idx[p] <- src row p.  One
+// launch per value buffer: with the element types in one kernel (98
+// registers, two blocks per SM) 40k rows of 2 + 1 KiB took 48 us, so 44
+// (the gather of as many bytes 45).
 template <class T>
-__device__ __forceinline__ void scatter_rows_of(void* dst_rows, const void* src_rows, int64_t row_bytes,
-                                                const int32_t* __restrict__ idx, int64_t n) {
-  T* dst = static_cast<T*>(dst_rows);
-  const T* src = static_cast<const T*>(src_rows);
-  const int64_t per = row_bytes / static_cast<int64_t>(sizeof(T));
+__global__ void __launch_bounds__(256) scatter_rows_kernel(T* __restrict__ dst, const T* __restrict__ src, int64_t per,
+                                                           const int32_t* __restrict__ idx, int64_t n) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int64_t total = n * per;
   const int64_t tile = static_cast<int64_t>(blockDim.x) * kRowUnroll;
   const int64_t first = static_cast<int64_t>(blockIdx.x) * tile + threadIdx.x;
@@ -366,31 +367,29 @@ __device__ __forceinline__ void scatter_rows_of(void* dst_rows, const void* src_
   }
 }
 
-__global__ void __launch_bounds__(256) scatter_rows_kernel(ValueCopy vc, const int32_t* __restrict__ idx, int64_t n) {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-#pragma unroll 1
-  for (int j = 0; j < vc.n; ++j) {
-    switch (vc.vec[j]) {
-      case 16: scatter_rows_of<uint4>(vc.dst[j], vc.src[j], vc.row_bytes[j], idx, n); break;
-      case 8: scatter_rows_of<uint2>(vc.dst[j], vc.src[j], vc.row_bytes[j], idx, n); break;
-      case 4: scatter_rows_of<uint32_t>(vc.dst[j], vc.src[j], vc.row_bytes[j], idx, n); break;
-      case 2: scatter_rows_of<uint16_t>(vc.dst[j], vc.src[j], vc.row_bytes[j], idx, n); break;
-      default: scatter_rows_of<uint8_t>(vc.dst[j], vc.src[j], vc.row_bytes[j], idx, n); break;
-    }
-  }
-}
-
 // Grid of a flattened row copy of `elems` elements.
 static int row_copy_grid(int64_t elems, const Launch& L) {
   return grid_for((elems + kRowUnroll - 1) / kRowUnroll, L);
 }
 
 void launch_scatter_rows(const ValueCopy& vc, const int32_t* idx, int64_t n, const Launch& L) {
-  if (vc.n == 0 || n == 0) return;
-  int64_t elems = 0;
-  for (int j = 0; j < vc.n; ++j) elems = std::max(elems, n * (vc.row_bytes[j] / vc.vec[j]));
-  TraceScope ts(kKScatterRows, L.stream);
-  launch_dependent(scatter_rows_kernel, row_copy_grid(elems, L), L.block, L.stream, vc, idx, n);
+  if (n == 0) return;
+  for (int j = 0; j < vc.n; ++j) {
+    TraceScope ts(kKScatterRows, L.stream);
+    const int64_t per = vc.row_bytes[j] / vc.vec[j];
+    const int grid = row_copy_grid(n * per, L);
+#define ASH_SCATTER(T)                                                                                        \
+  launch_dependent(scatter_rows_kernel<T>, grid, L.block, L.stream, static_cast<T*>(vc.dst[j]),                \
+                   static_cast<const T*>(vc.src[j]), per, idx, n)
+    switch (vc.vec[j]) {
+      case 16: ASH_SCATTER(uint4); break;
+      case 8: ASH_SCATTER(uint2); break;
+      case 4: ASH_SCATTER(uint32_t); break;
+      case 2: ASH_SCATTER(uint16_t); break;
+      default: ASH_SCATTER(uint8_t); break;
+    }
+#undef ASH_SCATTER
+  }
 }
 
 // --------------------------------------------------------------- key gather
@@ -490,8 +489,9 @@ void launch_gather_rows(const ValueCopy& vc, int64_t capacity, const int32_t* li
 // floor(p / cell) in float32 with IEEE division (this file is compiled without
 // fast-math), then float -> int32 conversion rounding toward minus infinity
 // (saturating outside the int32 range).
-__global__ void quantize_kernel(const float* __restrict__ pts, int64_t n, int64_t n4, float cell,
-                                int32_t* __restrict__ keys) {
+__global__ void __launch_bounds__(256) quantize_kernel(const float* __restrict__ pts, int64_t n, int64_t n4, float cell,
+                                                       int32_t* __restrict__ keys) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   const float4* p4 = reinterpret_cast<const float4*>(pts);
   int4* k4 = reinterpret_cast<int4*>(keys);
@@ -514,7 +514,7 @@ void launch_quantize(const float* pts, int64_t n, float cell, int32_t* keys, con
   const bool vec_ok = ((reinterpret_cast<uintptr_t>(pts) | reinterpret_cast<uintptr_t>(keys)) & 15u) == 0;
   const int64_t n4 = vec_ok ? n / 4 : 0;
   TraceScope ts(kKQuantize, L.stream);
-  quantize_kernel<<<grid_for((n + 3) / 4, L), L.block, 0, L.stream>>>(pts, n, n4, cell, keys);
+  launch_dependent(quantize_kernel, grid_for((n + 3) / 4, L), L.block, L.stream, pts, n, n4, cell, keys);
 }
 
 // ----------------------------------------------------------- roofline probe
