@@ -928,12 +928,24 @@ __global__ void __launch_bounds__(256, S == 4 && D <= 4 ? 6 : 1) claim_pref_kern
       fp[q] = fingerprint(h);
       ps[q] = home_bucket(h, t.n_buckets) * S + pref_slot<S>(fp[q]);
     }
+    // A key equal to the one before it has lost to it, whatever becomes of
+    // that one: points in scan order come in such runs, and without this all
+    // of a run meet in one slot (block keys of a depth frame, 307k in 2k
+    // blocks: 12.6 -> 7.0 us; random keys level).
+    bool follows[KPT];
+#pragma unroll
+    for (int q = 0; q < KPT; ++q) {
+      bool same = lane > 0;
+#pragma unroll
+      for (int j = 0; j < D; ++j) same &= __shfl_up_sync(0xFFFFFFFFu, k[q][j], 1) == k[q][j];
+      follows[q] = same;
+    }
     uint64_t old[KPT];
 #pragma unroll
     for (int q = 0; q < KPT; ++q) {
       const int64_t pos = wbase + q * 32 + lane;
       old[q] = kTombstone;
-      if (pos < n) {
+      if (pos < n && !follows[q]) {
         const uint64_t mine = (static_cast<uint64_t>(fp[q]) << 32) | (kClaimBit | static_cast<uint32_t>(pos));
         old[q] = atomicCAS(reinterpret_cast<unsigned long long*>(t.slots + ps[q]),
                            static_cast<unsigned long long>(kEmpty), static_cast<unsigned long long>(mine));
@@ -968,7 +980,9 @@ __global__ void __launch_bounds__(256, S == 4 && D <= 4 ? 6 : 1) claim_pref_kern
         bool eq = fm[q];
 #pragma unroll
         for (int j = 0; j < D; ++j) eq &= (row[q][j] == k[q][j]);
-        if (old[q] == kEmpty) {
+        if (follows[q]) {
+          slot_out[pos] = kClaimJoined;
+        } else if (old[q] == kEmpty) {
           slot_out[pos] = static_cast<int32_t>(ps[q]);
         } else if (!eq) {
           pending = true;
