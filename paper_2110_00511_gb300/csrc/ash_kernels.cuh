@@ -852,10 +852,14 @@ __device__ __forceinline__ void claim_slow_round(const TableView& t, const In& k
 // queued per warp and claimed 32 at a time: though 2 % of the keys, most
 // warps have one, and running the protocol for it at once cost more than all
 // its other keys' CASes (GB300, 10^8 keys by ranges: activate and find 9.18 ->
-// 8.56 ms).  The better choice when the table does not stay in L2: the loads bring the buckets in with deep miss queues
-// and the CASes then hit L2.  Slot order does not keep the preferred-slot
-// invariant (preferred-first placement measured 5-10 % slower here), so the
-// host clears the map's flag.
+// 8.56 ms).  The better choice when the table does not stay in L2: the loads
+// bring the buckets in with deep miss queues and the CASes then hit L2.  Input
+// order takes as many blocks as are resident at once: 10^7 claims 345 -> 322
+// us without the thin second wave of eight blocks per SM; the calls of a
+// ranged batch keep the larger grid (10^8 keys, activate and find, with five
+// resident blocks of 48 registers: 7.55 -> 7.82 ms).  Slot order does
+// not keep the preferred-slot invariant (preferred-first placement measured
+// 5-10 % slower here), so the host clears the map's flag.
 template <int D, int S, int KPT, class In = const int32_t*>
 __global__ void __launch_bounds__(256) claim_bucket_kernel(TableView t, const In keys, int64_t n,
                                                            int32_t* __restrict__ slot_out) {
@@ -1802,9 +1806,8 @@ struct DimLaunchers {
       auto* k = claim_pref_kernel<D, S, 1, In>;
       launch_dependent(k, resident_grid(k, grid_for(n, L), L), L.block, L.stream, t, keys, n, slot_out);
     } else {
-      // (capping this grid at its 4 resident blocks per SM measured 10-15 %
-      // slower on 1e7-key tables)
-      launch_dependent(claim_bucket_kernel<D, S, KPT, In>, g, L.block, L.stream, t, keys, n, slot_out);
+      auto* k = claim_bucket_kernel<D, S, KPT, In>;
+      launch_dependent(k, resident_grid(k, g, L), L.block, L.stream, t, keys, n, slot_out);
     }
   }
   template <int S, class In>
