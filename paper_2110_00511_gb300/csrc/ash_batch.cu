@@ -17,6 +17,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstddef>
 #include <cstring>
 #include <mutex>
 #include <vector>
@@ -58,13 +59,20 @@ struct BatchSnap {
   uint32_t seq;
 };
 
-struct BatchTable {
+struct alignas(16) BatchTable {
   BatchPhase ph[kPhases];
   int32_t n_ops;
   int32_t n_snaps;
   BatchSnap snaps[kBatchMaxOps];
   BatchOp ops[kBatchMaxOps];  // last: only the part in use is copied
 };
+
+// 16-byte units of the table's part in use; the last may reach past it, so the
+// table's size is a multiple of 16.
+constexpr int upload_units(int n_ops) {
+  return static_cast<int>((offsetof(BatchTable, ops) + sizeof(BatchOp) * n_ops + 15) / 16);
+}
+static_assert(upload_units(kBatchMaxOps) * 16 <= sizeof(BatchTable), "a full batch is uploaded within its table");
 
 // Copies the table's part in use from pinned host memory (the SMs read it
 // over the CPU-GPU link).
@@ -261,7 +269,7 @@ void launch_batch(const ash_batch* b, const ash_batch::Slot& s, cudaStream_t st)
     const int64_t tiles = tb->ph[phase].tiles;
     return static_cast<int>(tiles < b->grid ? tiles : b->grid);
   };
-  const int units = static_cast<int>((offsetof(BatchTable, ops) + sizeof(BatchOp) * tb->n_ops + 15) / 16);
+  const int units = upload_units(tb->n_ops);
   launch_dependent(batch_upload_kernel, (units + 1023) / 1024, 1024, st, reinterpret_cast<const uint4*>(s.h),
                    reinterpret_cast<uint4*>(s.d), units);
   if (tb->ph[kPhaseInsert].tiles > 0) {
