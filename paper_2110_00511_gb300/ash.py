@@ -211,8 +211,16 @@ def _stream_of(device_index):
 
 
 def _stream(device=None):
-    """The same for a torch.device, an index or None (the current device)."""
-    index = device if isinstance(device, int) else getattr(device, "index", None)
+    """The same for a torch.device, an index or None (the current device).  The
+    functions below take their stream from a tensor's device, so a tensor that
+    is not on a GPU is refused here, before its address reaches a kernel."""
+    if device is None or isinstance(device, int):
+        index = device
+    else:
+        device = torch.device(device)
+        if device.type != "cuda":
+            raise ValueError(f"expected a tensor or device of type cuda, got {device}")
+        index = device.index
     return _stream_of(torch.cuda.current_device() if index is None else index)
 
 
