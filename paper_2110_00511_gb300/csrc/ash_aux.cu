@@ -46,8 +46,8 @@ __global__ void __launch_bounds__(256) partition_scan_kernel(uint32_t* __restric
   if (threadIdx.x == 0) range_totals[blockIdx.x] = static_cast<uint32_t>(total);
 }
 
-void launch_partition_scan(uint32_t* counts, int G, int P, uint32_t* range_totals, const Launch& L) {
-  launch_dependent(partition_scan_kernel, P, 256, L.stream, counts, G, range_totals);
+cudaError_t launch_partition_scan(uint32_t* counts, int G, int P, uint32_t* range_totals, const Launch& L) {
+  return launch_dependent(partition_scan_kernel, P, 256, L.stream, counts, G, range_totals);
 }
 
 // Eight positions per thread: the dest loads, then the gathers, then the

@@ -116,6 +116,16 @@ Launch launch_of(const ash_map* m, cudaStream_t st);
 TableView view_of(const ash_map* m);
 // log2 of the home-bucket ranges that a call on n keys is partitioned into (0: input order).
 int partition_log(const ash_map* m, int64_t n);
+// Stream-ordered scratch of one partitioned call, freed on the same stream
+// after its last kernel (concurrent finds on one map each have their own).
+struct PartBufs {
+  void* mem = nullptr;
+  int32_t* keys = nullptr;  // key rows in range order
+  int32_t* dest = nullptr;  // place of input row pos in that order
+  int32_t* idx = nullptr;   // outputs in range order
+  uint8_t* mask = nullptr;
+};
+bool partition_call(ash_map* m, const int32_t* keys, int64_t n, int log_p, cudaStream_t st, PartBufs* pb);
 ash_status check_keys(const ash_map* m, const void* keys, int64_t n);
 // x2 growth / table rebuild so that a batch of n insert keys fits (may synchronise st).
 ash_status ensure_room(ash_map* m, int64_t n, cudaStream_t st);

@@ -1659,9 +1659,11 @@ struct Launch {
 // scheduled while the previous kernel on the stream drains, hiding the
 // launch latency between the two.  The kernel must execute
 // griddepcontrol.wait before it touches memory the previous kernel writes.
+// The result also stays behind as the last error, which the calls check at
+// their end (check_launch).
 template <class... P, class... A>
-inline void launch_dependent_smem(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t st,
-                                  A... args) {
+inline cudaError_t launch_dependent_smem(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t st,
+                                         A... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(grid));
   cfg.blockDim = dim3(static_cast<unsigned>(block));
@@ -1672,12 +1674,12 @@ inline void launch_dependent_smem(void (*kernel)(P...), int grid, int block, siz
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
 template <class... P, class... A>
-inline void launch_dependent(void (*kernel)(P...), int grid, int block, cudaStream_t st, A... args) {
-  launch_dependent_smem(kernel, grid, block, 0, st, args...);
+inline cudaError_t launch_dependent(void (*kernel)(P...), int grid, int block, cudaStream_t st, A... args) {
+  return launch_dependent_smem(kernel, grid, block, 0, st, args...);
 }
 
 // Blocks of `kernel` (block threads `block`, no dynamic shared memory) that
@@ -1714,7 +1716,7 @@ inline int grid_for(int64_t n, const Launch& L) {
 // Defined in ash_aux.cu.  Per range (one block each): the row of per-block
 // counts counts[p][0..G) becomes its exclusive scan, the row's total goes to
 // range_totals[p].
-void launch_partition_scan(uint32_t* counts, int G, int P, uint32_t* range_totals, const Launch& L);
+cudaError_t launch_partition_scan(uint32_t* counts, int G, int P, uint32_t* range_totals, const Launch& L);
 // idx[pos] = idx_p[dest[pos]], mask[pos] = idx[pos] >= 0: a partitioned call's
 // outputs back in input order.
 void launch_unpermute(const int32_t* dest, int64_t n, const int32_t* idx_p, int32_t* idx, uint8_t* mask,
@@ -1754,8 +1756,8 @@ struct DimKernels {
   void (*find_link)(int S, const TableView&, const int32_t*, int64_t, int32_t*, int32_t*, const int32_t*,
                     const Launch&);
   void (*find_group)(int S, const TableView&, const int32_t*, int64_t, int32_t*, uint8_t*, const Launch&);
-  // stable partition of n key rows by home-bucket range (scratch: see partition_bytes)
-  void (*partition)(const int32_t*, int64_t, int, uint32_t*, uint8_t*, int32_t*, int32_t*, const Launch&);
+  // stable partition of n key rows by home-bucket range; false: it was not enqueued whole
+  bool (*partition)(const int32_t*, int64_t, int, uint32_t*, uint8_t*, int32_t*, int32_t*, const Launch&);
   // the same operations on float32 points quantised in the kernels
   void (*find_pts)(int S, int kpt, const TableView&, const PointRows&, int64_t, int32_t*, uint8_t*, const Launch&);
   void (*claim_pts)(int S, int kpt, int pref, const TableView&, const PointRows&, int64_t, int32_t*, const Launch&);
@@ -1939,26 +1941,32 @@ struct DimLaunchers {
     else find_group_s<16>(t, keys, n, idx, mask, L);
   }
   // counts: partition_count_words(n, log_p, L) words; ranges: n bytes;
-  // keys_out: n rows; dest: n.
-  static void partition(const int32_t* keys, int64_t n, int log_p, uint32_t* counts, uint8_t* ranges,
+  // keys_out: n rows; dest: n.  False when the device refuses a step (its
+  // opt-in to the scatter's shared memory, or a launch): the outputs are then
+  // not to be used.
+  static bool partition(const int32_t* keys, int64_t n, int log_p, uint32_t* counts, uint8_t* ranges,
                         int32_t* keys_out, int32_t* dest, const Launch& L) {
-    TraceScope ts(kKPartition, L.stream, 3);
     int tpb = 0;
     const int G = partition_grid(n, L, &tpb);
     const int P = 1 << log_p;
     uint32_t* range_totals = counts + static_cast<int64_t>(P) * G;
-    launch_dependent(partition_count_kernel<D>, G, kCountThreads, L.stream, keys, n, log_p, tpb, counts, ranges);
-    launch_partition_scan(counts, G, P, range_totals, L);
-    static bool attr_set = false;  // per key dimension; above 48 KB the kernel must opt in
-    if (!attr_set) {
-      cudaFuncSetAttribute(partition_scatter_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(partition_scatter_smem<D>(1 << kPartMaxLog)));
-      attr_set = true;
-    }
-    launch_dependent_smem(partition_scatter_kernel<D>, G, kScatterThreads, partition_scatter_smem<D>(P), L.stream, keys,
-                          static_cast<const uint8_t*>(ranges), n, log_p, tpb,
-                          static_cast<const uint32_t*>(counts), static_cast<const uint32_t*>(range_totals), keys_out,
-                          dest);
+    // Above 48 KB with the static arrays (4 dimensions with 256 ranges, or 5
+    // and more) the kernel must opt in, on each device.  The call is cheap
+    // beside the 10^6 keys that a ranged call has, so nothing is remembered;
+    // always the dimension's most, so that concurrent calls ask for the same.
+    const size_t smem = partition_scatter_smem<D>(P);
+    if (smem > 44 * 1024 && cudaFuncSetAttribute(partition_scatter_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 static_cast<int>(partition_scatter_smem<D>(1 << kPartMaxLog))) !=
+                                cudaSuccess)
+      return false;
+    TraceScope ts(kKPartition, L.stream, 3);
+    return launch_dependent(partition_count_kernel<D>, G, kCountThreads, L.stream, keys, n, log_p, tpb, counts,
+                            ranges) == cudaSuccess &&
+           launch_partition_scan(counts, G, P, range_totals, L) == cudaSuccess &&
+           launch_dependent_smem(partition_scatter_kernel<D>, G, kScatterThreads, smem, L.stream, keys,
+                                 static_cast<const uint8_t*>(ranges), n, log_p, tpb,
+                                 static_cast<const uint32_t*>(counts), static_cast<const uint32_t*>(range_totals),
+                                 keys_out, dest) == cudaSuccess;
   }
   static DimKernels table() {
     DimKernels k;

@@ -271,18 +271,9 @@ int partition_log(const ash_map* m, int64_t n) {
   return mode == 2 ? std::max(lg, 3) : lg;
 }
 
-// Stream-ordered scratch of one partitioned call, freed on the same stream
-// after its last kernel (concurrent finds on one map each have their own).
-struct PartBufs {
-  void* mem = nullptr;
-  int32_t* keys = nullptr;  // key rows in range order
-  int32_t* dest = nullptr;  // place of input row pos in that order
-  int32_t* idx = nullptr;   // outputs in range order
-  uint8_t* mask = nullptr;
-};
-
-// False (nothing enqueued) when the scratch cannot be had: the call then
-// uses its keys in input order.
+// False when the scratch cannot be had or the device refuses a step of the
+// partition: the call then uses its keys in input order (what was enqueued
+// only touches the scratch, which is freed behind it).
 bool partition_call(ash_map* m, const int32_t* keys, int64_t n, int log_p, cudaStream_t st, PartBufs* pb) {
   auto up = [](int64_t b) { return (b + 255) / 256 * 256; };
   const int64_t words = up(ash::partition_count_words(n, log_p, launch_of(m, st)) * 4);
@@ -299,8 +290,12 @@ bool partition_call(ash_map* m, const int32_t* keys, int64_t n, int log_p, cudaS
   pb->idx = reinterpret_cast<int32_t*>(base + words + rows + ints);
   pb->mask = reinterpret_cast<uint8_t*>(base + words + rows + 2 * ints);
   // the masks' bytes hold the keys' ranges until the scatter has read them
-  m->K.partition(keys, n, log_p, reinterpret_cast<uint32_t*>(base), pb->mask, pb->keys, pb->dest, launch_of(m, st));
-  return true;
+  if (m->K.partition(keys, n, log_p, reinterpret_cast<uint32_t*>(base), pb->mask, pb->keys, pb->dest, launch_of(m, st)))
+    return true;
+  cudaGetLastError();
+  dev_free(m, base, st);
+  pb->mem = nullptr;
+  return false;
 }
 
 // The partitioned call's outputs back in input order; its scratch freed.
