@@ -574,7 +574,9 @@ constexpr int kClaimPrefFirst = 2;
 // bucket with an EMPTY slot, where the key is known to be absent; 3) the key
 // takes the first TOMBSTONE of the buckets without an EMPTY slot that it
 // walked past, else an EMPTY slot of the last bucket.  A lost CAS compares
-// with the winner's word and starts the walk again.
+// with the winner's word and starts the walk again.  A walk that meets no
+// EMPTY slot within max_probes buckets fails even past a tombstone: when
+// max_probes was lowered on a filled map, the key may sit further along.
 //
 // Equal keys of one batch cannot take two slots.  A slot only goes from free
 // (EMPTY or TOMBSTONE, and of one kind while it is free) to taken during an
@@ -657,8 +659,7 @@ __device__ __forceinline__ int32_t claim_key(const TableView& t, const In& keys,
       if (tomb == kNoIndex && tombs) tomb = b * S + __ffs(tombs) - 1;
       b = next_bucket(b, t.n_buckets);
       ++probe;
-      if (probe < t.max_probes || tomb == kNoIndex) continue;
-      // no EMPTY slot within max_probes buckets, but a tombstone
+      continue;
     }
     uint32_t slot = tomb;
     uint64_t free_word = kTombstone;
