@@ -463,7 +463,7 @@ ash_status ash_batch_run(ash_batch* b, const ash_batch_op* ops, int n_ops, ash_s
     snapped.push_back(m);
     tb->snaps[tb->n_snaps++] = {m->ctrl, m->snap_dev, m->snap_seq};
   }
-  if (k > 0) {
+  if (k > 0 || tb->n_snaps > 0) {  // snapshots that were numbered have to be published, work or not
     TraceScope ts(kKBatch, st, 7);
     if (wide) launch_batch<true>(b, sl, st);
     else launch_batch<false>(b, sl, st);
