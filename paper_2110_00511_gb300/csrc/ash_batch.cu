@@ -261,6 +261,11 @@ struct ash_batch {
 namespace {
 
 // The batch's kernels on st, empty phases left out.
+int batch_launches(const BatchTable& tb) {
+  return 1 + (tb.ph[kPhaseInsert].tiles > 0 ? 2 : 0) + (tb.ph[kPhaseFind].tiles > 0 ? 1 : 0) +
+         (tb.ph[kPhaseErase].tiles > 0 ? 2 : 0) + (tb.n_snaps > 0 ? 1 : 0);
+}
+
 template <bool WIDE>
 void launch_batch(const ash_batch* b, const ash_batch::Slot& s, cudaStream_t st) {
   const BatchTable* tb = s.h;
@@ -464,7 +469,7 @@ ash_status ash_batch_run(ash_batch* b, const ash_batch_op* ops, int n_ops, ash_s
     tb->snaps[tb->n_snaps++] = {m->ctrl, m->snap_dev, m->snap_seq};
   }
   if (k > 0 || tb->n_snaps > 0) {  // snapshots that were numbered have to be published, work or not
-    TraceScope ts(kKBatch, st, 7);
+    TraceScope ts(kKBatch, st, batch_launches(*tb));
     if (wide) launch_batch<true>(b, sl, st);
     else launch_batch<false>(b, sl, st);
     ash_status s = check_launch("batch_run");
