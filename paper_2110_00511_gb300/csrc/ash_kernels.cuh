@@ -42,6 +42,8 @@
 //                 of the probe sequence, no key comparisons.
 #pragma once
 
+#include <atomic>
+
 #include "ash_device.cuh"
 #include "ash_trace.h"
 
@@ -1654,6 +1656,7 @@ struct Launch {
   int grid_cap;  // SMs x blocks_per_sm
   int block;
   int sms = 0;   // SM count (0: unknown)
+  bool one_wave = true;  // resident_grid holds a grid to the blocks that fit at once
 };
 
 // Launch with programmatic stream serialisation: the kernel's blocks may be
@@ -1683,28 +1686,31 @@ inline cudaError_t launch_dependent(void (*kernel)(P...), int grid, int block, c
   return launch_dependent_smem(kernel, grid, block, 0, st, args...);
 }
 
-// Blocks of `kernel` (block threads `block`, no dynamic shared memory) that
-// fit on one SM, from the occupancy API, cached per kernel and block size.
-template <class K>
-inline int resident_blocks(K kernel, int block) {
-  static int cache[9] = {};  // block / 32 in 1..8
+// Blocks of Kernel (block threads `block`, no dynamic shared memory) that fit
+// on one SM, from the occupancy API.  The kernel is a template argument, so
+// each has a cache of its own: kernels of one signature differ in registers,
+// and who was called first must not set the others' grids.  (One architecture
+// is built, so the answer is the same on every device.)
+template <auto Kernel>
+inline int resident_blocks(int block) {
+  static std::atomic<int> cache[9] = {};  // block / 32 in 1..8
   const int slot = block / 32;
   if (slot < 1 || slot > 8) return 1;
-  if (cache[slot] == 0) {
-    int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, block, 0) != cudaSuccess || nb < 1) nb = 1;
-    cache[slot] = nb;
+  int nb = cache[slot].load(std::memory_order_relaxed);
+  if (nb == 0) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, Kernel, block, 0) != cudaSuccess || nb < 1) nb = 1;
+    cache[slot].store(nb, std::memory_order_relaxed);
   }
-  return cache[slot];
+  return nb;
 }
 
 // Grid of a grid-stride kernel whose registers allow fewer resident blocks
 // than the Launch's cap: no more blocks than fit at once, so no thin second
 // wave runs at low occupancy.
-template <class K>
-inline int resident_grid(K kernel, int want, const Launch& L) {
-  if (L.sms <= 0) return want;
-  const int cap = L.sms * resident_blocks(kernel, L.block);
+template <auto Kernel>
+inline int resident_grid(int want, const Launch& L) {
+  if (!L.one_wave || L.sms <= 0) return want;
+  const int cap = L.sms * resident_blocks<Kernel>(L.block);
   return want < cap ? want : cap;
 }
 
@@ -1806,11 +1812,11 @@ struct DimLaunchers {
     TraceScope ts(kKClaim, L.stream);
     const int g = grid_for((n + KPT - 1) / KPT, L);
     if (pref) {
-      auto* k = claim_pref_kernel<D, S, 1, In>;
-      launch_dependent(k, resident_grid(k, grid_for(n, L), L), L.block, L.stream, t, keys, n, slot_out);
+      constexpr auto k = claim_pref_kernel<D, S, 1, In>;
+      launch_dependent(k, resident_grid<k>(grid_for(n, L), L), L.block, L.stream, t, keys, n, slot_out);
     } else {
-      auto* k = claim_bucket_kernel<D, S, KPT, In>;
-      launch_dependent(k, resident_grid(k, g, L), L.block, L.stream, t, keys, n, slot_out);
+      constexpr auto k = claim_bucket_kernel<D, S, KPT, In>;
+      launch_dependent(k, resident_grid<k>(g, L), L.block, L.stream, t, keys, n, slot_out);
     }
   }
   template <int S, class In>
@@ -1893,8 +1899,8 @@ struct DimLaunchers {
                           int32_t* idx, uint8_t* mask, const Launch& L) {
     TraceScope ts(kKNeighbors, L.stream);
     constexpr int U = kNeighborUnroll;
-    auto* k = neighbors_kernel<D, S, U, Off>;
-    launch_dependent(k, resident_grid(k, grid_for((n * n_off + U - 1) / U, L), L), L.block, L.stream, t, keys, n, off,
+    constexpr auto k = neighbors_kernel<D, S, U, Off>;
+    launch_dependent(k, resident_grid<k>(grid_for((n * n_off + U - 1) / U, L), L), L.block, L.stream, t, keys, n, off,
                      static_cast<uint32_t>(n_off), idx, mask);
   }
   template <class Off>

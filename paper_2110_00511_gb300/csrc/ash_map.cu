@@ -890,7 +890,7 @@ ash_status insert_impl(ash_map* m, const int32_t* keys, const void* const* value
       if (p != P - 1) tvp.snap = nullptr;  // the last commit publishes the control block
       const int32_t* sk = ckeys + a * m->key_dim;
       Launch Lr = L;
-      if (!pref) Lr.sms = 0;  // not held to the resident blocks (see claim_bucket_kernel)
+      Lr.one_wave = pref;  // the bucket-first claim takes the larger grid here (see claim_bucket_kernel)
       m->K.claim(m->S, kpt, pref, tvp, sk, b - a, cidx + a, Lr);
       m->K.commit(ckpt, tvp, sk, b - a, cidx + a, cmask + a, inline_value ? &vr : nullptr, L);
     }
