@@ -29,10 +29,10 @@ def test_no_key_is_stored_twice(dim, buckets, claim_mode):
     assert before["used_slots"] > before["live"]  # tombstones, in the home buckets of keys that stayed
     t.max_probes = 1
     hm.set_tuning(t)
-    again = kept[: n // 50].contiguous()
-    for part in again.split(100):
+    batch = ash.Batch()
+    for part in kept.split(400):
         if claim_mode is None:
-            (_, new), = ash.Batch().run([(hm, ash.ASH_OP_ACTIVATE, part.contiguous(), None)])
+            (_, new), = batch.run([(hm, ash.ASH_OP_ACTIVATE, part.contiguous(), None)])
         else:
             new = hm.activate(part.contiguous())[1]
         assert not new.any()
