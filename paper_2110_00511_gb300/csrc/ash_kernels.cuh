@@ -145,6 +145,12 @@ __device__ __forceinline__ void probe_round(const TableView& t, const int32_t (&
 // issue 495 instructions per warp and query at 12 active lanes of 32 (now
 // 270 at 19).  GB300: 6M finds, half absent, on 5M entries 161 -> 127 us; 4M
 // finds, all present, 72 -> 61 us.
+//
+// With several keys per lane only the home buckets are probed together.  A
+// second probe_round over all of them cost their registers twice over (3-D, 16
+// slots, two keys: 128 instead of 64): 8M finds, half absent, of two keys per
+// lane in 16-slot buckets 221 us, now 174 (178 before the lookups went on in
+// place); of four keys 244, now 183; 8-D, 16 slots, two keys 334, now 221.
 template <int D, int S, int KPT>
 __device__ __forceinline__ void find_keys(const TableView& t, const int32_t (&k)[KPT][D], const bool (&ok)[KPT],
                                           int32_t (&out)[KPT]) {
@@ -160,14 +166,40 @@ __device__ __forceinline__ void find_keys(const TableView& t, const int32_t (&k)
     out[q] = -1;
   }
   probe_round<D, S, KPT, true>(t, k, fp, b, go, out, rare);
-  for (uint32_t probe = 1; probe < t.max_probes; ++probe) {
-    bool any = false;
+  if constexpr (KPT == 1) {
+    for (uint32_t probe = 1; probe < t.max_probes && go[0]; ++probe) {
+      b[0] = next_bucket(b[0], t.n_buckets);
+      probe_round<D, S, 1, false>(t, k, fp, b, go, out, rare);
+    }
+  } else {
+    // a lane's unsettled keys one after the other, in one piece of code
+    while (true) {
+      int at = -1;
 #pragma unroll
-    for (int q = 0; q < KPT; ++q) any |= go[q];
-    if (!any) break;
+      for (int q = KPT - 1; q >= 0; --q) at = go[q] ? q : at;
+      if (at < 0) break;
+      int32_t k1[1][D], out1[1] = {-1};
+      uint32_t fp1[1] = {0u}, b1[1] = {0u};
+      bool go1[1] = {true};
 #pragma unroll
-    for (int q = 0; q < KPT; ++q) b[q] = next_bucket(b[q], t.n_buckets);
-    probe_round<D, S, KPT, false>(t, k, fp, b, go, out, rare);
+      for (int q = 0; q < KPT; ++q) {
+        if (q == at) {
+#pragma unroll
+          for (int j = 0; j < D; ++j) k1[0][j] = k[q][j];
+          fp1[0] = fp[q];
+          b1[0] = b[q];
+          go[q] = false;
+        }
+      }
+#pragma unroll 1
+      for (uint32_t probe = 1; probe < t.max_probes && go1[0]; ++probe) {
+        b1[0] = next_bucket(b1[0], t.n_buckets);
+        probe_round<D, S, 1, false>(t, k1, fp1, b1, go1, out1, rare);
+      }
+#pragma unroll
+      for (int q = 0; q < KPT; ++q)
+        if (q == at) out[q] = out1[0];
+    }
   }
   if (rare) {
 #pragma unroll
@@ -391,10 +423,24 @@ __global__ void __launch_bounds__(256) neighbors_kernel(TableView t, const int32
   while (list.n > 0) list.template round<S>(t, idx, mask);
 }
 
+// Resident blocks that the find is compiled for, 0 where the compiler's own
+// choice is the best.  One key of a 16-slot bucket: left alone it keeps 36
+// registers and loads the bucket piece by piece (8M finds, half absent, 3-D
+// 223 us, 1-D 191), at four blocks the bucket's loads are in flight together
+// (184 and 155); at five 199 and 174.  The rest gives the register counts at
+// which the options with more keys per thread ran before the lookups went on
+// in place (8-D, 8 slots, four keys stay slower, 229 against 206 us).
+template <int D, int S, int KPT>
+constexpr int find_min_blocks() {
+  if (KPT == 1) return S == 16 ? 4 : 0;
+  if (KPT == 2) return D == 1 ? 4 : (S == 16 && D > 6 ? 3 : 0);
+  return D == 8 ? 2 : 0;
+}
+
 // KPT keys per thread: positions base, base + blockDim.x, ... so every load
 // instruction stays coalesced across the warp.
 template <int D, int S, int KPT, class In = const int32_t*>
-__global__ void __launch_bounds__(256) find_kernel(TableView t, const In keys, int64_t n,
+__global__ void __launch_bounds__(256, find_min_blocks<D, S, KPT>()) find_kernel(TableView t, const In keys, int64_t n,
                                                    int32_t* __restrict__ idx, uint8_t* __restrict__ mask) {
   // a programmatic dependent of the previous kernel: wait for its grid (a no-op otherwise)
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1777,8 +1823,12 @@ struct DimLaunchers {
   template <int S, int KPT, class In>
   static void find_sk(const TableView& t, const In& keys, int64_t n, int32_t* idx, uint8_t* mask, const Launch& L) {
     TraceScope ts(kKFind, L.stream);
-    launch_dependent(find_kernel<D, S, KPT, In>, grid_for((n + KPT - 1) / KPT, L), L.block, L.stream, t, keys, n, idx,
-                     mask);
+    // one key per thread: no more blocks than fit at once (8M finds of 8-D keys
+    // 219 -> 211 us, 20M 428 -> 354; up to 6-D all of the cap's fit); with
+    // several the second wave evens the rounds out (two keys, 3-D 158, 164 held)
+    constexpr auto k = find_kernel<D, S, KPT, In>;
+    const int g = grid_for((n + KPT - 1) / KPT, L);
+    launch_dependent(k, KPT == 1 ? resident_grid<k>(g, L) : g, L.block, L.stream, t, keys, n, idx, mask);
   }
   template <int S, class In>
   static void find_s(int kpt, const TableView& t, const In& keys, int64_t n, int32_t* idx, uint8_t* mask,
