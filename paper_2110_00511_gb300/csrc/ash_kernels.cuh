@@ -947,10 +947,16 @@ __global__ void __launch_bounds__(256) claim_bucket_kernel(TableView t, const In
 // stalling every warp for a few lanes (a second queue for those that then
 // need the full protocol cost registers and 3 % at 4M keys).  A CAS that
 // misses L2 waits on DRAM inside the atomic unit, so this path pays off while
-// the table stays in L2.  Six blocks per SM for 4-slot buckets (40 registers):
-// 4M claims 90 us, against 107 with four blocks and 105 with eight.
+// the table stays in L2.  Six blocks per SM for 4-slot buckets and up to four
+// dimensions (40 registers): 4M claims 90 us, against 107 with four blocks and
+// 105 with eight; points 117 (80 bytes spilled), against 121 with five and 126
+// with the compiler's choice.  Elsewhere the compiler's choice (0) is the best
+// one, and asking for any block at all (1) is not the same as leaving it: it
+// raises the registers by half.  2M claims with 1 | 0 | a bound: 3-D, 8 slots
+// 67 | 54 | 56 us (five blocks), 16 slots 88 | 63 | 65 (four), 5-D 61 | 53 |
+// 57 (five), 8-D 79 | 71 | 72 (four).
 template <int D, int S, int KPT, class In = const int32_t*>
-__global__ void __launch_bounds__(256, S == 4 && D <= 4 ? 6 : 1) claim_pref_kernel(TableView t, const In keys, int64_t n,
+__global__ void __launch_bounds__(256, S == 4 && D <= 4 ? 6 : 0) claim_pref_kernel(TableView t, const In keys, int64_t n,
                                                          int32_t* __restrict__ slot_out) {
   // a programmatic dependent of the previous kernel: wait for its grid (a no-op otherwise)
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1853,9 +1859,9 @@ struct DimLaunchers {
     find_in(S, kpt, t, p, n, idx, mask, L);
   }
   // pref: 1 = preferred slot first (claim_pref_kernel), 0 = bucket load first.
-  // The preferred-slot claim always takes one key per thread: with one
-  // queued key per lane in its dense rounds it needs 32 registers and runs
-  // at full occupancy, 4-8 % faster than two keys per thread on GB300.
+  // The preferred-slot claim always takes one key per thread, which with one
+  // queued key per lane in its dense rounds leaves more warps resident than
+  // two keys per thread (4-8 % faster on GB300).
   template <int S, int KPT, class In>
   static void claim_sk(int pref, const TableView& t, const In& keys, int64_t n, int32_t* slot_out,
                        const Launch& L) {

@@ -16,6 +16,10 @@ LIMITS = {
     "find_kernel<3, 4, 2>": 64, "find_kernel<3, 8, 2>": 64, "find_kernel<3, 16, 2>": 64,
     "find_kernel<3, 4, 4>": 80, "find_kernel<3, 8, 4>": 100, "find_kernel<3, 16, 4>": 80,
     "find_kernel<8, 4, 1>": 64, "find_kernel<8, 16, 2>": 96, "find_kernel<8, 16, 4>": 128,
+    # preferred-slot claims: six blocks for 4 slots and up to four dimensions, elsewhere as many as fit
+    "claim_pref_kernel<3, 4, 1>": 40, "claim_pref_kernel<4, 4, 1>": 40, "claim_pref_kernel<3, 8, 1>": 48,
+    "claim_pref_kernel<3, 16, 1>": 64, "claim_pref_kernel<5, 4, 1>": 40, "claim_pref_kernel<8, 4, 1>": 48,
+    "claim_pref_kernel<8, 8, 1>": 64,
 }
 
 
