@@ -902,15 +902,18 @@ __device__ __forceinline__ void claim_slow_round(const TableView& t, const In& k
 // warps have one, and running the protocol for it at once cost more than all
 // its other keys' CASes (GB300, 10^8 keys by ranges: activate and find 9.18 ->
 // 8.56 ms).  The better choice when the table does not stay in L2: the loads
-// bring the buckets in with deep miss queues and the CASes then hit L2.  Input
-// order takes as many blocks as are resident at once: 10^7 claims 345 -> 322
-// us without the thin second wave of eight blocks per SM; the calls of a
-// ranged batch keep the larger grid (10^8 keys, activate and find, with five
-// resident blocks of 48 registers: 7.55 -> 7.82 ms).  Slot order does
+// bring the buckets in with deep miss queues and the CASes then hit L2.  It
+// takes as many blocks as are resident at once: 10^7 keys in input order 307
+// us, 328 with eight blocks per SM (a thin second wave); the ranged calls on
+// 10^8 keys 2579 us, 2785 with eight.  Beyond L2, in input order, fewer still
+// (the host's cap, claim_blocks_per_sm).  8-slot buckets: compiled for four
+// blocks, the loads of both keys' buckets in flight, 8M keys 248 -> 230 us;
+// 4-slot ones with four or five blocks asked for 239 and 225 against 230, but
+// 20M inserts with values 728 and 776 against 761.  Slot order does
 // not keep the preferred-slot invariant (preferred-first placement measured
 // 5-10 % slower here), so the host clears the map's flag.
 template <int D, int S, int KPT, class In = const int32_t*>
-__global__ void __launch_bounds__(256) claim_bucket_kernel(TableView t, const In keys, int64_t n,
+__global__ void __launch_bounds__(256, S == 8 && KPT == 2 ? 4 : 0) claim_bucket_kernel(TableView t, const In keys, int64_t n,
                                                            int32_t* __restrict__ slot_out) {
   // a programmatic dependent of the previous kernel: wait for its grid (a no-op otherwise)
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1708,7 +1711,6 @@ struct Launch {
   int grid_cap;  // SMs x blocks_per_sm
   int block;
   int sms = 0;   // SM count (0: unknown)
-  bool one_wave = true;  // resident_grid holds a grid to the blocks that fit at once
 };
 
 // Launch with programmatic stream serialisation: the kernel's blocks may be
@@ -1761,7 +1763,7 @@ inline int resident_blocks(int block) {
 // wave runs at low occupancy.
 template <auto Kernel>
 inline int resident_grid(int want, const Launch& L) {
-  if (!L.one_wave || L.sms <= 0) return want;
+  if (L.sms <= 0) return want;
   const int cap = L.sms * resident_blocks<Kernel>(L.block);
   return want < cap ? want : cap;
 }

@@ -271,6 +271,19 @@ int partition_log(const ash_map* m, int64_t n) {
   return mode == 2 ? std::max(lg, 3) : lg;
 }
 
+// Blocks per SM, at most, of a bucket-first claim in input order.  Beyond L2
+// the blocks' buckets are in each other's way there: inserts with values of 20M
+// 3-D keys (table 2.4 times L2) 752 us with the five blocks that fit, 727 with
+// four, 743 with three; 40M 1811, 1735, 1703; 8-slot buckets 892, 855 (four),
+// 832 (three); 16-slot ones 1432 (three), 1333 (two), 1523 (one).  On smaller
+// tables every block that fits is wanted (10^7 keys, 1.2 times L2: 322 us with
+// five, 346 with four).  The line is the one above which calls without values
+// go by ranges.
+int claim_blocks_per_sm(const ash_map* m) {
+  if (2 * m->n_slots * 8 <= 3 * l2_bytes(m->device)) return m->tuning.blocks_per_sm;
+  return m->S == 4 ? 4 : (m->S == 8 ? 3 : 2);
+}
+
 // False when the scratch cannot be had or the device refuses a step of the
 // partition: the call then uses its keys in input order (what was enqueued
 // only touches the scratch, which is freed behind it).
@@ -889,13 +902,13 @@ ash_status insert_impl(ash_map* m, const int32_t* keys, const void* const* value
       ash::TableView tvp = tv;
       if (p != P - 1) tvp.snap = nullptr;  // the last commit publishes the control block
       const int32_t* sk = ckeys + a * m->key_dim;
-      Launch Lr = L;
-      Lr.one_wave = pref;  // the bucket-first claim takes the larger grid here (see claim_bucket_kernel)
-      m->K.claim(m->S, kpt, pref, tvp, sk, b - a, cidx + a, Lr);
+      m->K.claim(m->S, kpt, pref, tvp, sk, b - a, cidx + a, L);
       m->K.commit(ckpt, tvp, sk, b - a, cidx + a, cmask + a, inline_value ? &vr : nullptr, L);
     }
   } else {
-    m->K.claim(m->S, kpt, pref, tv, ckeys, n, cidx, L);
+    Launch Lc = L;
+    if (!pref) Lc.grid_cap = std::min(L.grid_cap, L.sms * claim_blocks_per_sm(m));
+    m->K.claim(m->S, kpt, pref, tv, ckeys, n, cidx, Lc);
     m->K.commit(ckpt, tv, ckeys, n, cidx, cmask, inline_value ? &vr : nullptr, L);
   }
   if (log_p > 0) partition_finish(m, pb, n, idx, mask, st);
