@@ -43,6 +43,7 @@
 #pragma once
 
 #include <atomic>
+#include <type_traits>
 
 #include "ash_device.cuh"
 #include "ash_trace.h"
@@ -1117,15 +1118,27 @@ __device__ __forceinline__ void copy_small_row(const ValueRow& v, int32_t i, int
 // KPT keys per thread per block iteration (blockDim.x * KPT keys).  Who won
 // each key: FLAGS, a position holding a slot index whose winner-flag bit
 // (t.lost) is clear, from two streamed reads; otherwise the slot word, read
-// at random, names the winning position.  The warps' counts of winners are
-// scanned by every warp for itself and ONE heap atomic serves the iteration
-// (Sec. 4.3: t is raised by the number of indices taken).  Winners then write
-// kB(i), the value row, the committed slot word and their outputs.  `turn`
-// alternates between 0 and 1 from tile to tile (TileShared).
+// at random, names the winning position.  The first warp scans the warps'
+// counts of winners and ONE heap atomic serves the iteration (Sec. 4.3: t is
+// raised by the number of indices taken).  Winners then write kB(i), the value
+// row, the committed slot word and their outputs.  `turn` alternates between 0
+// and 1 from tile to tile (TileShared).
+//
+// Bound by random sectors (the slot words); past L2 by DRAM, and then by how
+// many warps are resident and how early their loads go out.  So the prefix is
+// left in shared memory rather than in every warp's registers, the winners'
+// key rows are asked for right after the barrier, and two keys per thread are
+// held to eight blocks.  With every warp scanning for itself and the rows
+// loaded last, 8M keys of 5 dimensions took 156 us (now 149), of 8 163 (153),
+// of 3 131 (130), two per thread 137 (129) and, 2M in L2, 24 (20).
 template <int D, int KPT, bool VAL, class In, bool FLAGS = false>
 __device__ __forceinline__ void commit_tile(const TableView& t, const In& keys, int64_t n,
                                             int64_t base0, int32_t* __restrict__ idx, uint8_t* __restrict__ mask,
                                             const ValueRow& v, TileShared& sh, int turn) {
+  // points are quantised as they are loaded, and the batched kernel holds every
+  // dimension's code: both were slower with the rows' registers held longer
+  // (4M points 54 for 52 us)
+  constexpr bool kRowsEarly = FLAGS && std::is_pointer<In>::value;
   const int64_t base = base0 + threadIdx.x;
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -1169,9 +1182,10 @@ __device__ __forceinline__ void commit_tile(const TableView& t, const In& keys, 
     for (int q = 0; q < KPT; ++q) sh.cnt[turn][q * n_warps + warp] = __popc(won[q]);
   }
   __syncthreads();
-  const int c = lane < KPT * n_warps ? sh.cnt[turn][lane] : 0;
-  const int upto = warp_scan(c);
   if (threadIdx.x < 32) {
+    const int c = lane < KPT * n_warps ? sh.cnt[turn][lane] : 0;
+    const int upto = warp_scan(c);
+    sh.cnt[turn][lane] = upto - c;
     const int total = __shfl_sync(0xFFFFFFFFu, upto, 31);
     if (threadIdx.x == 0) {
       int got = 0, top = 0;
@@ -1197,13 +1211,15 @@ __device__ __forceinline__ void commit_tile(const TableView& t, const In& keys, 
 #pragma unroll
   for (int q = 0; q < KPT; ++q) {
     const int64_t pos = base + static_cast<int64_t>(q) * blockDim.x;
-    const int r = __shfl_sync(0xFFFFFFFFu, upto - c, q * n_warps + warp) + __popc(won[q] & ((1u << lane) - 1u));
+    const bool win = (won[q] >> lane) & 1u;
+    int32_t k[D];
+    if (kRowsEarly && win) load_input_key<D>(keys, pos, k);
+    const int r = sh.cnt[turn][q * n_warps + warp] + __popc(won[q] & ((1u << lane) - 1u));
     if (pos < n) {
-      if ((won[q] >> lane) & 1u) {
+      if (win) {
         if (r < got) {
           const int32_t i = (t.flags & kViewHeapIdentity) ? hbase + r : t.heap[hbase + r];
-          int32_t k[D];
-          load_input_key<D>(keys, pos, k);
+          if (!kRowsEarly) load_input_key<D>(keys, pos, k);
           store_kb<D>(t.kb, static_cast<uint32_t>(i), k);
           if constexpr (VAL) copy_small_row(v, i, pos);
           const uint32_t fp = FLAGS ? fingerprint(hash_key<D>(k)) : hi32(w[q]);
@@ -1224,7 +1240,7 @@ __device__ __forceinline__ void commit_tile(const TableView& t, const In& keys, 
 }
 
 template <int D, int KPT, bool VAL, class In = const int32_t*, bool FLAGS = false>
-__global__ void __launch_bounds__(256) commit_kernel(TableView t, const In keys, int64_t n,
+__global__ void __launch_bounds__(256, KPT == 2 ? 8 : 0) commit_kernel(TableView t, const In keys, int64_t n,
                                                      int32_t* __restrict__ idx, uint8_t* __restrict__ mask,
                                                      ValueRow v) {
   __shared__ TileShared sh;
