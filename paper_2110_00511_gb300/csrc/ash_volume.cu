@@ -439,13 +439,16 @@ __global__ void __launch_bounds__(kThreads) block_range_kernel(const int32_t* __
 // samples together) -> 73 (occupancy); 2, 3, 6 samples at once 75, 75, 83.
 //
 // x / b correctly rounded from y = 1 / b correctly rounded (Markstein, IBM J.
-// Res. Dev. 34, 1990): q = x y is within an ulp of the quotient, the remainder
-// x - b q is exact in one fused multiply-add, and q + remainder * y rounds to
-// the quotient, unless something over- or underflows.  Here it may: only
-// floor(q + 1/2) is used, which is 0 for every tiny quotient, and a quotient
-// past the range is refused whether it is huge, infinite or NaN.  y itself has
-// to be a normal number: for voxel sizes outside [2^-60, 2^60] the division is
-// made by __fdiv_rn (MUL false).
+// Res. Dev. 34, 1990): q = x y is within 1.5 ulp of the quotient, the remainder
+// x - b q takes 25 bits at most, so one fused multiply-add gives it to a unit
+// in its last place, and q + remainder * y before its rounding is off by less
+// than 2.5 ulp(q) / b (mantissas as integers).  Only quotients that close to a
+// midpoint of two floats could round the other way; of all pairs of mantissas
+// none does (the test enumerates them).  Over- and underflow change nothing
+// here: only floor(q + 1/2) is used, which is 0 for every tiny quotient, and a
+// quotient past the range is refused whether it is huge, infinite or NaN.  y
+// itself has to be a normal number: for voxel sizes outside [2^-60, 2^60] the
+// division is made by __fdiv_rn (MUL false).
 template <bool MUL>
 __device__ __forceinline__ float divide_by_voxel(float x, float voxel, float inv_voxel) {
   if constexpr (!MUL) return __fdiv_rn(x, voxel);
