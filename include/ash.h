@@ -78,13 +78,15 @@ typedef struct ash_tuning {
   int32_t max_probes;         /* bucket probes before a key fails; 0 = every bucket */
   int32_t auto_grow;          /* 1: insert/activate double the capacity until size+n <= c (Sec. 4.5) */
   float max_used_fraction;    /* rebuild the table when live+erased slots would pass this fraction
-                                 (0.65: erased slots stay as tombstones until a rebuild, and with
-                                 linear bucket probing a lookup that misses walks 1.5 buckets on
-                                 average at 0.6 of the slots used but 6 at 0.85) */
+                                 (0.65: with linear bucket probing a lookup that misses walks 1.5
+                                 buckets on average at 0.6 of the slots used but 6 at 0.85; an
+                                 erased slot counts while it is a tombstone, that is until a claim
+                                 takes it or a rebuild: where no probe chain passes, erase leaves
+                                 none) */
   int32_t inline_value_bytes; /* a map with ONE value buffer whose rows are 4, 8 or 16 bytes (at most
                                  this limit, both bases aligned to the row size) has them copied by
-                                 the committing thread; other layouts use a warp-per-row scatter
-                                 kernel after the commit */
+                                 the committing thread; other layouts are scattered after the
+                                 commit, by one kernel per value buffer */
   int32_t keys_per_thread;    /* 1, 2 or 4 keys handled together by each thread of the find,
                                  bucket-first claim and commit kernels (more independent memory
                                  requests in flight); the preferred-slot claim takes one key per

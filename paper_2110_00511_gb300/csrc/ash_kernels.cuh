@@ -2,8 +2,8 @@
 //
 // find            KPT query keys per thread: hash, load the home buckets of all
 //                 KPT keys back to back, verify the fingerprint match of each
-//                 against kB (Eq. (4)); keys that overflow their home bucket
-//                 take the scalar probe loop.
+//                 against kB (Eq. (4)); keys that their home bucket does not
+//                 settle go on from the next one (find_keys).
 // insert/activate two kernels (Sec. 4.3.1 lazy insertion, redesigned):
 //   claim         a key already committed is rejected.  Otherwise the thread
 //                 claims an EMPTY slot with a CAS writing {fingerprint,

@@ -853,7 +853,7 @@ ash_status insert_impl(ash_map* m, const int32_t* keys, const void* const* value
   const int pref = claim_prefers_slot(m);
   const int ckpt = m->tuning.commit_keys_per_thread ? m->tuning.commit_keys_per_thread : kpt;
   // one value buffer with small rows: copied by the committing thread;
-  // anything else: warp-per-row scatter after the commit
+  // anything else: scattered after the commit, one kernel per value buffer
   bool inline_value = false;
   ash::ValueRow vr{};
   ash::ValueCopy vc{};
