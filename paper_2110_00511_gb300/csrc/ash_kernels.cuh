@@ -906,8 +906,8 @@ __device__ __forceinline__ void claim_slow_round(const TableView& t, const In& k
 // bring the buckets in with deep miss queues and the CASes then hit L2.  It
 // takes as many blocks as are resident at once: 10^7 keys in input order 307
 // us, 328 with eight blocks per SM (a thin second wave); the ranged calls on
-// 10^8 keys 2579 us, 2785 with eight.  Beyond L2, in input order, fewer still
-// (the host's cap, claim_blocks_per_sm).  8-slot buckets: compiled for four
+// 10^8 keys 2579 us, 2785 with eight.  Beyond L2, in input order, the host
+// picks the grid (claim_launch).  8-slot buckets: compiled for four
 // blocks, the loads of both keys' buckets in flight, 8M keys 248 -> 230 us;
 // 4-slot ones with four or five blocks asked for 239 and 225 against 230, but
 // 20M inserts with values 728 and 776 against 761.  Slot order does
@@ -1727,6 +1727,7 @@ struct Launch {
   int grid_cap;  // SMs x blocks_per_sm
   int block;
   int sms = 0;   // SM count (0: unknown)
+  bool one_wave = true;  // resident_grid holds a grid to the blocks that fit at once
 };
 
 // Launch with programmatic stream serialisation: the kernel's blocks may be
@@ -1779,7 +1780,7 @@ inline int resident_blocks(int block) {
 // wave runs at low occupancy.
 template <auto Kernel>
 inline int resident_grid(int want, const Launch& L) {
-  if (L.sms <= 0) return want;
+  if (!L.one_wave || L.sms <= 0) return want;
   const int cap = L.sms * resident_blocks<Kernel>(L.block);
   return want < cap ? want : cap;
 }

@@ -271,17 +271,23 @@ int partition_log(const ash_map* m, int64_t n) {
   return mode == 2 ? std::max(lg, 3) : lg;
 }
 
-// Blocks per SM, at most, of a bucket-first claim in input order.  Beyond L2
-// the blocks' buckets are in each other's way there: inserts with values of 20M
-// 3-D keys (table 2.4 times L2) 752 us with the five blocks that fit, 727 with
-// four, 743 with three; 40M 1811, 1735, 1703; 8-slot buckets 892, 855 (four),
-// 832 (three); 16-slot ones 1432 (three), 1333 (two), 1523 (one).  On smaller
-// tables every block that fits is wanted (10^7 keys, 1.2 times L2: 322 us with
-// five, 346 with four).  The line is the one above which calls without values
-// go by ranges.
-int claim_blocks_per_sm(const ash_map* m) {
-  if (2 * m->n_slots * 8 <= 3 * l2_bytes(m->device)) return m->tuning.blocks_per_sm;
-  return m->S == 4 ? 4 : (m->S == 8 ? 3 : 2);
+// Launch of a bucket-first claim in input order.  Up to 1.5 times L2 every
+// block that fits at once is wanted (10^7 keys, 1.2 times L2: 322 us with five
+// per SM, 346 with four), and no more.  Beyond it (the line above which calls
+// without values go by ranges) the blocks' buckets are in each other's way:
+// inserts with values of 20M 3-D keys (table 2.4 times L2) 752 us with the five
+// blocks that fit, 727 with four, 743 with three; of 40M 1811, 1735, 1703;
+// 8-slot buckets 892, 855 (four), 832 (three).  16-slot buckets are the faster
+// in several waves, which go over the input one after the other: 20M 1433 us
+// with the three blocks that fit, 1336 with two, 1267 in waves; 40M 4120, 4010,
+// 3585.
+ash::Launch claim_launch(const ash_map* m, cudaStream_t st) {
+  ash::Launch L = launch_of(m, st);
+  if (2 * m->n_slots * 8 > 3 * l2_bytes(m->device)) {
+    if (m->S == 16) L.one_wave = false;
+    else L.grid_cap = std::min(L.grid_cap, L.sms * (m->S == 4 ? 4 : 3));
+  }
+  return L;
 }
 
 // False when the scratch cannot be had or the device refuses a step of the
@@ -906,9 +912,7 @@ ash_status insert_impl(ash_map* m, const int32_t* keys, const void* const* value
       m->K.commit(ckpt, tvp, sk, b - a, cidx + a, cmask + a, inline_value ? &vr : nullptr, L);
     }
   } else {
-    Launch Lc = L;
-    if (!pref) Lc.grid_cap = std::min(L.grid_cap, L.sms * claim_blocks_per_sm(m));
-    m->K.claim(m->S, kpt, pref, tv, ckeys, n, cidx, Lc);
+    m->K.claim(m->S, kpt, pref, tv, ckeys, n, cidx, pref ? L : claim_launch(m, st));
     m->K.commit(ckpt, tv, ckeys, n, cidx, cmask, inline_value ? &vr : nullptr, L);
   }
   if (log_p > 0) partition_finish(m, pb, n, idx, mask, st);

@@ -37,6 +37,8 @@ int main(int argc, char**) {
   L.sms = 2;
   const int held = 2 * ash::resident_blocks<probe_kernel<40>>(256);
   ok = ok && ash::resident_grid<probe_kernel<40>>(1000, L) == held && ash::resident_grid<probe_kernel<40>>(1, L) == 1;
+  L.one_wave = false;
+  ok = ok && ash::resident_grid<probe_kernel<40>>(1000, L) == 1000;
   return ok ? 0 : 1;
 }
 """
