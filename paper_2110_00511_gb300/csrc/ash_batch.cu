@@ -468,19 +468,23 @@ ash_status ash_batch_run(ash_batch* b, const ash_batch_op* ops, int n_ops, ash_s
     snapped.push_back(m);
     tb->snaps[tb->n_snaps++] = {m->ctrl, m->snap_dev, m->snap_seq};
   }
+  // What the batch does to the maps' invariants holds from its first launch on,
+  // also when a later one is refused.
+  for (int i = 0; i < n_ops; ++i)
+    if (ops[i].op == ASH_OP_INSERT || ops[i].op == ASH_OP_ACTIVATE) ops[i].map->pref_placed = false;  // keys placed in slot order
+    else if (ops[i].op == ASH_OP_ERASE) ops[i].map->heap_identity = false;
+  ash_status s = ASH_OK;
   if (k > 0 || tb->n_snaps > 0) {  // snapshots that were numbered have to be published, work or not
     TraceScope ts(kKBatch, st, batch_launches(*tb));
     if (wide) launch_batch<true>(b, sl, st);
     else launch_batch<false>(b, sl, st);
-    ash_status s = check_launch("batch_run");
-    if (s != ASH_OK) return s;
+    s = check_launch("batch_run");
   }
-  for (ash_map* m : snapped) snapshot_issued(m);
-  for (int i = 0; i < n_ops; ++i)
-    if (ops[i].op == ASH_OP_INSERT || ops[i].op == ASH_OP_ACTIVATE) ops[i].map->pref_placed = false;  // keys placed in slot order
-    else if (ops[i].op == ASH_OP_ERASE) ops[i].map->heap_identity = false;
+  // the upload reads the slot's table until then, whatever followed it
   if (cudaEventRecord(sl.done, st) != cudaSuccess) return cuda_fail(cudaGetLastError(), "cudaEventRecord");
   sl.used = true;
+  if (s != ASH_OK) return s;
+  for (ash_map* m : snapped) snapshot_issued(m);
   return ASH_OK;
 }
 
