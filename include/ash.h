@@ -74,7 +74,8 @@ typedef struct ash_tuning {
   int32_t slots_per_bucket;   /* 4, 8 or 16 eight-byte slots: 32, 64 or 128 B buckets */
   float slots_per_capacity;   /* table slots per unit of capacity (2.0: load <= 0.5) */
   int32_t block_threads;      /* threads per block of the map kernels (multiple of 32, <= 256) */
-  int32_t blocks_per_sm;      /* grid = SM count x blocks_per_sm (grid-stride loops) */
+  int32_t blocks_per_sm;      /* grid = SM count x blocks_per_sm (grid-stride loops) at most; some
+                                 kernels take only the blocks that fit at once, or fewer */
   int32_t max_probes;         /* bucket probes before a key fails; 0 = every bucket */
   int32_t auto_grow;          /* 1: insert/activate double the capacity until size+n <= c (Sec. 4.5) */
   float max_used_fraction;    /* rebuild the table when live+erased slots would pass this fraction
