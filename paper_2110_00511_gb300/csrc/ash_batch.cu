@@ -260,12 +260,13 @@ struct ash_batch {
 
 namespace {
 
-// The batch's kernels on st, empty phases left out.
+// How many kernels launch_batch launches.
 int batch_launches(const BatchTable& tb) {
   return 1 + (tb.ph[kPhaseInsert].tiles > 0 ? 2 : 0) + (tb.ph[kPhaseFind].tiles > 0 ? 1 : 0) +
          (tb.ph[kPhaseErase].tiles > 0 ? 2 : 0) + (tb.n_snaps > 0 ? 1 : 0);
 }
 
+// The batch's kernels on st, empty phases left out.
 template <bool WIDE>
 void launch_batch(const ash_batch* b, const ash_batch::Slot& s, cudaStream_t st) {
   const BatchTable* tb = s.h;

@@ -257,10 +257,11 @@ int claim_prefers_slot(const ash_map* m) {
 //   11.8          4960 / 7898    2302 / 3969    1775 / 2107 (at 7.1)
 // (measured with eight claim blocks per SM; on those that fit at once the
 // ranged activates are 35 us faster at 2.36 and 200 at 11.8; inserts into maps
-// with value buffers go in input order, so kB is not in range order there).  Ranges of L2/4 or L2 took 8.3 and 8.7 ms where L2/2
-// took 7.5 (both calls at 11.8).  The kernels bring a range's buckets into L2
-// themselves: a prefetch of each range before them cost 0.1 ms, and one that
-// ran beside the kernel before it 0.3 ms.
+// with value buffers go in input order, so kB is not in range order there).
+// Ranges of L2/4 or L2 took 8.3 and 8.7 ms where L2/2 took 7.5 (both calls at
+// 11.8).  The kernels bring a range's buckets into L2 themselves: a prefetch of
+// each range before them cost 0.1 ms, and one that ran beside the kernel before
+// it 0.3 ms.
 int partition_log(const ash_map* m, int64_t n) {
   const int mode = m->tuning.partition_keys;
   if (mode == 1 || n <= 0) return 0;
